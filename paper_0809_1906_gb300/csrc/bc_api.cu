@@ -171,6 +171,20 @@ cudaError_t fetch(std::vector<T> &dst, const T *src, size_t count) {
     return cudaMemcpy(dst.data(), src, count * sizeof(T), cudaMemcpyDefault);
 }
 
+// Whether kernels of the current device may write T values straight to p: its
+// own device memory, aligned for T (a copy would take any alignment).
+template <class T>
+bool device_writable(const T *p) {
+    if (!p || reinterpret_cast<uintptr_t>(p) % alignof(T) != 0) return false;
+    cudaPointerAttributes a{};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();  // not a CUDA pointer
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 }  // namespace
 
 // Work items of one level sweep: one per vertex, except vertices with more
@@ -2085,24 +2099,35 @@ int bc_forward_rows(bc_graph *g, const int32_t *sources, int32_t k, uint64_t *si
     if (r) return r;
     if (nsrc == 0) return BC_OK;
     const size_t cells = (size_t)nsrc * g->n;
+    // outputs in this device's memory are written by the kernels themselves;
+    // others through a device copy of the rows
     DevBuf<uint64_t> ds;
     DevBuf<int32_t> dd;
-    if (sigma) CK(ds.ensure(cells));
-    if (dist) CK(dd.ensure(cells));
+    uint64_t *sig_rows = device_writable(sigma) ? sigma : nullptr;
+    int32_t *dist_rows = device_writable(dist) ? dist : nullptr;
+    const bool copy_sig = sigma && !sig_rows, copy_dist = dist && !dist_rows;
+    if (copy_sig) {
+        CK(ds.ensure(cells));
+        sig_rows = ds.p;
+    }
+    if (copy_dist) {
+        CK(dd.ensure(cells));
+        dist_rows = dd.p;
+    }
     CK(cudaMemsetAsync(&g->ctl->status, 0, sizeof(uint32_t), st));
     g->timing = false;
     if (g->weighted && opt && (opt->flags & BC_DENSE)) {
         if (!sigma || !dist) return fail(BC_ERR_ARG, "BC_DENSE rows of a weighted graph need both outputs");
-        r = run_minplus(g, nsrc, st, false, ds.p, dd.p);
+        r = run_minplus(g, nsrc, st, false, sig_rows, dist_rows);
     } else if (g->weighted)
-        r = run_weighted(g, nsrc, opt, st, false, false, sigma ? ds.p : nullptr, dist ? dd.p : nullptr);
+        r = run_weighted(g, nsrc, opt, st, false, false, sig_rows, dist_rows);
     else
-        r = run_batches(g, nsrc, W, opt, st, false, false, sigma ? ds.p : nullptr, dist ? dd.p : nullptr);
+        r = run_batches(g, nsrc, W, opt, st, false, false, sig_rows, dist_rows);
     uint32_t status = 0;
     if (!r) {
         cudaError_t e = cudaSuccess;
-        if (sigma) e = cudaMemcpyAsync(sigma, ds.p, cells * 8, cudaMemcpyDefault, st);
-        if (e == cudaSuccess && dist) e = cudaMemcpyAsync(dist, dd.p, cells * 4, cudaMemcpyDefault, st);
+        if (copy_sig) e = cudaMemcpyAsync(sigma, ds.p, cells * 8, cudaMemcpyDefault, st);
+        if (e == cudaSuccess && copy_dist) e = cudaMemcpyAsync(dist, dd.p, cells * 4, cudaMemcpyDefault, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&status, &g->ctl->status, 4, cudaMemcpyDefault, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) r = fail(BC_ERR_CUDA, std::string("forward rows: ") + cudaGetErrorString(e));

@@ -584,24 +584,71 @@ __global__ void __launch_bounds__(kBlock, 2) k_hash(const MsParams p, const int 
     }
 }
 
-// Rows of the forward pass for bc_forward_rows: out[b][v] for this batch.
+// Rows of the forward pass for bc_forward_rows: out[b][v] for this batch. The
+// batch state is laid out vertex by vertex (sources contiguous), the rows
+// source by source (vertices contiguous), so a warp takes tiles of 32
+// vertices x 32 sources: lane k holds word j of vertex v0+k for every level
+// and keeps the level number of each of its 32 pairs as bit planes (plane p:
+// OR of the words of the levels with bit p set), and sigma goes through
+// shared memory. Every global access is then contiguous over the warp. Bound:
+// DRAM, 20 bytes per pair (8 of sigma read, 12 of rows written). With one
+// thread per pair, whose stores stepped a whole row apart, and a copy of the
+// rows to the caller's device buffers, the call took 1119 us for 512 sources
+// of a 23,756-vertex R-MAT graph; with these tiles written in place, 594 us.
+constexpr int kRowBlock = 128;
+constexpr int kRowWarps = kRowBlock / 32;
+constexpr int kRowPlanes = 20;  // levels below 2^20 (the frontier words of 2^20 levels would take over 4 TB)
 template <int W>
-__global__ void __launch_bounds__(kBlock) k_rows(const MsParams p, const int L, uint64_t *sig_out,
-                                                 int32_t *dist_out) {
+__global__ void __launch_bounds__(kRowBlock) k_rows(const MsParams p, const int L, uint64_t *sig_out,
+                                                    int32_t *dist_out) {
     pdl::enter();
     constexpr int B = 32 * W;
+    __shared__ uint64_t s_tile[kRowWarps][32][33];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    uint64_t(*tile)[33] = s_tile[wib];
     const size_t nW = (size_t)p.n * W;
-    const size_t total = (size_t)p.n * B;
-    for (size_t i = (size_t)blockIdx.x * kBlock + threadIdx.x; i < total; i += (size_t)gridDim.x * kBlock) {
-        const int v = (int)(i / B);
-        const int b = (int)(i % B);
-        if (b >= p.nb) continue;
-        int lev = -1;
-        for (int l = 0; l <= L; ++l)
-            if ((p.F[(size_t)l * nW + (size_t)v * W + (b >> 5)] >> (b & 31)) & 1u) lev = l;
-        const size_t o = (size_t)b * p.n + v;
-        if (dist_out) dist_out[o] = lev;
-        if (sig_out) sig_out[o] = lev >= 0 ? p.sigma[(size_t)v * B + b] : 0ull;
+    const int ntiles = (p.n + 31) / 32;
+    int np = 0;  // planes in use
+    while (np < kRowPlanes && (L >> np) != 0) ++np;
+    const int units = ntiles * W;
+    for (int u = blockIdx.x * kRowWarps + wib; u < units; u += gridDim.x * kRowWarps) {
+        const int j = u % W, v0 = 32 * (u / W), vk = v0 + lane;
+        const int nb = p.nb - 32 * j;  // sources of this word
+        if (nb <= 0) continue;
+        const bool in = vk < p.n;
+        if (sig_out) {
+            const int nk = p.n - v0 < 32 ? p.n - v0 : 32;
+            const uint64_t *sg = p.sigma + (size_t)v0 * B + 32 * j + lane;
+#pragma unroll 8
+            for (int k = 0; k < 32; ++k) tile[k][lane] = k < nk ? __ldg(sg + (size_t)k * B) : 0ull;
+            __syncwarp();
+        }
+        uint32_t reached = 0u, plane[kRowPlanes];
+#pragma unroll
+        for (int q = 0; q < kRowPlanes; ++q) plane[q] = 0u;
+        const uint32_t *Fv = p.F + (size_t)(in ? vk : 0) * W + j;
+#pragma unroll 4
+        for (int l = 0; l <= L; ++l) {
+            const uint32_t w = in ? __ldg(Fv + (size_t)l * nW) : 0u;
+            reached |= w;
+#pragma unroll
+            for (int q = 0; q < kRowPlanes; ++q)
+                if (q < np && ((l >> q) & 1)) plane[q] |= w;
+        }
+        const int ns = nb < 32 ? nb : 32;
+        for (int s = 0; s < ns; ++s) {
+            const bool r = (reached >> s) & 1u;
+            const size_t o = (size_t)(32 * j + s) * p.n + vk;
+            if (in && dist_out) {
+                int lev = 0;
+#pragma unroll
+                for (int q = 0; q < kRowPlanes; ++q)
+                    if (q < np) lev |= (int)((plane[q] >> s) & 1u) << q;
+                dist_out[o] = r ? lev : -1;
+            }
+            if (in && sig_out) sig_out[o] = r ? tile[lane][s] : 0ull;
+        }
+        __syncwarp();  // the next tile overwrites this one
     }
 }
 
@@ -751,8 +798,11 @@ void ms_launch_hash(int W, const MsParams &p, int nlevels, cudaStream_t st) {
 
 void ms_launch_rows(int W, const MsParams &p, int nlevels, uint64_t *sig_out, int32_t *dist_out,
                     cudaStream_t st) {
-    const int g = 4 * sm_count();
-    BCGB_DISPATCH_W(W, pdl::launch(k_rows<kW>, g, kBlock, 0, st, p, nlevels, sig_out, dist_out));
+    const int units = ((p.n + 31) / 32) * W;  // (tile, word) pairs
+    const int need = (units + kRowWarps - 1) / kRowWarps;
+    const int cap = 6 * sm_count();  // the tiles' shared memory: six blocks per SM
+    const int g = need < 1 ? 1 : (need < cap ? need : cap);
+    BCGB_DISPATCH_W(W, pdl::launch(k_rows<kW>, g, kRowBlock, 0, st, p, nlevels, sig_out, dist_out));
 }
 
 void ms_launch_merge(const double *src, double *dst, int32_t n, const DevCtl *from, DevCtl *to, cudaStream_t st) {
