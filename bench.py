@@ -541,8 +541,9 @@ def cfg_wdense(c):
         kinds = {nat.KERNEL_NAMES[k]: h.kernel_time(k) for k in nat.KERNEL_NAMES}
         ms_s = c.timed(lambda: (h.run(stream=c.stream), h.result()), 2, 1)
     steps, mp_ms = kinds["dense"]
-    # one product step: 512 sources x n x n (add + min) pairs; lanes x clock = 1 issue per lane
-    elem = steps * 512.0 * g.n * g.n
+    # one launched step: every (arc, source) pair once (add and min, or compare and add);
+    # lanes x clock = 1 issue per lane
+    elem = steps * float(g.n) * 2.0 * g.m
     lane_peak = 152 * 128 * 2.07e9
     ach = elem / (mp_ms / 1e3)
     return {"metric": METRIC, "unit": UNIT, "value": g.n * g.m / (ms_d / 1e3), "ms_per_step": ms_d,
@@ -550,8 +551,8 @@ def cfg_wdense(c):
                                    "BC_DENSE: distance products with counts + pair formula",
                        "kernels_ms": {k: {"launches": v[0], "total_ms": v[1]} for k, v in kinds.items()},
                        "product_steps": steps},
-            "roofline": {"bound": "alu", "kernel": "k_mp_step", "achieved": ach / 1e12, "peak": lane_peak / 1e12,
-                         "unit": "T (min,+) elements/s", "frac": ach / lane_peak,
+            "roofline": {"bound": "alu", "kernel": "k_mp_dist, k_mp_count", "achieved": ach / 1e12,
+                         "peak": lane_peak / 1e12, "unit": "T (arc, source) elements/s", "frac": ach / lane_peak,
                          "peak_source": "152 SMs x 128 int32 lanes x 2.07 GHz, one element per lane-instruction",
                          "traffic": None},
             "vs_bucket_kernel_same_graph": {"ms": ms_s, "value": g.n * g.m / (ms_s / 1e3)},

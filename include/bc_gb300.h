@@ -93,9 +93,9 @@ extern "C" {
 #define BC_DENSE 0x20u       /* the algebraic forms of Section 3. Unweighted graphs: levels >= 1 as
                                 tensor-core products with the 0/1 adjacency matrix, forward
                                 (ComputePathCount) and backward (ComputeDependency), Section 3.1;
-                                n <= 65536, batch 128. Weighted graphs: distance products with path
-                                counts on the dense weight matrix until a step changes nothing
-                                (Section 3.2), then BC by Algorithm 2's pair formula; every vertex a
+                                n <= 65536, batch 128. Weighted graphs: distance products over the
+                                weight matrix's arcs until a step changes nothing, then the path
+                                counts the same way (Section 3.2), BC by Algorithm 2's pair formula; every vertex a
                                 source, n <= 16384 (bc_forward_rows: n <= 32768), n * max weight < 2^30 - 1;
                                 directed or not (the unweighted tensor-core form is undirected only). */
 #define BC_SPARSE_BACKWARD 0x40u /* with BC_DENSE: run the backward pass on the sparse kernel instead */

@@ -362,8 +362,9 @@ struct bc_graph {
     DevBuf<double> gbcpart;
     DevBuf<int32_t> gmeta;  // [3][gNB]: active list, valid sources, depth
 
-    // weighted algebraic forward (BC_DENSE on a weighted graph): dense weights
-    DevBuf<int32_t> mpW;
+    // weighted algebraic forward (BC_DENSE on a weighted graph): in-arcs by weight class
+    DevBuf<int32_t> mpcol, mpw;
+    bool mp_ready = false;
 
     // weighted path: per-wave state
     int32_t maxw = 1;
@@ -407,7 +408,8 @@ void free_graph(bc_graph *g) {
     g->part.release();
     g->cval.release();
     for (auto *b : {&g->F, &g->ufr, &g->V, &g->pmask, &g->cnt}) b->release();
-    g->mpW.release();
+    g->mpcol.release();
+    g->mpw.release();
     g->gsigma.release();
     for (auto *b : {&g->gF, &g->gV, &g->gufr}) b->release();
     g->gbcpart.release();
@@ -1785,11 +1787,14 @@ int run_pairs(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStrea
 }
 
 // Weighted algebraic forward (Section 3.2; BC_DENSE on a weighted graph):
-// per batch of sources, distance products with path counts on the dense
-// weight matrix until a step changes nothing (minplus.cu). Rows of the
-// staged sources [b0, b0 + nsrc) go to rows_sig / rows_dist in that order.
+// distance products until a step changes nothing, then the counts over the
+// arcs on shortest paths (minplus.cu). Rows of the staged sources
+// [b0, b0 + nsrc) go to rows_sig / rows_dist in that order. All sources run as
+// one batch while their state (24 bytes per pair) stays within kMpBudget: one
+// batch of 2001 sources fills the GPU where four of 512 left it two thirds
+// empty in the last wave of every step.
 constexpr int32_t kMpMaxN = 32768;
-constexpr int kMpBatch = 512;
+constexpr size_t kMpBudget = 4ull << 30;
 
 int run_minplus(bc_graph *g, int32_t nsrc, cudaStream_t st, bool hash, uint64_t *rows_sig, int32_t *rows_dist) {
     const int32_t n = g->n;
@@ -1798,42 +1803,72 @@ int run_minplus(bc_graph *g, int32_t nsrc, cudaStream_t st, bool hash, uint64_t 
         return fail(BC_ERR_UNSUPPORTED, "BC_DENSE on a weighted graph needs n * max weight < 2^30 - 1");
     if (!rows_sig || !rows_dist) return fail(BC_ERR_ARG, "weighted dense forward writes full rows");
     const int sms = sm_count_host();
-    if (!g->mpW.p) {
-        CK(g->mpW.ensure((size_t)n * n));
-        if (bcgb::mp_build_weights(g->row_ptr.p, g->col.p, g->w.p, n, g->mpW.p, sms, st))
-            return fail(BC_ERR_CUDA, "weight matrix build");
+    const bcgb::MpArcs in = g->directed ? bcgb::MpArcs{g->row_ptr_in.p, g->col_in.p, g->w_in.p, g->maxw}
+                                        : bcgb::MpArcs{g->row_ptr.p, g->col.p, g->w.p, g->maxw};
+    if (!g->mp_ready) {  // the arcs by weight, once per handle
+        CK(g->mpcol.ensure((size_t)std::max<int64_t>(g->narcs, 1)));
+        CK(g->mpw.ensure((size_t)std::max<int64_t>(g->narcs, 1)));
+        if (bcgb::mp_order_arcs(in.row_ptr, in.col, in.w, n, in.maxw, g->mpcol.p, g->mpw.p, sms, st))
+            return fail(BC_ERR_CUDA, "arc order");
+        CK(cudaStreamSynchronize(st));  // a later call may come on another stream
+        g->mp_ready = true;
     }
-    const int B = std::min<int32_t>(kMpBatch, std::max<int32_t>(nsrc, 1));
+    const bcgb::MpArcs arcs{in.row_ptr, g->mpcol.p, g->mpw.p, in.maxw};
+    auto padded = [](size_t k) { return (k + bcgb::kMpSrc - 1) / bcgb::kMpSrc * bcgb::kMpSrc; };
+    const size_t most = std::min<size_t>(  // at most 2^20: whole 128-source columns of the step's grid
+        1u << 20, std::max<size_t>(512, kMpBudget / ((size_t)24 * n) / bcgb::kMpSrc * bcgb::kMpSrc));
+    const int S = (int)std::min(padded((size_t)std::max<int32_t>(nsrc, 1)), most);
     ScopedBuf<int32_t> xd;
     ScopedBuf<uint64_t> xc;
-    ScopedBuf<uint32_t> flag;
-    CK(xd.ensure(2 * (size_t)B * n));
-    CK(xc.ensure(2 * (size_t)B * n));
-    CK(flag.ensure(1));
-    for (int32_t b0 = 0; b0 < nsrc; b0 += B) {
-        const int nb = std::min<int32_t>(B, nsrc - b0);
-        const size_t half = (size_t)B * n;
-        int cur = 0;
-        if (bcgb::mp_init(xd.p, xc.p, g->sources.p + b0, nb, n, sms, st)) return fail(BC_ERR_CUDA, "min-plus init");
-        for (int step = 0;; ++step) {
-            if (step > n) return fail(BC_ERR_BOUNDS, "distance products did not settle within n steps");
-            CK(cudaMemsetAsync(flag.p, 0, sizeof(uint32_t), st));
-            {
+    ScopedBuf<uint8_t> marks;   // change marks: [3][n][S / kMpSrc], the phases' start and two steps'
+    ScopedBuf<uint32_t> flags;  // [1 + kMpAhead][S / kMpSrc]: the newest step read, then those in flight
+    const size_t nblk = (size_t)S / bcgb::kMpSrc;
+    CK(xd.ensure(2 * (size_t)S * n));
+    CK(xc.ensure(2 * (size_t)S * n));
+    CK(marks.ensure(3 * nblk * n));
+    CK(flags.ensure((1 + bcgb::kMpAhead) * nblk));
+    const size_t half = (size_t)S * n;
+    std::vector<uint32_t> last(nblk);
+    // steps of one phase until one changes nothing; kMpAhead is even, so the
+    // state is back in the first buffer whenever the flags are read
+    static_assert(bcgb::kMpAhead % 2 == 0, "the phase ends in the buffer it started from");
+    auto settle = [&](auto &&step) -> int {
+        uint32_t *in_flight = flags.p + nblk, *newest = flags.p + bcgb::kMpAhead * nblk;
+        uint8_t *m1 = marks.p + nblk * n, *m2 = m1 + nblk * n;
+        for (int done = 0;; done += bcgb::kMpAhead) {
+            if (done > n) return fail(BC_ERR_BOUNDS, "distance products did not settle within n steps");
+            if (done)
+                CK(cudaMemcpyAsync(flags.p, newest, nblk * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st));
+            else
+                CK(cudaMemsetAsync(flags.p, 0xff, nblk * sizeof(uint32_t), st));
+            CK(cudaMemsetAsync(in_flight, 0, bcgb::kMpAhead * nblk * sizeof(uint32_t), st));
+            for (int i = 0; i < bcgb::kMpAhead; ++i) {
                 Timer t(g, st, BC_KERNEL_DENSE);
-                if (bcgb::mp_step(xd.p + cur * half, xc.p + cur * half, xd.p + (1 - cur) * half, xc.p + (1 - cur) * half,
-                                  g->mpW.p, g->sources.p + b0, nb, n, flag.p, &g->ctl->status, st))
+                const uint8_t *cx = done + i == 0 ? marks.p : (i & 1 ? m1 : m2);
+                if (step(i & 1, cx, i & 1 ? m2 : m1, flags.p + i * nblk, flags.p + (i + 1) * nblk))
                     return fail(BC_ERR_CUDA, "min-plus step launch");
             }
-            uint32_t f = 0;
-            CK(cudaMemcpyAsync(&f, flag.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+            CK(cudaMemcpyAsync(last.data(), newest, nblk * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
             CK(cudaStreamSynchronize(st));
-            cur ^= 1;
-            if (!(f & 1u)) break;
+            if (std::none_of(last.begin(), last.end(), [](uint32_t f) { return f != 0u; })) return BC_OK;
         }
+    };
+    for (int32_t b0 = 0; b0 < nsrc; b0 += S) {
+        const int nb = std::min<int32_t>(S, nsrc - b0);
+        if (bcgb::mp_init(xd.p, xc.p, marks.p, g->sources.p + b0, nb, n, S, sms, st))
+            return fail(BC_ERR_CUDA, "min-plus init");
+        int r = settle([&](int from, const uint8_t *cx, uint8_t *cy, const uint32_t *prev, uint32_t *flag) {
+            return bcgb::mp_dist_step(xd.p + from * half, xd.p + (1 - from) * half, arcs, n, S, cx, cy, prev, flag, st);
+        });
+        if (!r)
+            r = settle([&](int from, const uint8_t *cx, uint8_t *cy, const uint32_t *prev, uint32_t *flag) {
+                return bcgb::mp_count_step(xd.p, xc.p + from * half, xc.p + (1 - from) * half, arcs, n, S, cx, cy, prev,
+                                           flag, &g->ctl->status, st);
+            });
+        if (r) return r;
         int32_t *dr = rows_dist + (size_t)b0 * n;
         uint64_t *sr = rows_sig + (size_t)b0 * n;
-        if (bcgb::mp_rows(xd.p + cur * half, xc.p + cur * half, nb, n, dr, sr, sms, st))
-            return fail(BC_ERR_CUDA, "min-plus rows");
+        if (bcgb::mp_rows(xd.p, xc.p, nb, n, S, dr, sr, sms, st)) return fail(BC_ERR_CUDA, "min-plus rows");
         if (hash && bcgb::mp_row_hashes(dr, sr, nb, n, g->h_sigma.p + b0, g->h_dist.p + b0, g->dist_sum.p + b0,
                                         g->reach.p + b0, sms, st))
             return fail(BC_ERR_CUDA, "row summaries");
