@@ -375,6 +375,12 @@ struct bc_graph {
     std::vector<int32_t> h_sources;  // host copy of the staged source list
     DevBuf<uint64_t> wsigma;
     DevBuf<float> wcval, wrows;
+    struct WPack {  // the packed kernel's arcs and row records
+        DevBuf<uint32_t> arc, arc_in, rec, rec_in;
+        bool ready = false;
+    };
+    WPack wpack[2];  // of the caller's numbering, of the relabelled copy
+    int32_t wG64 = 0;  // sources that wdist, wsigma, wcval hold (64-bit kernel)
     // the weighted sweep's relabelled copy of the graph (built on first
     // use): the CSR (and a directed graph's in-arc CSR) in a numbering with
     // locality, old -> new ids (wperm, also on the host) and new -> old
@@ -429,6 +435,8 @@ void free_graph(bc_graph *g) {
         if (g->side[i]) cudaStreamDestroy(g->side[i]);
     }
     if (g->side_fork) cudaEventDestroy(g->side_fork);
+    for (auto &pk : g->wpack)
+        for (auto *b : {&pk.arc, &pk.arc_in, &pk.rec, &pk.rec_in}) b->release();
     g->wds.release();
     g->wredo.release();
     g->bc.release();
@@ -1572,14 +1580,33 @@ int ensure_relabel(bc_graph *g) {
     return BC_OK;
 }
 
+// Packed arcs and records of the packed kernel, for one numbering; once per
+// handle.
+int ensure_packed(bc_graph *g, bool relabel, cudaStream_t st) {
+    auto &pk = g->wpack[relabel ? 1 : 0];
+    if (pk.ready || g->n > bcgb::kWPackN) return BC_OK;
+    const int sms = sm_count_host();
+    const size_t m = (size_t)std::max<int64_t>(g->narcs, 1), r = 8 * (size_t)std::max(g->n, 1);
+    CK(pk.arc.ensure(m));
+    CK(pk.rec.ensure(r));
+    bcgb::w_pack_arcs(relabel ? g->prow_ptr.p : g->row_ptr.p, relabel ? g->pcol.p : g->col.p,
+                      relabel ? g->pw.p : g->w.p, g->n, g->narcs, pk.arc.p, pk.rec.p, sms, st);
+    if (g->directed) {
+        CK(pk.arc_in.ensure(m));
+        CK(pk.rec_in.ensure(r));
+        bcgb::w_pack_arcs(relabel ? g->prow_ptr_in.p : g->row_ptr_in.p, relabel ? g->pcol_in.p : g->col_in.p,
+                          relabel ? g->pw_in.p : g->w_in.p, g->n, g->narcs, pk.arc_in.p, pk.rec_in.p, sms, st);
+    }
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(st));  // a later call may come on another stream
+    pk.ready = true;
+    return BC_OK;
+}
+
 // Weighted sweep (csrc/sssp_packed.cu; csrc/sssp_weighted.cu for 64-bit
 // counts): waves of G sources, one CTA each. G is opt->batch if set, else
-// kWSmallPerSm sources per SM for the 128-thread CTAs of small graphs, else
-// three per SM, two of them resident (512-thread CTAs: on the relabelled
-// 512x512 grid 1 / 2 / 3 / 4 per SM measured 258 / 257 / 241 / 252 ms, with
-// 256-thread CTAs 274 / 255 / 253 / 256; on the caller's row-major numbering
-// more sources in flight only added random DRAM sectors), capped so the wave
-// state stays within 8 GiB. Waves run on
+// as many sources as are resident (w_packed_per_sm; 512-thread CTAs: three per
+// SM, two of them resident), capped so the wave state stays within 8 GiB. Waves run on
 // kWeightedLanes lanes: wave k runs on lane k % lanes, each with its own stream,
 // state, delta rows and BC accumulator, so one wave's slowest sources overlap
 // the next waves. The delta rows of a wave are added to its lane's BC in
@@ -1589,7 +1616,6 @@ int ensure_relabel(bc_graph *g) {
 // they are flagged and computed again at the end by the 64-bit kernel, whose
 // delta rows are added in the order of the flagged sources.
 constexpr int kWeightedLanes = 2;  // measured: 3 or 4 lanes no faster on the 512x512 grid
-constexpr int kWSmallPerSm = 8;    // wave of the 128-thread CTAs (small graphs), per SM: all resident
 
 constexpr double kWeightedLaneBudget = 24.0 * (1 << 30);  // packed wave state of all lanes
 
@@ -1600,10 +1626,12 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
     if (K > bcgb::kMaxRing)
         return fail(BC_ERR_UNSUPPORTED, "weighted path: maximum weight must be below " +
                                             std::to_string(bcgb::kMaxRing));
-    int C = (int)std::min<int64_t>(std::max<int64_t>(1024, (4ll << 20) / K / 4), (int64_t)n + 1);
-    C = std::max(C, 64);
-    const size_t per_src = (size_t)n * (4 + 8 + 4 + 4 + 4 + 4 + 8) + 4 + (size_t)K * C * 4;
-    const int per_sm = bcgb::w_packed_threads(n) == 128 ? kWSmallPerSm : 3;
+    // bucket entries: four times their mean number if the ring held every vertex
+    // once, up to 4 MB a source (a fuller bucket is read by a scan over the vertices)
+    const int C = (int)std::min<int64_t>({std::max<int64_t>(64, 4 * (((int64_t)n + K - 1) / K)),
+                                          std::max<int64_t>(1024, (1ll << 20) / K), (int64_t)n + 64});
+    const size_t per_src = (size_t)n * (8 + 4 + 4 + 4) + 4 + (size_t)K * C * 4;
+    const int per_sm = bcgb::w_packed_per_sm(n, g->maxw);
     int G = (opt && opt->batch > 0) ? opt->batch : per_sm * sm_count_host();
     G = (int)std::min<size_t>((size_t)G, std::max<size_t>(1, (8ull << 30) / per_src));
     G = std::max(1, std::min(G, std::max(nsrc, 1)));
@@ -1614,9 +1642,6 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
     int lanes = g->timing ? 1 : std::min<int32_t>(kWeightedLanes, nwaves);
     while (lanes > 1 && lanes * lane_bytes > kWeightedLaneBudget) --lanes;
     if (g->wG < G || g->wK != K || g->wC != C) {
-        CK(g->wdist.ensure((size_t)G * n));
-        CK(g->wsigma.ensure((size_t)G * n));
-        CK(g->wcval.ensure((size_t)G * n));
         CK(g->worder.ensure((size_t)G * n));
         CK(g->wgrp.ensure((size_t)G * (n + 1)));
         CK(g->wslots.ensure((size_t)G * K * C));
@@ -1674,6 +1699,17 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
         base.col_in = relabel ? g->pcol_in.p : g->col_in.p;
         base.w_in = relabel ? g->pw_in.p : g->w_in.p;
     }
+    if (n <= bcgb::kWPackN) {
+        const int r = ensure_packed(g, relabel, st);
+        if (r) return r;
+        const auto &pk = g->wpack[relabel ? 1 : 0];
+        base.rec = reinterpret_cast<const uint4 *>(pk.rec.p);
+        base.arc = pk.arc.p;
+        if (g->directed) {
+            base.rec_in = reinterpret_cast<const uint4 *>(pk.rec_in.p);
+            base.arc_in = pk.arc_in.p;
+        }
+    }
     base.ctl = g->ctl;
     for (int32_t k = 0; k < nwaves; ++k) {
         const int32_t w0 = k * G;
@@ -1724,8 +1760,16 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
             rpos.push_back(i);
             rsrc.push_back(relabel ? g->h_wperm[(size_t)g->h_sources[(size_t)i]] : g->h_sources[(size_t)i]);
         }
-    for (size_t r0 = 0; r0 < rpos.size(); r0 += (size_t)G) {
-        const int nr = (int)std::min<size_t>((size_t)G, rpos.size() - r0);
+    // its launches hold at most three sources per SM (its CTAs are 256 threads)
+    const int G64 = std::min(G, 3 * sm_count_host());
+    if (!rpos.empty() && g->wG64 < G64) {
+        CK(g->wdist.ensure((size_t)G64 * n));
+        CK(g->wsigma.ensure((size_t)G64 * n));
+        CK(g->wcval.ensure((size_t)G64 * n));
+        g->wG64 = G64;
+    }
+    for (size_t r0 = 0; r0 < rpos.size(); r0 += (size_t)G64) {
+        const int nr = (int)std::min<size_t>((size_t)G64, rpos.size() - r0);
         CK(cudaMemcpyAsync(g->wpos.p, rpos.data() + r0, (size_t)nr * sizeof(int32_t), cudaMemcpyHostToDevice, st));
         CK(cudaMemcpyAsync(g->wsrc.p, rsrc.data() + r0, (size_t)nr * sizeof(int32_t), cudaMemcpyHostToDevice, st));
         bcgb::WParams p = base;
@@ -2296,8 +2340,8 @@ int bc_autotune(bc_graph *g, int32_t sample, bc_options *out, void *cuda_stream)
         return BC_OK;
     };
     if (g->weighted) {
-        // sources per wave of the bucket kernel: 1 to 4 or 8 per SM
-        for (int per : {1, 2, 3, 4, 8}) {
+        // sources per wave of the bucket kernel: 1 to 32 per SM
+        for (int per : {1, 2, 3, 4, 8, 16, 32}) {
             bc_options o{};
             o.flags = BC_NO_HASH;
             o.batch = per * sm_count_host();

@@ -292,13 +292,26 @@ __global__ void __launch_bounds__(kWBlock, 4) k_wsssp(const WParams p) {
     }
 }
 
-// BC(v) += sum over the wave's rows in row order (FP64).
+// BC(v) += sum over the wave's rows (FP64, a fixed order: eight interleaved
+// runs of rows, then those). A block takes 32 vertices; one run per warp keeps
+// eight times as many loads in flight as one chain of all rows per vertex.
 __global__ void __launch_bounds__(256) k_wreduce(const float *__restrict__ rows, int32_t nrows, int32_t n,
                                                  const int32_t *__restrict__ vid, double *__restrict__ bc) {
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+    __shared__ double s_sum[8][33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    for (int v0 = 32 * blockIdx.x; v0 < n; v0 += 32 * gridDim.x) {
+        const int v = v0 + x;
         double acc = 0.0;
-        for (int r = 0; r < nrows; ++r) acc += (double)rows[(size_t)r * n + v];
-        bc[vid ? vid[v] : v] += acc;
+        if (v < n)
+#pragma unroll 4
+            for (int r = y; r < nrows; r += 8) acc += (double)rows[(size_t)r * n + v];
+        s_sum[y][x] = acc;
+        __syncthreads();
+        if (y == 0 && v < n) {
+            for (int q = 1; q < 8; ++q) acc += s_sum[q][x];
+            bc[vid ? vid[v] : v] += acc;
+        }
+        __syncthreads();
     }
 }
 
@@ -310,8 +323,8 @@ void w_launch_wave(const WParams &p, int nsrc, cudaStream_t st) {
 
 void w_launch_reduce(const float *rows, int nrows, int n, const int32_t *vid, double *bc, int sms,
                      cudaStream_t st) {
-    int g = (n + 255) / 256;
-    g = g > 4 * sms ? 4 * sms : (g < 1 ? 1 : g);
+    int g = (n + 31) / 32;
+    g = g > 8 * sms ? 8 * sms : (g < 1 ? 1 : g);
     k_wreduce<<<g, 256, 0, st>>>(rows, nrows, n, vid, bc);
 }
 

@@ -11,6 +11,11 @@ namespace bcgb {
 
 constexpr int kMaxRing = 4096;  // bucket ring size limit: max weight < kMaxRing
 
+constexpr int kArcWBits = 12;  // packed arc: head << 12 | weight (weights are below kMaxRing = 2^12)
+constexpr uint32_t kArcWMask = (1u << kArcWBits) - 1u;
+static_assert(kMaxRing == 1 << kArcWBits, "a packed arc holds every weight of the bucket path");
+constexpr int32_t kWPackN = (1 << (32 - kArcWBits)) - 1;  // n at most this: every packed arc is below the end marks
+
 struct WParams {
     int32_t n;
     int32_t K;     // ring size (> max weight)
@@ -22,6 +27,10 @@ struct WParams {
     const int32_t *col_in;
     const int32_t *w_in;
     const int32_t *w;
+    const uint4 *rec;         // packed kernel: the first arcs of each row as a 32-byte record, and
+    const uint32_t *arc;      // the packed arcs (null above kWPackN vertices: it reads the CSR)
+    const uint4 *rec_in;
+    const uint32_t *arc_in;
     const int32_t *sources;  // this wave's sources
     const int32_t *vid;      // the caller's id of each vertex when the graph was relabelled (null: the same);
                              // summaries and rows use the caller's ids
@@ -51,16 +60,33 @@ struct WParams {
 void locality_order(int32_t n, const int32_t *row_ptr, const int32_t *col, int32_t *perm);
 void launch_map_ids(const int32_t *perm, const int32_t *in, int32_t *out, int32_t k, cudaStream_t st);
 
+// Packed arcs of a CSR and the records of its rows (rec [8 n]).
+void w_pack_arcs(const int32_t *row_ptr, const int32_t *col, const int32_t *w, int n, int64_t m, uint32_t *arc,
+                 uint32_t *rec, int sms, cudaStream_t st);
 void w_launch_wave(const WParams &p, int nsrc, cudaStream_t st);         // 64-bit counts
 void w_launch_wave_packed(const WParams &p, int nsrc, cudaStream_t st);  // packed state, 32-bit counts
-// Threads per source of the packed kernel: a distance step settles about n /
-// (distinct distances) vertices, so small graphs leave wide CTAs idle at every
-// barrier while large ones need the threads. Square grids with 5% long-range
-// edges, best wave of each (ms): n = 4096 (all sources) 128 threads 18.1, 512
-// threads 58.2; n = 16384 (2048 sources) 11.8 / 35.0; n = 65536 30.5 / 41.0;
-// n = 262144 146.4 / 123.4. The switch sits between the last two sizes.
+// Threads per source of the packed kernel. A distance step settles n / (distinct
+// distances) vertices, and the number of distinct distances grows with the
+// largest weight, so n / maxw stands for a step's width: narrow steps leave
+// wide CTAs idle at every barrier, wide ones are worked through in turns by
+// narrow CTAs. Square grids with 5% long-range edges, weights 1..maxw, all
+// sources up to n = 4096, else 2048; ms with 32 / 64 / 128 / 256 threads (and as
+// many sources resident as 64 registers a thread allow); the 128-thread
+// kernel before records, ballots and one-warp sources in brackets:
+//   n = 2304,  maxw 100 (width 23):   1.53 / 1.86 / 2.82 / 5.10  (3.56)
+//   n = 4096,  maxw 100 (width 41):   3.12 / 3.91 / 6.06 / 10.1  (7.88)
+//   n = 10000, maxw 100 (width 100):  4.29 / 4.06 / 4.68 / 7.44  (5.82)
+//   n = 17956, maxw 100 (width 180):  8.36 / 7.96 / 7.47 / 9.83  (9.19)
+//   n = 1024,  maxw 3   (width 341):  0.30 / 0.27 / 0.24 / 0.30  (0.38)
+//   n = 10000, maxw 3   (width 3333): 3.00 / 2.69 / 2.09 / 2.13  (2.71)
+//   n = 17956, maxw 3   (width 5985): 6.54 / 6.10 / 4.55 / 3.60  (5.58)
+// From kWSmallN vertices on a source's state (8 n bytes) no longer fits L2
+// beside the others', and fewer, wider sources win: n = 262144, maxw 100, 4096
+// sources, 256 threads at four per SM 246 ms, 512 at three per SM (two
+// resident) 221 ms (241 before).
 constexpr int32_t kWSmallN = 131072;
-int w_packed_threads(int32_t n);
+int w_packed_threads(int32_t n, int32_t maxw);
+int w_packed_per_sm(int32_t n, int32_t maxw);  // sources per SM of a default wave
 // bc[vid[v]] += the FP64 sum over r < nrows of rows[r][v], rows in order (vid null: bc[v])
 void w_launch_reduce(const float *rows, int nrows, int n, const int32_t *vid, double *bc, int sms,
                      cudaStream_t st);
