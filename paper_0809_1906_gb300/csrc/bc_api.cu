@@ -190,14 +190,17 @@ bool device_writable(const T *p) {
 // Work items of one level sweep: one per vertex, except vertices with more
 // than `chunk` arcs, which are split into chunks combining through slots.
 struct ItemPlan {
-    int32_t chunk = 0, nitems = 0, nslots = 0;
-    DevBuf<int32_t> blob;  // item_v, item_beg, item_end, item_slot [nitems], slot_first, slot_nch [nslots]
-    const int32_t *item_v = nullptr, *item_beg = nullptr, *item_end = nullptr, *item_slot = nullptr;
+    int32_t chunk = 0, nitems = 0, nheavy = 0, nslots = 0;
+    DevBuf<int32_t> blob;  // items (vertex, first arc, end, slot) [nitems][4], their vertices
+                           // [nitems], slot_first, slot_nch [nslots]
+    const int4 *items = nullptr;
+    const int32_t *item_v = nullptr;
     const int32_t *slot_first = nullptr, *slot_nch = nullptr;
     void release() {
         blob.release();
-        item_v = item_beg = item_end = item_slot = slot_first = slot_nch = nullptr;
-        chunk = nitems = nslots = 0;
+        items = nullptr;
+        item_v = slot_first = slot_nch = nullptr;
+        chunk = nitems = nheavy = nslots = 0;
     }
 };
 
@@ -513,11 +516,11 @@ int check_graph(int32_t n, const std::vector<int32_t> &rp, const std::vector<int
 // which are split into chunks that combine through partial slots. Heavy
 // chunks come first, then vertices by descending degree.
 int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int32_t> &rp) {
-    if (pl.chunk == chunk && pl.item_v) return BC_OK;
+    if (pl.chunk == chunk && pl.items) return BC_OK;
     const int32_t n = g->n;
     // items: the chunks of the split vertices (in vertex order), then the
     // other vertices by decreasing degree (a stable counting sort: degree <= chunk)
-    int64_t nitems = 0, nslots = 0;
+    int64_t nitems = 0, nslots = 0, nlight = 0;
     std::vector<int32_t> cnt((size_t)chunk + 2, 0);
     for (int32_t v = 0; v < n; ++v) {
         const int64_t deg = rp[v + 1] - rp[v];
@@ -528,13 +531,21 @@ int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int3
         } else {
             ++cnt[(size_t)(chunk - deg) + 1];
             ++nitems;
+            if (deg <= bcgb::kLightDeg) ++nlight;
         }
     }
     for (size_t x = 1; x < cnt.size(); ++x) cnt[x] += cnt[x - 1];
-    // one host block, one device allocation and one copy for the six arrays
-    std::vector<int32_t> h((size_t)(4 * nitems + 2 * nslots));
-    int32_t *iv = h.data(), *ib = iv + nitems, *ie = ib + nitems, *is = ie + nitems;
-    int32_t *sf = is + nitems, *sn = sf + nslots;
+    // one host block, one device allocation and one copy for the items and slots
+    std::vector<int32_t> h((size_t)(5 * nitems + 2 * nslots));
+    int32_t *sf = h.data() + 5 * nitems, *sn = sf + nslots;
+    auto put = [&](int64_t at, int32_t v, int64_t beg, int64_t end, int64_t slot) {
+        int32_t *x = h.data() + 4 * at;
+        x[0] = v;
+        x[1] = (int32_t)beg;
+        x[2] = (int32_t)end;
+        x[3] = (int32_t)slot;
+        h[(size_t)(4 * nitems + at)] = v;
+    };
     int64_t k = 0;
     for (int32_t v = 0; v < n; ++v) {
         const int64_t deg = rp[v + 1] - rp[v];
@@ -542,10 +553,7 @@ int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int3
         const int64_t nch = (deg + chunk - 1) / chunk;
         const int32_t first = (int32_t)k;
         for (int64_t c = 0; c < nch; ++c, ++k) {
-            iv[k] = v;
-            ib[k] = (int32_t)(rp[v] + c * chunk);
-            ie[k] = (int32_t)std::min<int64_t>(rp[v + 1], rp[v] + (c + 1) * chunk);
-            is[k] = (int32_t)k;
+            put(k, v, rp[v] + c * chunk, std::min<int64_t>(rp[v + 1], rp[v] + (c + 1) * chunk), k);
             sf[k] = first;
             sn[k] = (int32_t)nch;
         }
@@ -554,20 +562,16 @@ int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int3
         const int64_t deg = rp[v + 1] - rp[v];
         if (deg > chunk) continue;
         const int64_t t = nslots + cnt[(size_t)(chunk - deg)]++;
-        iv[t] = v;
-        ib[t] = rp[v];
-        ie[t] = rp[v + 1];
-        is[t] = -1;
+        put(t, v, rp[v], rp[v + 1], -1);
     }
     pl.nitems = (int32_t)nitems;
+    pl.nheavy = (int32_t)(nitems - nlight);
     pl.nslots = (int32_t)nslots;
     CK(pl.blob.ensure(h.size()));
     if (!h.empty()) CK(cudaMemcpy(pl.blob.p, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    pl.item_v = pl.blob.p;
-    pl.item_beg = pl.item_v + nitems;
-    pl.item_end = pl.item_beg + nitems;
-    pl.item_slot = pl.item_end + nitems;
-    pl.slot_first = pl.item_slot + nitems;
+    pl.items = reinterpret_cast<const int4 *>(pl.blob.p);
+    pl.item_v = pl.blob.p + 4 * nitems;
+    pl.slot_first = pl.item_v + nitems;
     pl.slot_nch = pl.slot_first + nslots;
     pl.chunk = chunk;
     // partial slots depend on the plans: force the state to be re-sized
@@ -591,10 +595,9 @@ int build_plans(bc_graph *g, const bc_options *opt) {
 
 void use_plan(bcgb::MsParams &p, const ItemPlan &pl) {
     p.nitems = pl.nitems;
+    p.items = pl.items;
     p.item_v = pl.item_v;
-    p.item_beg = pl.item_beg;
-    p.item_end = pl.item_end;
-    p.item_slot = pl.item_slot;
+    p.nheavy = pl.nheavy;
     p.slot_first = pl.slot_first;
     p.slot_nch = pl.slot_nch;
 }

@@ -77,9 +77,12 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x) {
 }
 #endif
 
+constexpr int kLightDeg = 8;  // a light vertex has at most this many arcs (msbfs_light.cuh)
+
 struct MsParams {
     int32_t n;
     int32_t nitems;
+    int32_t nheavy;  // the first of them one warp each, the others (at most kLightDeg arcs) in packs
     int32_t nw32;  // words of one union-frontier bitmap
     int32_t Lcap;  // level slots in F / ufr
     int32_t nb;    // sources in this batch (<= B)
@@ -89,10 +92,8 @@ struct MsParams {
     const int32_t *row_ptr;  // out-arcs: level 0->1 and the backward sweep
     const int32_t *col;
     const int32_t *col_f;    // arcs the forward sweep pulls over: in-arcs (= col when undirected)
-    const int32_t *item_v;
-    const int32_t *item_beg;
-    const int32_t *item_end;
-    const int32_t *item_slot;   // -1: whole vertex; else partial slot of a chunk
+    const int4 *items;  // work items: vertex, first arc, end, partial slot of a chunk (-1: the whole vertex)
+    const int32_t *item_v;  // their vertices alone
     const int32_t *slot_first;  // first slot of the chunk's vertex
     const int32_t *slot_nch;    // number of chunks of that vertex
     const int32_t *sources;     // this batch's source ids [nb]

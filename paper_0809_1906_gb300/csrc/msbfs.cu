@@ -28,6 +28,7 @@
 
 #include "bc_internal.cuh"
 #include "msbfs_body.cuh"
+#include "msbfs_light.cuh"
 #include "pdl.cuh"
 
 namespace bcgb {
@@ -47,6 +48,12 @@ using body::transpose32;
 constexpr uint32_t kFilterRatio = 32;
 __device__ __forceinline__ bool filter_level(const MsParams &p, int l) {
     return p.lsize == nullptr || (uint64_t)p.lsize[l] * kFilterRatio < (uint64_t)p.n;
+}
+
+// Light vertices that a warp takes at a time.
+__device__ __forceinline__ int light_share(int nlight, int warps) {
+    const int c = (nlight + warps - 1) / warps;
+    return c < 32 ? c : 32;
 }
 
 template <int W>
@@ -212,13 +219,12 @@ __global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const i
     // item k's vertex (visited words; the new frontier row cleared when
     // nothing is left to find), then the warp works through the active ones.
     const int G = gridDim.x * kWarps;
-    for (int g0 = blockIdx.x * kWarps + wib; g0 < p.nitems; g0 += 32 * G) {
+    for (int g0 = blockIdx.x * kWarps + wib; g0 < p.nheavy; g0 += 32 * G) {
         bool act = false;
         __syncwarp();  // the previous group's reads of s_U are done
         const int ik = g0 + lane * G;
-        if (ik < p.nitems) {
+        if (ik < p.nheavy) {
             const int vk = p.item_v[ik];
-            const int sk = p.item_slot[ik];
             uint32_t a[W], f[W];
             load_row<W>(Vin + (size_t)vk * W, a);
             load_row<W>(Fl + (size_t)vk * W, f);
@@ -232,20 +238,20 @@ __global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const i
                 any |= u;
             }
             act = any != 0u;
-            if (!act && (sk < 0 || p.slot_first[sk] == sk))
+            if (!act) {  // nothing left to find: the new frontier row is empty
+                const int sk = __ldg(&p.items[ik].w);
+                if (sk < 0 || p.slot_first[sk] == sk)
 #pragma unroll
-                for (int j = 0; j < W; ++j) Fn[(size_t)vk * W + j] = 0u;
+                    for (int j = 0; j < W; ++j) Fn[(size_t)vk * W + j] = 0u;
+            }
         }
         unsigned todo = __ballot_sync(kFull, act);
         __syncwarp();
         while (todo) {
             const int kk = __ffs(todo) - 1;
             todo &= todo - 1;
-            const int it = g0 + kk * G;
-            const int v = p.item_v[it];
-            const int beg = p.item_beg[it];
-            const int end = p.item_end[it];
-            const int slot = p.item_slot[it];
+            const int4 item = __ldg(p.items + g0 + kk * G);
+            const int v = item.x, beg = item.y, end = item.z, slot = item.w;
             uint32_t U[W];
 #pragma unroll
             for (int j = 0; j < W; ++j) U[j] = s_U[wib][kk][j];
@@ -301,6 +307,41 @@ __global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const i
             if (joined && lane == 0) atomicAdd(&s_front, 1u);
             if (lane == 0) p.cnt[first] = 0u;
         }
+    }
+    // light vertices (the items' tail): a warp takes up to 32 consecutive ones,
+    // an even share when there are fewer, and works through them pack by pack
+    const int nlight = p.nitems - p.nheavy;
+    const int share = light_share(nlight, G);
+    // from the last warp down: the first ones have the more heavy items
+    for (int g0 = (G - 1 - (int)(blockIdx.x * kWarps + wib)) * share; g0 < nlight; g0 += G * share) {
+        bool act = false;
+        int4 item = make_int4(0, 0, 0, 0);
+        __syncwarp();  // the previous group's reads of s_U are done
+        if (lane < share && g0 + lane < nlight) {
+            item = __ldg(p.items + p.nheavy + g0 + lane);
+            uint32_t a[W], f[W];
+            load_row<W>(Vin + (size_t)item.x * W, a);
+            load_row<W>(Fl + (size_t)item.x * W, f);
+            uint32_t any = 0;
+#pragma unroll
+            for (int j = 0; j < W; ++j) {
+                const uint32_t vis = a[j] | f[j];
+                Vout[(size_t)item.x * W + j] = vis;
+                const uint32_t u = ~vis & valid_word(p.nb, j);
+                s_U[wib][lane][j] = u;
+                any |= u;
+            }
+            act = any != 0u && item.y < item.z;
+            if (!act)
+#pragma unroll
+                for (int j = 0; j < W; ++j) Fn[(size_t)item.x * W + j] = 0u;
+        }
+        const unsigned lt = __ballot_sync(kFull, act);
+        __syncwarp();
+        if (lt)
+            body::fwd_light<W, true>(lt, item.x, item.y, item.z - item.y, s_U[wib],
+                                     *reinterpret_cast<body::LightScratch<W> *>(ws.buf), p.col_f, ufl_f, Fl, Sl,
+                                     p.sigma, wide, ones, Sn, Fn, ufn, lane, ovf, arcs, produced, wide_next, &s_front);
     }
     const unsigned wovf = __ballot_sync(kFull, ovf);
     const unsigned wwide = __ballot_sync(kFull, wide_next);
@@ -409,11 +450,11 @@ __global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const 
     // k-th next item's vertex is at level l for any source (the same for all
     // chunks of v), then the warp works through the active items
     const int G = gridDim.x * kWarps;
-    for (int g0 = blockIdx.x * kWarps + wib; g0 < p.nitems; g0 += 32 * G) {
+    for (int g0 = blockIdx.x * kWarps + wib; g0 < p.nheavy; g0 += 32 * G) {
         bool act = false;
         __syncwarp();  // the previous group's reads of s_f are done
         const int ik = g0 + lane * G;
-        if (ik < p.nitems) {
+        if (ik < p.nheavy) {
             const int vk = p.item_v[ik];
             uint32_t f[W];
             load_row<W>(Fl + (size_t)vk * W, f);
@@ -436,11 +477,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const 
                 const unsigned k2 = __fns(todo, 0, 2);  // two active items ahead
                 if (k2 < 32u) prefetch_sigma((int)k2);
             }
-            const int it = g0 + kk * G;
-            const int v = p.item_v[it];
-            const int beg = p.item_beg[it];
-            const int end = p.item_end[it];
-            const int slot = p.item_slot[it];
+            const int4 item = __ldg(p.items + g0 + kk * G);
+            const int v = item.x, beg = item.y, end = item.z, slot = item.w;
             uint32_t f[W];
 #pragma unroll
             for (int j = 0; j < W; ++j) f[j] = s_f[wib][kk][j];
@@ -497,6 +535,33 @@ __global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const 
             body::finalize_dep<W>(p.sigma, Sl, sig_ones, Cl, p.bc, v, f, S, lane);
             if (lane == 0) p.cnt[first] = 0u;
         }
+    }
+    // light vertices, as in the forward sweep
+    const int nlight = p.nitems - p.nheavy;
+    const int share = light_share(nlight, G);
+    // from the last warp down: the first ones have the more heavy items
+    for (int g0 = (G - 1 - (int)(blockIdx.x * kWarps + wib)) * share; g0 < nlight; g0 += G * share) {
+        bool act = false;
+        int4 item = make_int4(0, 0, 0, 0);
+        __syncwarp();  // the previous group's reads of s_f are done
+        if (lane < share && g0 + lane < nlight) {
+            item = __ldg(p.items + p.nheavy + g0 + lane);
+            uint32_t f[W];
+            load_row<W>(Fl + (size_t)item.x * W, f);
+            uint32_t any = 0;
+#pragma unroll
+            for (int j = 0; j < W; ++j) {
+                s_f[wib][lane][j] = f[j];
+                any |= f[j];
+            }
+            act = any != 0u;
+        }
+        const unsigned lt = __ballot_sync(kFull, act);
+        __syncwarp();
+        if (lt)
+            body::bwd_light<W, true, true>(lt, item.x, item.y, item.z - item.y, s_f[wib],
+                                           *reinterpret_cast<body::LightScratch<W> *>(ws.buf), p.col, ufs_f, Fs, Cs,
+                                           p.sigma, Sl, sig_ones, Cl, p.bc, lane);
     }
     if (lane == 0 && ws.fail) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
 }
@@ -678,6 +743,8 @@ int sm_count() {
 }
 
 // dynamic shared memory of the level kernels: one row stage per warp
+static_assert(sizeof(body::LightScratch<8>) <= stage::kFwdStageBytes && sizeof(body::LightScratch<8>) <= stage::kBwdStageBytes,
+              "a pack's scratch shares the warp's row stage");
 constexpr size_t kFwdSmem = (size_t)kWarps * stage::kFwdStageBytes;
 constexpr size_t kBwdSmem = (size_t)kWarps * stage::kBwdStageBytes;
 

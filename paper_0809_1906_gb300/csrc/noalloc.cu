@@ -43,7 +43,7 @@ constexpr size_t kOffF = align256(kOffCval + (size_t)2 * kMaxN * kB * sizeof(flo
 constexpr size_t kOffUfr = align256(kOffF + (size_t)kLcap * kMaxN * kW * sizeof(uint32_t));
 constexpr size_t kOffV = align256(kOffUfr + (size_t)kLcap * kNw32 * sizeof(uint32_t));
 constexpr size_t kOffItems = align256(kOffV + (size_t)2 * kMaxN * kW * sizeof(uint32_t));
-constexpr size_t kOffSrc = align256(kOffItems + (size_t)4 * kMaxN * sizeof(int32_t));
+constexpr size_t kOffSrc = align256(kOffItems + (size_t)5 * kMaxN * sizeof(int32_t));
 constexpr size_t kOffCtl = align256(kOffSrc + (size_t)kMaxN * sizeof(int32_t));
 constexpr size_t kOffHctl = align256(kOffCtl + sizeof(bcgb::DevCtl));
 constexpr size_t kOffDummy = align256(kOffHctl + sizeof(bcgb::HostCtl));
@@ -79,18 +79,16 @@ cudaError_t scratch_address(unsigned char **out) {
 // Also writes the work items (one per vertex) and, when sources is null, the
 // list 0..n-1. Any violation sets bit 1 of *bad.
 __global__ void k_noalloc_prepare(int32_t n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                                  const int32_t *__restrict__ sources, int32_t nsrc, int32_t *items,
-                                  int32_t *iota, uint32_t *bad) {
+                                  const int32_t *__restrict__ sources, int32_t nsrc, int4 *items,
+                                  int32_t *item_v, int32_t *iota, uint32_t *bad) {
     const int stride = gridDim.x * blockDim.x;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     if (tid == 0 && row_ptr[0] != 0) atomicOr(bad, 1u);
     for (int v = tid; v < n; v += stride) {
         const int a = row_ptr[v], b = row_ptr[v + 1];
         if (b < a) atomicOr(bad, 1u);
-        items[v] = v;                 // item_v
-        items[kMaxN + v] = a;         // item_beg
-        items[2 * kMaxN + v] = b;     // item_end
-        items[3 * kMaxN + v] = -1;    // item_slot: no split vertices here
+        items[v] = make_int4(v, a, b, -1);  // no split vertices here
+        item_v[v] = v;
         if (!sources) iota[v] = v;
     }
     const int m2 = row_ptr[n];
@@ -117,16 +115,16 @@ extern "C" int bc_run_noalloc(int32_t n, const int32_t *row_ptr, const int32_t *
     bcgb::MsParams p{};
     p.n = n;
     p.nitems = n;
+    p.nheavy = n;  // in vertex order: the light ones are not set apart
     p.nw32 = (n + 31) / 32;
     p.Lcap = kLcap;
     p.row_ptr = row_ptr;
     p.col = col;
     p.col_f = col;  // undirected: the forward pulls over the same arcs
-    int32_t *items = reinterpret_cast<int32_t *>(base + kOffItems);
-    p.item_v = items;
-    p.item_beg = items + kMaxN;
-    p.item_end = items + 2 * kMaxN;
-    p.item_slot = items + 3 * kMaxN;
+    int4 *items = reinterpret_cast<int4 *>(base + kOffItems);
+    int32_t *item_v = reinterpret_cast<int32_t *>(items + kMaxN);
+    p.items = items;
+    p.item_v = item_v;
     int32_t *dummy = reinterpret_cast<int32_t *>(base + kOffDummy);
     p.slot_first = dummy;  // never read: no item has a slot
     p.slot_nch = dummy;
@@ -149,7 +147,7 @@ extern "C" int bc_run_noalloc(int32_t n, const int32_t *row_ptr, const int32_t *
     // the scratch keeps the previous call's contents: clear what must start at zero
     if (cudaMemsetAsync(p.ctl, 0, sizeof(bcgb::DevCtl), st) != cudaSuccess) return BC_ERR_CUDA;
     if (cudaMemsetAsync(bc, 0, (size_t)n * sizeof(double), st) != cudaSuccess) return BC_ERR_CUDA;
-    k_noalloc_prepare<<<64, 256, 0, st>>>(n, row_ptr, col, sources, nsrc, items, iota, &p.ctl->pad[0]);
+    k_noalloc_prepare<<<64, 256, 0, st>>>(n, row_ptr, col, sources, nsrc, items, item_v, iota, &p.ctl->pad[0]);
     uint32_t bad = 0;
     if (cudaMemcpyAsync(&bad, &p.ctl->pad[0], sizeof(bad), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
