@@ -191,7 +191,7 @@ bool device_writable(const T *p) {
 // than `chunk` arcs, which are split into chunks combining through slots.
 struct ItemPlan {
     int32_t chunk = 0, nitems = 0, nheavy = 0, nslots = 0;
-    DevBuf<int32_t> blob;  // items (vertex, first arc, end, slot) [nitems][4], their vertices
+    DevBuf<int32_t> blob;  // items (vertex, first arc, end, 0) [nitems][4], their vertices
                            // [nitems], slot_first, slot_nch [nslots]
     const int4 *items = nullptr;
     const int32_t *item_v = nullptr;
@@ -204,6 +204,11 @@ struct ItemPlan {
     }
 };
 
+// A handle's control block: DevCtl, then the sweep's finish counter and barrier
+// words, cleared together before a run.
+constexpr size_t kCtlSweepAt = 256;
+static_assert(sizeof(bcgb::DevCtl) <= kCtlSweepAt - 128, "the finish counter lies between the two");
+constexpr size_t kCtlBytes = kCtlSweepAt + bcgb::kSweepSyncBytes;
 constexpr int kSweepLanes = 8;                    // concurrent batches of the unweighted sweep
 constexpr int kSideStreams = 4;                   // side streams of the dense path's per-batch summaries
 constexpr double kLaneBudgetBytes = 8.0 * (1 << 30);  // batch state of the extra lanes
@@ -322,8 +327,15 @@ struct bc_graph {
     DevBuf<int32_t> sources;
     DevBuf<int32_t> src_index;  // caller's index of each staged source (reordered runs)
     bool reordered = false;
-    DevBuf<uint64_t> h_sigma, h_dist;
-    DevBuf<int64_t> dist_sum, reach;
+    // per-source summaries, four rows of one block (ensure_summaries)
+    DevBuf<uint64_t> summ;
+    size_t summ_row = 0;  // entries of a row
+    struct {
+        uint64_t *p = nullptr;
+    } h_sigma, h_dist;
+    struct {
+        int64_t *p = nullptr;
+    } dist_sum, reach;
     int32_t last_nsrc = 0;
     bool has_run = false, has_hash = false;
     cudaStream_t last_stream = nullptr;
@@ -364,6 +376,15 @@ struct bc_graph {
     DevBuf<uint32_t> gF, gV, gufr;
     DevBuf<double> gbcpart;
     DevBuf<int32_t> gmeta;  // [3][gNB]: active list, valid sources, depth
+
+    // the one-launch sweep: group 0's BC sums (its barrier words follow the control block)
+    DevBuf<double> sweep_bc;
+    bool clear_pending = false;  // clear_outputs has still to run
+    // ctl->status as last read from the device, current while status_known
+    uint32_t status = 0;
+    bool status_known = false;
+    std::vector<uint64_t> summ_host;  // bc_source_hashes
+    int staged_all = 0;  // `sources` holds every vertex: 1 in id order, 2 in landmark order (0: anything else)
 
     // weighted algebraic forward (BC_DENSE on a weighted graph): in-arcs by weight class
     DevBuf<int32_t> mpcol, mpw;
@@ -417,6 +438,7 @@ void free_graph(bc_graph *g) {
     g->part.release();
     g->cval.release();
     for (auto *b : {&g->F, &g->ufr, &g->V, &g->pmask, &g->cnt}) b->release();
+    g->sweep_bc.release();
     g->mpcol.release();
     g->mpw.release();
     g->gsigma.release();
@@ -443,10 +465,7 @@ void free_graph(bc_graph *g) {
     g->wds.release();
     g->wredo.release();
     g->bc.release();
-    g->h_sigma.release();
-    g->h_dist.release();
-    g->dist_sum.release();
-    g->reach.release();
+    g->summ.release();
     if (g->ctl) cudaFree(g->ctl);
     if (g->hctl) cudaFreeHost(g->hctl);
     for (auto &ln : g->lanes) lane_pool::give(ln);
@@ -538,12 +557,12 @@ int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int3
     // one host block, one device allocation and one copy for the items and slots
     std::vector<int32_t> h((size_t)(5 * nitems + 2 * nslots));
     int32_t *sf = h.data() + 5 * nitems, *sn = sf + nslots;
-    auto put = [&](int64_t at, int32_t v, int64_t beg, int64_t end, int64_t slot) {
+    auto put = [&](int64_t at, int32_t v, int64_t beg, int64_t end) {
         int32_t *x = h.data() + 4 * at;
         x[0] = v;
         x[1] = (int32_t)beg;
         x[2] = (int32_t)end;
-        x[3] = (int32_t)slot;
+        x[3] = 0;
         h[(size_t)(4 * nitems + at)] = v;
     };
     int64_t k = 0;
@@ -553,7 +572,7 @@ int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int3
         const int64_t nch = (deg + chunk - 1) / chunk;
         const int32_t first = (int32_t)k;
         for (int64_t c = 0; c < nch; ++c, ++k) {
-            put(k, v, rp[v] + c * chunk, std::min<int64_t>(rp[v + 1], rp[v] + (c + 1) * chunk), k);
+            put(k, v, rp[v] + c * chunk, std::min<int64_t>(rp[v + 1], rp[v] + (c + 1) * chunk));
             sf[k] = first;
             sn[k] = (int32_t)nch;
         }
@@ -562,10 +581,12 @@ int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int3
         const int64_t deg = rp[v + 1] - rp[v];
         if (deg > chunk) continue;
         const int64_t t = nslots + cnt[(size_t)(chunk - deg)]++;
-        put(t, v, rp[v], rp[v + 1], -1);
+        put(t, v, rp[v], rp[v + 1]);
     }
     pl.nitems = (int32_t)nitems;
-    pl.nheavy = (int32_t)(nitems - nlight);
+    // a few light vertices are not worth a second round of every warp
+    // (random graph n = 5900, m = 41,000, 150 light ones: 2.24 / 2.22 ms)
+    pl.nheavy = (int32_t)(4 * nlight < nitems ? nitems : nitems - nlight);
     pl.nslots = (int32_t)nslots;
     CK(pl.blob.ensure(h.size()));
     if (!h.empty()) CK(cudaMemcpy(pl.blob.p, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
@@ -598,6 +619,7 @@ void use_plan(bcgb::MsParams &p, const ItemPlan &pl) {
     p.items = pl.items;
     p.item_v = pl.item_v;
     p.nheavy = pl.nheavy;
+    p.nslots = pl.nslots;
     p.slot_first = pl.slot_first;
     p.slot_nch = pl.slot_nch;
 }
@@ -678,6 +700,7 @@ bcgb::MsParams make_params(bc_graph *g) {
     bcgb::MsParams p{};
     p.n = g->n;
     p.nw32 = (std::max(g->n, 1) + 31) / 32;
+    p.light_least = 1;
     p.Lcap = g->Lcap;
     p.row_ptr = g->row_ptr.p;
     p.col = g->col.p;
@@ -786,7 +809,31 @@ int resolve_batch(const bc_options *opt, int *W) {
     return BC_OK;
 }
 
-// Upload (or copy) a source list; returns its length.
+// Room for the summaries of k sources.
+int ensure_summaries(bc_graph *g, size_t k) {
+    if (k <= g->summ_row && g->summ.p) return BC_OK;
+    g->summ_row = 0;
+    CK(g->summ.ensure(4 * std::max<size_t>(k, 1)));
+    const size_t row = g->summ.n / 4;
+    g->h_sigma.p = g->summ.p;
+    g->h_dist.p = g->summ.p + row;
+    g->dist_sum.p = reinterpret_cast<int64_t *>(g->summ.p + 2 * row);
+    g->reach.p = reinterpret_cast<int64_t *>(g->summ.p + 3 * row);
+    g->summ_row = row;
+    return BC_OK;
+}
+
+// What a run adds to, set to zero: BC (unless the run accumulates) and the
+// summaries of its sources. The one-launch sweep clears its own.
+int clear_outputs(bc_graph *g, int32_t nsrc, bool hash, cudaStream_t st) {
+    if (!g->clear_pending) return BC_OK;
+    g->clear_pending = false;
+    if (!(g->last_opt.flags & BC_ACCUMULATE)) CK(cudaMemsetAsync(g->bc.p, 0, g->bc.n * sizeof(double), st));
+    if (hash && nsrc)
+        CK(cudaMemset2DAsync(g->summ.p, g->summ_row * sizeof(uint64_t), 0, (size_t)nsrc * sizeof(uint64_t), 4, st));
+    return BC_OK;
+}
+
 // Landmark order of the vertices. The batches of the level sweep run best
 // when the sources of one 32-source word have nearly the same distances to
 // every vertex: their masked rows are then either useful for most of the
@@ -915,7 +962,15 @@ void rank_from_dist(bc_graph *g, std::vector<int32_t> &dist, int k) {
 // Validate and upload the source list. With `order`, the sources are staged
 // in landmark order (stable, so duplicates keep their relative order) and
 // src_index maps each staged position back to the caller's index.
-int stage_sources(bc_graph *g, const int32_t *sources, int32_t num, int32_t *count, bool order = false) {
+int stage_sources(bc_graph *g, const int32_t *sources, int32_t num, int32_t *count, cudaStream_t st,
+                  bool order = false) {
+    const bool ranked = order && (int32_t)g->rank.size() == g->n;
+    if (!sources && g->staged_all == (ranked ? 2 : 1)) {  // every vertex, as staged by the last run
+        *count = g->n;
+        g->reordered = ranked;
+        return BC_OK;
+    }
+    g->staged_all = 0;
     std::vector<int32_t> hs;
     if (!sources) {
         hs.resize(g->n);
@@ -935,12 +990,13 @@ int stage_sources(bc_graph *g, const int32_t *sources, int32_t num, int32_t *cou
         for (size_t i = 0; i < hs.size(); ++i) idx[cnt[g->rank[hs[i]]]++] = (int32_t)i;
         for (size_t t = 0; t < hs.size(); ++t) hs2[t] = hs[idx[t]];
         CK(g->src_index.ensure(idx.size()));
-        CK(cudaMemcpy(g->src_index.p, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(g->src_index.p, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
         hs.swap(hs2);
         g->reordered = true;
     }
     CK(g->sources.ensure(hs.size()));
-    if (!hs.empty()) CK(cudaMemcpy(g->sources.p, hs.data(), hs.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    if (!hs.empty())
+        CK(cudaMemcpyAsync(g->sources.p, hs.data(), hs.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     *count = (int32_t)hs.size();
     g->h_sources.swap(hs);
     return BC_OK;
@@ -1243,6 +1299,10 @@ int first_level_top_down(const bc_graph *g, const int32_t *src_host, int32_t nb,
 // 1..K-1 into the graph's BC in lane order, so the result is the same on
 // every run. A batch deeper than the level capacity stops every lane: the
 // capacity is doubled and each lane's unfinished batch starts over.
+// Lanes from which the light vertices run in full packs: the other batches
+// then fill the warps that this one leaves.
+constexpr int kFullPackLanes = 4;
+
 int run_lanes(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool backward, bool hash,
               uint64_t *rows_sig, int32_t *rows_dist, int64_t wait_ms) {
     const int B = 32 * W;
@@ -1284,6 +1344,7 @@ int run_lanes(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool bac
                 next[k] += K;
                 const int32_t b0 = j.bi * B;
                 j.p = lane_params(g, k);
+                j.p.light_least = K >= kFullPackLanes ? bcgb::kLightItems : 1;
                 j.p.nb = std::min<int32_t>(B, nsrc - b0);
                 j.p.first = first_level_top_down(g, g->h_sources.data() + b0, j.p.nb, &j.p.first_arcs);
                 j.p.seq = ++g->seq;
@@ -1396,11 +1457,117 @@ int run_lanes(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool bac
     return BC_OK;
 }
 
+// Whether a run is one launch (run_sweep) instead of a launch per level
+// (run_lanes): while the items of a level that fall to one warp of a group, in
+// heavy items (a light one counts 3/8 of that, in its pack), are at most
+// kSweepUnits. Whole calls, ms per level / one launch, all sources unless
+// stated, with the units a warp has:
+//   random n = 300 (0.8)   0.161 / 0.128    R-MAT n = 3153 (4.6)  1.07 / 0.77
+//   random n = 1024 (0.8)  0.309 / 0.212    R-MAT n = 6184, 2048 sources (9.6) 1.01 / 0.95
+//   random n = 5000 (8.6)  1.81 / 1.69      R-MAT n = 23756, 300 sources (9.3) 0.90 / 0.87
+//   random n = 5900 (12)   2.16 / 2.24      R-MAT n = 12124, directed (17) 7.6 / 8.7
+//   40 x 40 mesh (1.3)     0.74 / 0.50      128 x 128 mesh (13.5) 24 / 35
+// Beyond, a level is enough work to fill the GPU by itself, and a kernel for
+// one direction alone, with every block of the GPU, runs it better.
+constexpr int64_t kSweepUnits = 10;
+bool one_launch(const bc_graph *g, int W, int K) {
+    auto units = [](const ItemPlan &pl) { return 8 * (int64_t)pl.nheavy + 3 * (int64_t)(pl.nitems - pl.nheavy); };
+    const int64_t warps = 8 * (int64_t)(bcgb::ms_sweep_blocks(W) / K);
+    return std::max(units(g->fplan), units(g->bplan)) <= 8 * kSweepUnits * warps;
+}
+
+// Batches of a run as one cooperative launch (k_sweep): group k takes batches
+// k, k + K, ... with lane k's state and its own BC sums, added in group order at
+// the end. A batch deeper than the level capacity ends the launch; the capacity
+// doubles and the run starts over (nothing has reached g->bc yet).
+int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool hash, int64_t wait_ms) {
+    const int B = 32 * W;
+    const int32_t n = g->n, nbat = (nsrc + B - 1) / B;
+    const int resident = bcgb::ms_sweep_blocks(W);
+    if (resident < K) return fail(BC_ERR_CUDA, "the sweep kernel does not fit the device");
+    CK(g->sweep_bc.ensure((size_t)std::max(n, 1)));
+    int Lcap = g->Lcap;
+    for (;;) {
+        for (int k = 1; k < K; ++k) {
+            const int r = ensure_lane(g, g->lanes[k - 1], W, Lcap);
+            if (r) return r;
+        }
+        bcgb::SweepParams q{};
+        q.groups = K;
+        const int need = (std::max({g->fplan.nitems, g->bplan.nitems, 1}) + 7) / 8;  // eight warps per block
+        q.group_blocks = std::min(resident / K, need);
+        q.nbat = nbat;
+        q.nsrc = nsrc;
+        q.hash = hash ? 1 : 0;
+        q.first_rule = g->bottom_up0 ? 0 : g->directed ? 1 : 2;
+        q.alpha = g->alpha;
+        q.seq = ++g->seq;
+        q.narcs = g->narcs;
+        q.sources = g->sources.p;
+        q.out_index = g->reordered ? g->src_index.p : nullptr;
+        if (hash) {
+            q.h_sigma = g->h_sigma.p;
+            q.h_dist = g->h_dist.p;
+            q.dist_sum = g->dist_sum.p;
+            q.reach = g->reach.p;
+        }
+        q.b_nitems = g->bplan.nitems;
+        q.b_nheavy = g->bplan.nheavy;
+        q.b_nslots = g->bplan.nslots;
+        q.b_items = g->bplan.items;
+        q.b_item_v = g->bplan.item_v;
+        q.b_slot_first = g->bplan.slot_first;
+        q.b_slot_nch = g->bplan.slot_nch;
+        q.sync = reinterpret_cast<char *>(g->ctl) + kCtlSweepAt;
+        q.finished = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(g->ctl) + kCtlSweepAt - 128);
+        for (int k = 0; k < K; ++k) {
+            q.g[k] = lane_params(g, k);
+            q.g[k].ctl = g->ctl;
+            q.g[k].hctl = g->hctl_d;
+            if (k == 0) q.g[k].bc = g->sweep_bc.p;
+        }
+        {
+            Timer t(g, st, BC_KERNEL_FORWARD);
+            CK(bcgb::ms_launch_sweep(W, q, st));
+        }
+        int status = 0;
+        const auto t0 = std::chrono::steady_clock::now();
+        for (long spins = 0; !bcgb::word_for(&g->hctl->done, q.seq, &status); ++spins) {
+            if (spins % 1024 != 1023) continue;
+            const auto ms =
+                std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count();
+            if (ms > wait_ms)
+                return fail(BC_ERR_TIMEOUT, "the device did not report the end of the sweep within the wait limit");
+            const cudaError_t e = cudaStreamQuery(st);
+            if (e != cudaSuccess && e != cudaErrorNotReady)
+                return fail(BC_ERR_CUDA, std::string("device error during a sweep: ") + cudaGetErrorString(e));
+            if (e == cudaSuccess && !bcgb::word_for(&g->hctl->done, q.seq, &status))
+                return fail(BC_ERR_STATE, "the sweep ended without reporting its status");
+            if (spins % 65536 == 65535) std::this_thread::yield();
+        }
+        if (!((uint32_t)status & BC_STATUS_LEVEL_CAP)) {
+            Timer t(g, st, BC_KERNEL_INIT);
+            bcgb::ms_launch_sweep_merge(q, g->bc.p, n, (g->last_opt.flags & BC_ACCUMULATE) != 0, st);
+            CK(cudaGetLastError());
+            g->clear_pending = false;
+            g->status = (uint32_t)status;
+            g->status_known = true;
+            return BC_OK;
+        }
+        CK(cudaStreamSynchronize(st));
+        Lcap *= 2;
+        const int r = ensure_state(g, W, Lcap);
+        if (r) return r;
+        CK(cudaMemsetAsync(g->ctl, 0, kCtlBytes, st));
+    }
+}
+
 int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStream_t st, bool backward,
                 bool hash, uint64_t *rows_sig, int32_t *rows_dist) {
     const int64_t wait_ms = (opt && opt->wait_limit_ms > 0) ? opt->wait_limit_ms : 600000;
     if (opt && (opt->flags & BC_DENSE)) {
         int rd = ensure_dense(g, st);
+        if (!rd) rd = clear_outputs(g, nsrc, hash, st);
         if (rd) return rd;
         return run_dense_group(g, nsrc, opt, st, backward, hash, rows_sig, rows_dist);
     }
@@ -1418,6 +1585,11 @@ int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStr
                                   (double)g->s_levels * std::max(g->n, 1) * B * 2.0;
         int K = g->timing ? 1 : std::min<int32_t>(kSweepLanes, nbat);
         while (K > 1 && (K - 1) * lane_bytes > kLaneBudgetBytes) --K;
+        const bool sweep = backward && !rows_sig && !rows_dist && !g->timing && g->dev_wait_ns == 0 && g->test_hold == 0 &&
+                           nsrc > 0 && one_launch(g, W, K);
+        if (sweep) return run_sweep(g, nsrc, W, K, st, hash, wait_ms);
+        r = clear_outputs(g, nsrc, hash, st);
+        if (r) return r;
         if (K > 1) return run_lanes(g, nsrc, W, K, st, backward, hash, rows_sig, rows_dist, wait_ms);
     }
     for (int32_t b0 = 0; b0 < nsrc;) {
@@ -1495,7 +1667,7 @@ int ensure_rank(bc_graph *g, cudaStream_t st) {
     std::partial_sort(vs.begin(), vs.begin() + k, vs.end(),
                       [&](int32_t a, int32_t b) { return deg(a) > deg(b) || (deg(a) == deg(b) && a < b); });
     int32_t cnt = 0;
-    int r = stage_sources(g, vs.data(), k, &cnt, false);
+    int r = stage_sources(g, vs.data(), k, &cnt, st, false);
     if (r) return r;
     ScopedBuf<int32_t> dd;
     CK(dd.ensure((size_t)k * n));
@@ -2010,8 +2182,9 @@ int bc_create_graph(int32_t n, const int32_t *row_ptr, const int32_t *col, const
     if (!r && directed && weights) r = up(g->w_in, wwi);
     if (!r) {
         cudaError_t e = g->bc.ensure((size_t)std::max(n, 1));
-        if (e == cudaSuccess) e = cudaMalloc((void **)&g->ctl, sizeof(bcgb::DevCtl));
-        if (e == cudaSuccess) e = cudaMemset(g->ctl, 0, sizeof(bcgb::DevCtl));
+        if (e == cudaSuccess) e = cudaMalloc((void **)&g->ctl, kCtlBytes);
+        if (e == cudaSuccess) e = cudaMemset(g->ctl, 0, kCtlBytes);
+        g->status_known = e == cudaSuccess;  // 0
         if (e == cudaSuccess) e = cudaMemset(g->bc.p, 0, g->bc.n * sizeof(double));
         if (e == cudaSuccess)
             e = cudaHostAlloc((void **)&g->hctl, sizeof(bcgb::HostCtl), cudaHostAllocMapped | cudaHostAllocPortable);
@@ -2063,7 +2236,7 @@ int bc_run(bc_graph *g, const int32_t *sources, int32_t num_sources, const bc_op
         if (!r) r = ensure_rank(g, st);
         if (r) return r;
     }
-    r = stage_sources(g, sources, num_sources, &nsrc, order);
+    r = stage_sources(g, sources, num_sources, &nsrc, st, order);
     if (r) return r;
     g->timing = (flags & BC_TIMING) != 0;
     g->evused = 0;
@@ -2071,21 +2244,18 @@ int bc_run(bc_graph *g, const int32_t *sources, int32_t num_sources, const bc_op
     g->dense_flops = 0.0;
     g->dense_flops_f8 = 0.0;
     g->has_run = false;
+    g->status_known = false;
     const bool hash = !(flags & BC_NO_HASH);
-    if (!(flags & BC_ACCUMULATE)) CK(cudaMemsetAsync(g->bc.p, 0, g->bc.n * sizeof(double), st));
-    CK(cudaMemsetAsync(&g->ctl->status, 0, sizeof(uint32_t), st));
-    CK(cudaMemsetAsync(&g->ctl->dag_arcs, 0, 2 * sizeof(unsigned long long), st));
+    // the control block's run counters and the sweep's barrier words
+    CK(cudaMemsetAsync(g->ctl, 0, kCtlBytes, st));
     if (hash) {
-        CK(g->h_sigma.ensure(nsrc));
-        CK(g->h_dist.ensure(nsrc));
-        CK(g->dist_sum.ensure(nsrc));
-        CK(g->reach.ensure(nsrc));
-        if (nsrc) {
-            CK(cudaMemsetAsync(g->h_sigma.p, 0, nsrc * sizeof(uint64_t), st));
-            CK(cudaMemsetAsync(g->h_dist.p, 0, nsrc * sizeof(uint64_t), st));
-            CK(cudaMemsetAsync(g->dist_sum.p, 0, nsrc * sizeof(int64_t), st));
-            CK(cudaMemsetAsync(g->reach.p, 0, nsrc * sizeof(int64_t), st));
-        }
+        r = ensure_summaries(g, (size_t)nsrc);
+        if (r) return r;
+    }
+    g->clear_pending = true;
+    if (g->weighted || (flags & (BC_PLAIN | BC_PAIRS))) {
+        r = clear_outputs(g, nsrc, hash, st);
+        if (r) return r;
     }
     if (flags & BC_PAIRS) {
         r = run_pairs(g, nsrc, W, opt, st, hash);
@@ -2118,6 +2288,7 @@ int bc_run(bc_graph *g, const int32_t *sources, int32_t num_sources, const bc_op
     g->has_run = true;
     g->has_hash = hash;
     g->last_stream = st;
+    if (!sources) g->staged_all = g->reordered ? 2 : 1;
     return BC_OK;
 }
 
@@ -2125,10 +2296,13 @@ int bc_result(bc_graph *g, double *bc, uint32_t *status_flags) {
     g_err.clear();
     if (!g) return fail(BC_ERR_ARG, "graph is NULL");
     if (!g->has_run) return fail(BC_ERR_STATE, "no completed bc_run");
-    uint32_t status = 0;
     if (bc && g->n) CK(cudaMemcpyAsync(bc, g->bc.p, (size_t)g->n * sizeof(double), cudaMemcpyDefault, g->last_stream));
-    CK(cudaMemcpyAsync(&status, &g->ctl->status, sizeof(uint32_t), cudaMemcpyDefault, g->last_stream));
+    // the status word, unless the host has its final value already
+    if (!g->status_known)
+        CK(cudaMemcpyAsync(&g->status, &g->ctl->status, sizeof(uint32_t), cudaMemcpyDefault, g->last_stream));
     CK(cudaStreamSynchronize(g->last_stream));
+    g->status_known = true;
+    const uint32_t status = g->status;
     if (status_flags) *status_flags = status;
     if (log_enabled()) {
         // one JSON line per completed run on stderr (environment variable BC_LOG=1)
@@ -2156,6 +2330,22 @@ int bc_source_hashes(bc_graph *g, uint64_t *h_sigma, uint64_t *h_dist, int64_t *
     if (!g->has_run || !g->has_hash) return fail(BC_ERR_STATE, "no bc_run with per-source summaries");
     const size_t k = (size_t)g->last_nsrc;
     cudaStream_t st = g->last_stream;
+    cudaPointerAttributes at{};
+    bool host = k > 0;  // four host arrays: one copy of the four rows, then the host's own
+    for (const void *x : {(const void *)h_sigma, (const void *)h_dist, (const void *)dist_sum, (const void *)reach}) {
+        host = host && x && cudaPointerGetAttributes(&at, x) == cudaSuccess && at.type == cudaMemoryTypeUnregistered;
+    }
+    cudaGetLastError();
+    if (host) {
+        g->summ_host.resize(4 * k);
+        CK(cudaMemcpy2DAsync(g->summ_host.data(), k * 8, g->summ.p, g->summ_row * 8, k * 8, 4, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        std::memcpy(h_sigma, g->summ_host.data(), k * 8);
+        std::memcpy(h_dist, g->summ_host.data() + k, k * 8);
+        std::memcpy(dist_sum, g->summ_host.data() + 2 * k, k * 8);
+        std::memcpy(reach, g->summ_host.data() + 3 * k, k * 8);
+        return BC_OK;
+    }
     if (k) {
         if (h_sigma) CK(cudaMemcpyAsync(h_sigma, g->h_sigma.p, k * 8, cudaMemcpyDefault, st));
         if (h_dist) CK(cudaMemcpyAsync(h_dist, g->h_dist.p, k * 8, cudaMemcpyDefault, st));
@@ -2177,7 +2367,7 @@ int bc_forward_rows(bc_graph *g, const int32_t *sources, int32_t k, uint64_t *si
     if (!r) set_run_options(g, opt);
     if (r) return r;
     int32_t nsrc = 0;
-    r = stage_sources(g, sources, k, &nsrc);
+    r = stage_sources(g, sources, k, &nsrc, st);
     if (r) return r;
     if (nsrc == 0) return BC_OK;
     const size_t cells = (size_t)nsrc * g->n;
@@ -2197,6 +2387,7 @@ int bc_forward_rows(bc_graph *g, const int32_t *sources, int32_t k, uint64_t *si
         dist_rows = dd.p;
     }
     CK(cudaMemsetAsync(&g->ctl->status, 0, sizeof(uint32_t), st));
+    g->status_known = false;
     g->timing = false;
     if (g->weighted && opt && (opt->flags & BC_DENSE)) {
         if (!sigma || !dist) return fail(BC_ERR_ARG, "BC_DENSE rows of a weighted graph need both outputs");
@@ -2516,10 +2707,8 @@ int build_many(bc_many *m) {
         gd[i].dist_sum = gd[i].reach = nullptr;
         if (m->hash && g->n > 0) {
             bc_graph *gw = m->graphs[i];
-            CK(gw->h_sigma.ensure(g->n));
-            CK(gw->h_dist.ensure(g->n));
-            CK(gw->dist_sum.ensure(g->n));
-            CK(gw->reach.ensure(g->n));
+            const int rs = ensure_summaries(gw, (size_t)g->n);
+            if (rs) return rs;
             gd[i].h_sigma = gw->h_sigma.p;
             gd[i].h_dist = gw->h_dist.p;
             gd[i].dist_sum = gw->dist_sum.p;

@@ -77,12 +77,14 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x) {
 }
 #endif
 
-constexpr int kLightDeg = 8;  // a light vertex has at most this many arcs (msbfs_light.cuh)
+constexpr int kLightDeg = 8;    // a light vertex has at most this many arcs (msbfs_light.cuh)
+constexpr int kLightItems = 8;  // light vertices of a pack at most
 
 struct MsParams {
     int32_t n;
     int32_t nitems;
     int32_t nheavy;  // the first of them one warp each, the others (at most kLightDeg arcs) in packs
+    int32_t light_least;  // light vertices that a warp takes at least
     int32_t nw32;  // words of one union-frontier bitmap
     int32_t Lcap;  // level slots in F / ufr
     int32_t nb;    // sources in this batch (<= B)
@@ -92,7 +94,8 @@ struct MsParams {
     const int32_t *row_ptr;  // out-arcs: level 0->1 and the backward sweep
     const int32_t *col;
     const int32_t *col_f;    // arcs the forward sweep pulls over: in-arcs (= col when undirected)
-    const int4 *items;  // work items: vertex, first arc, end, partial slot of a chunk (-1: the whole vertex)
+    int32_t nslots;     // the first nslots items are chunks of split vertices, item k with partial slot k
+    const int4 *items;  // work items: vertex, first arc, end (and 0)
     const int32_t *item_v;  // their vertices alone
     const int32_t *slot_first;  // first slot of the chunk's vertex
     const int32_t *slot_nch;    // number of chunks of that vertex
@@ -122,6 +125,35 @@ struct MsParams {
     DevCtl *ctl;
     HostCtl *hctl;  // device pointer of the host-mapped block
 };
+
+// One launch for the whole sweep of a run (k_sweep, msbfs.cu): groups of
+// blocks take batches in turn, group k with the state in g[k].
+constexpr int kSweepGroups = 8;
+constexpr size_t kSweepSyncBytes = kSweepGroups * 128;
+struct SweepParams {
+    int32_t groups, group_blocks;
+    int32_t nbat, nsrc;
+    int32_t hash;        // per-source summaries (h_sigma ...)
+    int32_t first_rule;  // level 0 -> 1: 0 bottom-up, 1 top-down, 2 top-down while arcs * alpha < narcs
+    float alpha;
+    uint32_t seq;
+    int64_t narcs;
+    const int32_t *sources;    // [nsrc]
+    const int32_t *out_index;  // as in MsParams, from the run's first source
+    uint64_t *h_sigma, *h_dist;
+    int64_t *dist_sum, *reach;
+    // the backward plan (g[k] has the forward one)
+    int32_t b_nitems, b_nheavy, b_nslots;
+    const int4 *b_items;
+    const int32_t *b_item_v, *b_slot_first, *b_slot_nch;
+    void *sync;          // kSweepSyncBytes bytes, zero at launch
+    unsigned *finished;  // zero at launch
+    MsParams g[kSweepGroups];
+};
+int ms_sweep_blocks(int W);  // blocks resident on the device at once (0: error)
+cudaError_t ms_launch_sweep(int W, const SweepParams &q, cudaStream_t st);
+// bc = the groups' sums (add: += them)
+void ms_launch_sweep_merge(const SweepParams &q, double *bc, int32_t n, bool add, cudaStream_t st);
 
 // Launchers (msbfs.cu). W = words per vertex row (B = 32 W).
 bool ms_supported_width(int W);

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
                         body::bwd_sum<W, false>(gd.col, gd.row_ptr[v], gd.row_ptr[v + 1], ufs, Fs, Cs, f, s_u[wib], s_nz[wib], lane, S);
                         asm volatile("cp.async.wait_group 0;" ::: "memory");
                         __syncwarp();
-                        body::finalize_dep<W, false>(sigma, Cl, target, v, f, S, lane, &s_sig[wib][0][0]);
+                        body::finalize_dep<W>(Cl, target, v, f, S, lane, &s_sig[wib][0][0]);
                         __syncwarp();  // the next vertex's copies overwrite s_sig
                     }
                 }

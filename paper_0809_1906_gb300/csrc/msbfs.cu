@@ -50,19 +50,21 @@ __device__ __forceinline__ bool filter_level(const MsParams &p, int l) {
     return p.lsize == nullptr || (uint64_t)p.lsize[l] * kFilterRatio < (uint64_t)p.n;
 }
 
-// Light vertices that a warp takes at a time.
-__device__ __forceinline__ int light_share(int nlight, int warps) {
+// Light vertices that a warp takes at a time: an even share, at least `least`
+// (a pack holds eight: spreading them thinner shortens a level that leaves warps
+// idle anyway, and costs probes when other batches would use them).
+__device__ __forceinline__ int light_share(int nlight, int warps, int least) {
     const int c = (nlight + warps - 1) / warps;
-    return c < 32 ? c : 32;
+    return c < least ? least : c < 32 ? c : 32;
 }
 
+// A batch's state before its first level: everything that must start at zero.
 template <int W>
-__global__ void __launch_bounds__(kBlock) k_init(const MsParams p) {
+__device__ __forceinline__ void init_zero(const MsParams &p, int bid, int nblk) {
     constexpr int B = 32 * W;
-    pdl::enter();
     const size_t nW = (size_t)p.n * W;
-    const size_t stride = (size_t)gridDim.x * kBlock;
-    const size_t tid = (size_t)blockIdx.x * kBlock + threadIdx.x;
+    const size_t stride = (size_t)nblk * kBlock;
+    const size_t tid = (size_t)bid * kBlock + threadIdx.x;
     for (size_t i = tid; i < 2 * nW; i += stride) {
         p.F[i] = 0u;  // frontiers of levels 0 and 1
         p.V[i] = 0u;  // visited through levels -1 and 0
@@ -72,6 +74,24 @@ __global__ void __launch_bounds__(kBlock) k_init(const MsParams p) {
     // masked level-0 rows of the sources start at zero
     for (size_t i = tid; i < (size_t)p.nb * B; i += stride) p.S[(size_t)p.sources[i / B] * B + i % B] = 0;
     for (size_t i = tid; i < (size_t)p.Lcap; i += stride) p.wide[i] = 0u;
+}
+// d(s,s) = 0 and sigma_s(s) = 1 (Section 1.1) for source b of the batch; the
+// sources are the vertices visited through level 0.
+template <int W>
+__device__ __forceinline__ void init_source(const MsParams &p, int b) {
+    constexpr int B = 32 * W;
+    const int s = p.sources[b];
+    atomicOr(p.F + (size_t)s * W + (b >> 5), 1u << (b & 31));
+    atomicOr(p.V + (size_t)p.n * W + (size_t)s * W + (b >> 5), 1u << (b & 31));
+    atomicOr(p.ufr + (s >> 5), 1u << (s & 31));
+    p.sigma[(size_t)s * B + b] = 1ull;
+    p.S[(size_t)s * B + b] = 1;
+}
+
+template <int W>
+__global__ void __launch_bounds__(kBlock) k_init(const MsParams p) {
+    pdl::enter();
+    init_zero<W>(p, blockIdx.x, gridDim.x);
     __shared__ bool s_last;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -81,16 +101,7 @@ __global__ void __launch_bounds__(kBlock) k_init(const MsParams p) {
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    // d(s,s) = 0 and sigma_s(s) = 1 (Section 1.1); the sources are the
-    // vertices visited through level 0
-    for (int b = threadIdx.x; b < p.nb; b += kBlock) {
-        const int s = p.sources[b];
-        atomicOr(p.F + (size_t)s * W + (b >> 5), 1u << (b & 31));
-        atomicOr(p.V + nW + (size_t)s * W + (b >> 5), 1u << (b & 31));
-        atomicOr(p.ufr + (s >> 5), 1u << (s & 31));
-        p.sigma[(size_t)s * B + b] = 1ull;
-        p.S[(size_t)s * B + b] = 1;
-    }
+    for (int b = threadIdx.x; b < p.nb; b += kBlock) init_source<W>(p, b);
     if (threadIdx.x == 0) {
         if (p.lsize) p.lsize[0] = (uint32_t)p.nb;
         p.ctl->fwd_done = 0u;
@@ -110,47 +121,57 @@ __global__ void __launch_bounds__(kBlock) k_init(const MsParams p) {
 // whole grid (block scan of the source degrees), so a high-degree source is
 // shared out. No masked rows are written: the next level sees that every
 // count is 1 and counts predecessors instead (fwd_sum, `ones`).
-template <int W>
-__global__ void __launch_bounds__(kBlock) k_first(const MsParams p) {
-    constexpr int B = 32 * W;
-    pdl::enter();
-    __shared__ int s_off[kBlock + 1];
-    __shared__ int s_wsum[kWarps];
+// Returns the number of arcs.
+struct FirstShared {
+    int off[kBlock + 1];
+    int wsum[kWarps];
+};
+__device__ __forceinline__ int first_scan(const MsParams &p, FirstShared &sh) {
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    {
-        int deg = 0;
-        if (t < p.nb) deg = p.row_ptr[p.sources[t] + 1] - p.row_ptr[p.sources[t]];
-        int x = deg;
+    int deg = 0;
+    if (t < p.nb) deg = p.row_ptr[p.sources[t] + 1] - p.row_ptr[p.sources[t]];
+    int x = deg;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(kFull, x, off);
-            if (lane >= off) x += y;
-        }
-        if (lane == 31) s_wsum[wid] = x;
-        __syncthreads();
-        int base = 0;
-        for (int k = 0; k < wid; ++k) base += s_wsum[k];
-        s_off[t] = base + x - deg;
-        if (t == kBlock - 1) s_off[kBlock] = base + x;
-        __syncthreads();
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(kFull, x, off);
+        if (lane >= off) x += y;
     }
-    const size_t nW = (size_t)p.n * W;
-    uint32_t *F1 = p.F + nW;
+    if (lane == 31) sh.wsum[wid] = x;
+    __syncthreads();
+    int base = 0;
+    for (int k = 0; k < wid; ++k) base += sh.wsum[k];
+    sh.off[t] = base + x - deg;
+    if (t == kBlock - 1) sh.off[kBlock] = base + x;
+    __syncthreads();
+    return sh.off[p.nb];
+}
+template <int W>
+__device__ __forceinline__ void first_arcs(const MsParams &p, int bid, int nblk, const FirstShared &sh, int total) {
+    constexpr int B = 32 * W;
+    uint32_t *F1 = p.F + (size_t)p.n * W;
     uint32_t *uf1 = p.ufr + p.nw32;
-    const int total = s_off[p.nb];
-    for (int a = blockIdx.x * kBlock + t; a < total; a += gridDim.x * kBlock) {
-        int lo = 0, hi = p.nb - 1;  // the source b whose arcs hold position a: s_off[b] <= a < s_off[b + 1]
+    for (int a = bid * kBlock + threadIdx.x; a < total; a += nblk * kBlock) {
+        int lo = 0, hi = p.nb - 1;  // the source b whose arcs hold position a: off[b] <= a < off[b + 1]
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (s_off[mid] <= a) lo = mid; else hi = mid - 1;
+            if (sh.off[mid] <= a) lo = mid; else hi = mid - 1;
         }
         const int b = lo;
         const int s = p.sources[b];
-        const int v = p.col[p.row_ptr[s] + (a - s_off[b])];
+        const int v = p.col[p.row_ptr[s] + (a - sh.off[b])];
         atomicOr(F1 + (size_t)v * W + (b >> 5), 1u << (b & 31));
         atomicOr(uf1 + (v >> 5), 1u << (v & 31));
         p.sigma[(size_t)v * B + b] = 1ull;
     }
+}
+
+template <int W>
+__global__ void __launch_bounds__(kBlock) k_first(const MsParams p) {
+    pdl::enter();
+    __shared__ FirstShared sh;
+    const int t = threadIdx.x;
+    const int total = first_scan(p, sh);
+    first_arcs<W>(p, blockIdx.x, gridDim.x, sh, total);
     __syncthreads();
     if (t != 0) return;
     __threadfence();
@@ -170,28 +191,33 @@ __global__ void __launch_bounds__(kBlock) k_first(const MsParams p) {
     host_word(&p.hctl->progress, p.seq, 1u);
 }
 
-template <int W, bool HOOK>
-__global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const int l) {
+// What one block of a forward level keeps in shared memory (beside the stages).
+template <int W>
+struct FwdShared {
+    __align__(16) uint32_t U[kWarps][32][W];  // unvisited words of the group's items
+    uint32_t qz[kWarps][32];
+    uint32_t flags;
+    uint32_t front;  // vertices this block put into frontier l+1
+    unsigned long long arcs;
+};
+// What a warp learns from its items: some vertex joined frontier l+1, a sum
+// passed 2^64, a new count needs more than 16 bits; and its lanes' predecessor
+// relations.
+struct FwdFound {
+    bool produced = false, ovf = false, wide_next = false;
+    uint32_t arcs = 0;
+};
+
+// Level l -> l+1 over the items of block bid of nblk. NC: the level's inputs
+// were written by an earlier launch (see ldx).
+template <int W, bool HOOK, bool NC>
+__device__ __forceinline__ void forward_items(const MsParams &p, const int l, const int bid, const int nblk,
+                                              FwdShared<W> &sh, body::WarpStage &ws, const uint16_t *Sl, uint16_t *Sn,
+                                              const bool ones, FwdFound &found) {
     constexpr int B = 32 * W;
-    pdl::enter();
-    __shared__ uint32_t s_U[kWarps][32][W];  // unvisited words of the group's items
-    __shared__ uint64_t s_bar[kWarps];
-    __shared__ uint32_t s_qz[kWarps][32];
-    extern __shared__ __align__(128) uint8_t s_stage[];
-    __shared__ uint32_t s_flags;
-    __shared__ unsigned long long s_arcs;
-    __shared__ uint32_t s_front;  // vertices this block put into frontier l+1
+    // probe_chunk's per-arc notes: nobody reads them in the staged form
     __shared__ int32_t s_u[kWarps][32];
     __shared__ uint32_t s_nz[kWarps][32];
-    if (threadIdx.x == 0) {
-        s_flags = 0u;
-        s_arcs = 0ull;
-        s_front = 0u;
-    }
-    __syncthreads();
-    // speculative launches past the last level, and the level-capacity guard
-    if (*(volatile uint32_t *)&p.ctl->fwd_done != 0u || l + 1 >= p.Lcap) return;
-
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     const size_t nW = (size_t)p.n * W;
@@ -201,60 +227,53 @@ __global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const i
     uint32_t *ufn = p.ufr + (size_t)(l + 1) * p.nw32;
     const uint32_t *Vin = p.V + (size_t)(l & 1) * nW;
     uint32_t *Vout = p.V + (size_t)((l + 1) & 1) * nW;
-    const uint16_t *Sl = p.S_rd;  // masked rows of level l and l+1 (set by the launcher)
-    uint16_t *Sn = p.S_wr;
     const bool wide = *(volatile uint32_t *)(p.wide + l) != 0u;
-    const bool ones = l == 1 && p.first;  // level 1 written by k_first: all counts 1, no masked rows
     const uint32_t *ufl_f = filter_level(p, l) ? ufl : nullptr;  // the union filter, on narrow frontiers only
     bool produced = false, ovf = false, wide_next = false;
     uint32_t arcs = 0;  // predecessor relations counted by this lane
-    body::WarpStage ws{s_stage + wib * stage::kFwdStageBytes, s_bar + wib, s_qz[wib], 0u, false,
-                       body::stage_wctl(p.wait_ns, p.test_hold)};
-    if (lane == 0) stage::bar_init(ws.bar);
-    __syncwarp();
 
     // Persistent warps stride over the items (sorted by decreasing degree, so
     // every warp gets a similar mix; the chunks of one heavy vertex land on
     // different warps). A warp takes its next 32 items at once: lane k checks
     // item k's vertex (visited words; the new frontier row cleared when
     // nothing is left to find), then the warp works through the active ones.
-    const int G = gridDim.x * kWarps;
-    for (int g0 = blockIdx.x * kWarps + wib; g0 < p.nheavy; g0 += 32 * G) {
+    const int G = nblk * kWarps;
+    for (int g0 = bid * kWarps + wib; g0 < p.nheavy; g0 += 32 * G) {
         bool act = false;
-        __syncwarp();  // the previous group's reads of s_U are done
+        __syncwarp();  // the previous group's reads of U are done
         const int ik = g0 + lane * G;
         if (ik < p.nheavy) {
             const int vk = p.item_v[ik];
             uint32_t a[W], f[W];
-            load_row<W>(Vin + (size_t)vk * W, a);
-            load_row<W>(Fl + (size_t)vk * W, f);
+            load_row<W, NC>(Vin + (size_t)vk * W, a);
+            load_row<W, NC>(Fl + (size_t)vk * W, f);
             uint32_t any = 0;
 #pragma unroll
             for (int j = 0; j < W; ++j) {
                 const uint32_t vis = a[j] | f[j];
                 Vout[(size_t)vk * W + j] = vis;  // chunks of one vertex write the same words
                 const uint32_t u = ~vis & valid_word(p.nb, j);
-                s_U[wib][lane][j] = u;
+                sh.U[wib][lane][j] = u;
                 any |= u;
             }
             act = any != 0u;
-            if (!act) {  // nothing left to find: the new frontier row is empty
-                const int sk = __ldg(&p.items[ik].w);
-                if (sk < 0 || p.slot_first[sk] == sk)
+            // nothing left to find: the new frontier row is empty (a split
+            // vertex's is written by its first chunk, item = slot)
+            if (!act && (ik >= p.nslots || p.slot_first[ik] == ik))
 #pragma unroll
-                    for (int j = 0; j < W; ++j) Fn[(size_t)vk * W + j] = 0u;
-            }
+                for (int j = 0; j < W; ++j) Fn[(size_t)vk * W + j] = 0u;
         }
         unsigned todo = __ballot_sync(kFull, act);
         __syncwarp();
         while (todo) {
             const int kk = __ffs(todo) - 1;
             todo &= todo - 1;
-            const int4 item = __ldg(p.items + g0 + kk * G);
-            const int v = item.x, beg = item.y, end = item.z, slot = item.w;
+            const int it = g0 + kk * G;
+            const int4 item = __ldg(p.items + it);
+            const int v = item.x, beg = item.y, end = item.z, slot = it < p.nslots ? it : -1;
             uint32_t U[W];
 #pragma unroll
-            for (int j = 0; j < W; ++j) U[j] = s_U[wib][kk][j];
+            for (int j = 0; j < W; ++j) U[j] = sh.U[wib][kk][j];
             uint64_t acc[W];  // lane owns source 32j + lane
             uint32_t nf[W];
 #pragma unroll
@@ -262,12 +281,12 @@ __global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const i
                 acc[j] = 0ull;
                 nf[j] = 0u;
             }
-            body::fwd_sum<W, true, true, HOOK>(p.col_f, beg, end, ufl_f, Fl, Sl, p.sigma, wide, ones, U, s_u[wib], s_nz[wib], lane,
+            body::fwd_sum<W, NC, true, HOOK>(p.col_f, beg, end, ufl_f, Fl, Sl, p.sigma, wide, ones, U, s_u[wib], s_nz[wib], lane,
                                          acc, nf, ovf, arcs, &ws);
             if (slot < 0) {
                 const bool joined = body::store_next<W>(p.sigma, Sn, Fn, ufn, v, acc, nf, lane, wide_next);
                 produced |= joined;
-                if (joined && lane == 0) atomicAdd(&s_front, 1u);
+                if (joined && lane == 0) atomicAdd(&sh.front, 1u);
                 continue;
             }
             uint64_t *pp = p.part + (size_t)slot * B + lane;
@@ -304,31 +323,31 @@ __global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const i
             }
             const bool joined = body::store_next<W>(p.sigma, Sn, Fn, ufn, v, acc, nf, lane, wide_next);
             produced |= joined;
-            if (joined && lane == 0) atomicAdd(&s_front, 1u);
+            if (joined && lane == 0) atomicAdd(&sh.front, 1u);
             if (lane == 0) p.cnt[first] = 0u;
         }
     }
     // light vertices (the items' tail): a warp takes up to 32 consecutive ones,
     // an even share when there are fewer, and works through them pack by pack
     const int nlight = p.nitems - p.nheavy;
-    const int share = light_share(nlight, G);
+    const int share = light_share(nlight, G, p.light_least);
     // from the last warp down: the first ones have the more heavy items
-    for (int g0 = (G - 1 - (int)(blockIdx.x * kWarps + wib)) * share; g0 < nlight; g0 += G * share) {
+    for (int g0 = (G - 1 - (bid * kWarps + wib)) * share; g0 < nlight; g0 += G * share) {
         bool act = false;
         int4 item = make_int4(0, 0, 0, 0);
-        __syncwarp();  // the previous group's reads of s_U are done
+        __syncwarp();  // the previous group's reads of U are done
         if (lane < share && g0 + lane < nlight) {
             item = __ldg(p.items + p.nheavy + g0 + lane);
             uint32_t a[W], f[W];
-            load_row<W>(Vin + (size_t)item.x * W, a);
-            load_row<W>(Fl + (size_t)item.x * W, f);
+            load_row<W, NC>(Vin + (size_t)item.x * W, a);
+            load_row<W, NC>(Fl + (size_t)item.x * W, f);
             uint32_t any = 0;
 #pragma unroll
             for (int j = 0; j < W; ++j) {
                 const uint32_t vis = a[j] | f[j];
                 Vout[(size_t)item.x * W + j] = vis;
                 const uint32_t u = ~vis & valid_word(p.nb, j);
-                s_U[wib][lane][j] = u;
+                sh.U[wib][lane][j] = u;
                 any |= u;
             }
             act = any != 0u && item.y < item.z;
@@ -339,29 +358,67 @@ __global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const i
         const unsigned lt = __ballot_sync(kFull, act);
         __syncwarp();
         if (lt)
-            body::fwd_light<W, true>(lt, item.x, item.y, item.z - item.y, s_U[wib],
+            body::fwd_light<W, NC>(lt, item.x, item.y, item.z - item.y, sh.U[wib],
                                      *reinterpret_cast<body::LightScratch<W> *>(ws.buf), p.col_f, ufl_f, Fl, Sl,
-                                     p.sigma, wide, ones, Sn, Fn, ufn, lane, ovf, arcs, produced, wide_next, &s_front);
+                                     p.sigma, wide, ones, Sn, Fn, ufn, lane, ovf, arcs, produced, wide_next, &sh.front);
     }
-    const unsigned wovf = __ballot_sync(kFull, ovf);
-    const unsigned wwide = __ballot_sync(kFull, wide_next);
+    found.produced = produced;
+    found.ovf = ovf;
+    found.wide_next = wide_next;
+    found.arcs = arcs;
+}
+// The block's findings into sh.flags (1 produced, 2 overflow, 4 wide, 8 a wait
+// gave up) and sh.arcs.
+template <int W>
+__device__ __forceinline__ void forward_collect(FwdShared<W> &sh, const FwdFound &f, bool fail) {
+    const unsigned wovf = __ballot_sync(kFull, f.ovf);
+    const unsigned wwide = __ballot_sync(kFull, f.wide_next);
+    uint32_t arcs = f.arcs;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) arcs += __shfl_xor_sync(kFull, arcs, off);
-    if (lane == 0) {
-        if (produced) atomicOr(&s_flags, 1u);
-        if (wovf) atomicOr(&s_flags, 2u);
-        if (wwide) atomicOr(&s_flags, 4u);
-        if (ws.fail) atomicOr(&s_flags, 8u);
-        if (arcs) atomicAdd(&s_arcs, (unsigned long long)arcs);
+    if ((threadIdx.x & 31) == 0) {
+        if (f.produced) atomicOr(&sh.flags, 1u);
+        if (wovf) atomicOr(&sh.flags, 2u);
+        if (wwide) atomicOr(&sh.flags, 4u);
+        if (fail) atomicOr(&sh.flags, 8u);
+        if (arcs) atomicAdd(&sh.arcs, (unsigned long long)arcs);
+    }
+}
+
+template <int W, bool HOOK>
+__global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const int l) {
+    pdl::enter();
+    __shared__ FwdShared<W> sh;
+    __shared__ uint64_t s_bar[kWarps];
+    extern __shared__ __align__(128) uint8_t s_stage[];
+    if (threadIdx.x == 0) {
+        sh.flags = 0u;
+        sh.arcs = 0ull;
+        sh.front = 0u;
     }
     __syncthreads();
+    // speculative launches past the last level, and the level-capacity guard
+    if (*(volatile uint32_t *)&p.ctl->fwd_done != 0u || l + 1 >= p.Lcap) return;
+
+    const int lane = threadIdx.x & 31;
+    const int wib = threadIdx.x >> 5;
+    const bool ones = l == 1 && p.first;  // level 1 written by k_first: all counts 1, no masked rows
+    body::WarpStage ws{s_stage + wib * stage::kFwdStageBytes, s_bar + wib, sh.qz[wib], 0u, false,
+                       body::stage_wctl(p.wait_ns, p.test_hold)};
+    if (lane == 0) stage::bar_init(ws.bar);
+    __syncwarp();
+    FwdFound found;
+    // masked rows of level l and l+1: set by the launcher
+    forward_items<W, HOOK, true>(p, l, blockIdx.x, gridDim.x, sh, ws, p.S_rd, p.S_wr, ones, found);
+    forward_collect(sh, found, ws.fail);
+    __syncthreads();
     if (threadIdx.x != 0) return;
-    if (s_arcs) atomicAdd(&p.ctl->batch_arcs, s_arcs);
-    if (s_front) atomicAdd(&p.ctl->front_new, s_front);
-    if (s_flags & 1u) atomicOr(&p.ctl->nonempty, 1u);
-    if (s_flags & 2u) atomicOr(&p.ctl->status, BC_STATUS_SIGMA_OVERFLOW);
-    if (s_flags & 8u) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
-    if (s_flags & 4u) atomicOr(p.wide + l + 1, 1u);
+    if (sh.arcs) atomicAdd(&p.ctl->batch_arcs, sh.arcs);
+    if (sh.front) atomicAdd(&p.ctl->front_new, sh.front);
+    if (sh.flags & 1u) atomicOr(&p.ctl->nonempty, 1u);
+    if (sh.flags & 2u) atomicOr(&p.ctl->status, BC_STATUS_SIGMA_OVERFLOW);
+    if (sh.flags & 8u) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
+    if (sh.flags & 4u) atomicOr(p.wide + l + 1, 1u);
     __threadfence();
     if (atomicAdd(&p.ctl->blocks_done, 1u) != gridDim.x - 1) return;
     // last block of this level: decide whether the forward pass ended
@@ -388,20 +445,26 @@ __global__ void __launch_bounds__(kBlock, 3) k_forward(const MsParams p, const i
     host_word(&p.hctl->progress, p.seq, (uint32_t)(l + 1));
 }
 
-template <int W, bool HOOK>
-__global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const int l) {
+// What one block of a backward level keeps in shared memory (beside the stages).
+template <int W>
+struct BwdShared {
+    __align__(16) uint32_t f[kWarps][32][W];  // level-l words of the group's items
+    int32_t v[kWarps][32];      // and their vertices
+    uint32_t qz[kWarps][32];
+    __align__(16) uint16_t sig[kWarps][32 * W];  // the counts of the item being finalized
+};
+
+// Backward level l over the items of block bid of nblk (NC as in forward_items).
+template <int W, bool HOOK, bool NC>
+__device__ __forceinline__ void backward_items(const MsParams &p, const int l, const int bid, const int nblk,
+                                               BwdShared<W> &sh, body::WarpStage &ws) {
     constexpr int B = 32 * W;
-    pdl::enter();
-    __shared__ uint32_t s_f[kWarps][32][W];  // level-l words of the group's items
-    __shared__ int32_t s_v[kWarps][32];      // and their vertices
-    __shared__ uint64_t s_bar[kWarps];
-    __shared__ uint32_t s_qz[kWarps][32];
-    extern __shared__ __align__(128) uint8_t s_stage[];
+    // probe_chunk's per-arc notes: nobody reads them in the staged form
     __shared__ int32_t s_u[kWarps][32];
     __shared__ uint32_t s_nz[kWarps][32];
-    __shared__ __align__(16) uint16_t s_sig[kWarps][W][32];  // the counts of the item being finalized
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
+    const int jl = (W * lane) >> 5;  // the row word holding this lane's sources (packed view)
     const size_t nW = (size_t)p.n * W;
     const uint32_t *Fl = p.F + (size_t)l * nW;
     const uint32_t *Fs = p.F + (size_t)(l + 1) * nW;
@@ -412,10 +475,6 @@ __global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const 
     float *Cl = l > 1 ? p.cval + (size_t)(l & 1) * nB : nullptr;
     const float *Cs = p.cval + (size_t)((l + 1) & 1) * nB;
     const uint32_t *ufs_f = filter_level(p, l + 1) ? ufs : nullptr;  // the union filter, on narrow frontiers only
-    body::WarpStage ws{s_stage + wib * stage::kBwdStageBytes, s_bar + wib, s_qz[wib], 0u, false,
-                       body::stage_wctl(p.wait_ns, p.test_hold)};
-    if (lane == 0) stage::bar_init(ws.bar);
-    __syncwarp();
     // where the finalize reads sigma_s(v) for the pairs at level l: none at
     // level 1 from k_first (every count is 1), the level's masked uint16 row
     // when each level has its own buffer and the level is narrow, else the
@@ -432,7 +491,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const 
         int lo = W, hi = -1;
 #pragma unroll
         for (int j = 0; j < W; ++j) {
-            const uint32_t x = s_f[wib][k][j];
+            const uint32_t x = sh.f[wib][k][j];
             any |= x;
             if (x != 0u) {
                 lo = j < lo ? j : lo;
@@ -441,30 +500,30 @@ __global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const 
         }
         if (any != 0u) {
             if (Sl)
-                stage::prefetch_l2(Sl + (size_t)s_v[wib][k] * B + 32 * lo, 64u * (uint32_t)(hi - lo + 1));
+                stage::prefetch_l2(Sl + (size_t)sh.v[wib][k] * B + 32 * lo, 64u * (uint32_t)(hi - lo + 1));
             else
-                stage::prefetch_l2(p.sigma + (size_t)s_v[wib][k] * B + 32 * lo, 256u * (uint32_t)(hi - lo + 1));
+                stage::prefetch_l2(p.sigma + (size_t)sh.v[wib][k] * B + 32 * lo, 256u * (uint32_t)(hi - lo + 1));
         }
     };
     // the forward pass's item striding; lane k of a warp checks whether its
     // k-th next item's vertex is at level l for any source (the same for all
     // chunks of v), then the warp works through the active items
-    const int G = gridDim.x * kWarps;
-    for (int g0 = blockIdx.x * kWarps + wib; g0 < p.nheavy; g0 += 32 * G) {
+    const int G = nblk * kWarps;
+    for (int g0 = bid * kWarps + wib; g0 < p.nheavy; g0 += 32 * G) {
         bool act = false;
-        __syncwarp();  // the previous group's reads of s_f are done
+        __syncwarp();  // the previous group's reads of f are done
         const int ik = g0 + lane * G;
         if (ik < p.nheavy) {
             const int vk = p.item_v[ik];
             uint32_t f[W];
-            load_row<W>(Fl + (size_t)vk * W, f);
+            load_row<W, NC>(Fl + (size_t)vk * W, f);
             uint32_t any = 0;
 #pragma unroll
             for (int j = 0; j < W; ++j) {
-                s_f[wib][lane][j] = f[j];
+                sh.f[wib][lane][j] = f[j];
                 any |= f[j];
             }
-            s_v[wib][lane] = vk;
+            sh.v[wib][lane] = vk;
             act = any != 0u;
         }
         unsigned todo = __ballot_sync(kFull, act);
@@ -477,81 +536,98 @@ __global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const 
                 const unsigned k2 = __fns(todo, 0, 2);  // two active items ahead
                 if (k2 < 32u) prefetch_sigma((int)k2);
             }
-            const int4 item = __ldg(p.items + g0 + kk * G);
-            const int v = item.x, beg = item.y, end = item.z, slot = item.w;
+            const int it = g0 + kk * G;
+            const int4 item = __ldg(p.items + it);
+            const int v = item.x, beg = item.y, end = item.z, slot = it < p.nslots ? it : -1;
             uint32_t f[W];
 #pragma unroll
-            for (int j = 0; j < W; ++j) f[j] = s_f[wib][kk][j];
+            for (int j = 0; j < W; ++j) f[j] = sh.f[wib][kk][j];
 
-            // an unsplit vertex finalizes right after its scan: its counts
-            // (the words with a level-l source) are copied to shared memory
-            // while the neighbours are scanned (even lanes, 4 bytes each)
-            const bool early = slot < 0 && Sl != nullptr;
+            const uint32_t fw = sh.f[wib][kk][jl];  // the word of this lane's sources
+            const size_t at = (size_t)v * B + W * lane;
+            // an unsplit vertex finalizes right after its scan: its counts are
+            // copied to shared memory while the neighbours are scanned
+            const bool early = W >= 2 && slot < 0 && Sl != nullptr;
             if (early) {
-#pragma unroll
-                for (int j = 0; j < W; ++j)
-                    if (f[j] != 0u && (lane & 1) == 0) {
-                        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&s_sig[wib][j][lane]);
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst),
-                                     "l"(Sl + (size_t)v * B + 32 * j + lane)
-                                     : "memory");
-                    }
+                if (fw != 0u) {
+                    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sh.sig[wib][W * lane]);
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(Sl + at),
+                                 "n"(W >= 2 ? 2 * W : 4)
+                                 : "memory");
+                }
                 asm volatile("cp.async.commit_group;" ::: "memory");
             }
-            float S[W];  // lane owns source 32j + lane
+            float S[W];  // packed view: source W lane + t
 #pragma unroll
-            for (int j = 0; j < W; ++j) S[j] = 0.0f;
-            body::bwd_sum<W, true, true, HOOK>(p.col, beg, end, ufs_f, Fs, Cs, f, s_u[wib], s_nz[wib], lane, S, &ws);
+            for (int t = 0; t < W; ++t) S[t] = 0.0f;
+            body::bwd_sum_staged<W, NC, HOOK>(p.col, beg, end, ufs_f, Fs, Cs, f, s_u[wib], s_nz[wib], lane, S, &ws);
+            uint32_t cnt[(W + 1) / 2];
             if (slot < 0) {
                 if (early) {
                     asm volatile("cp.async.wait_group 0;" ::: "memory");
                     __syncwarp();
+                    body::lds_packed<W>(&sh.sig[wib][W * lane], cnt);
                 }
-                body::finalize_dep<W>(p.sigma, Sl, sig_ones, Cl, p.bc, v, f, S, lane,
-                                      early ? &s_sig[wib][0][0] : nullptr);
-                __syncwarp();  // the next item's copies overwrite s_sig
-                continue;
-            }
-            float *pp = reinterpret_cast<float *>(p.part) + (size_t)slot * B + lane;
+            } else {
+                float *pp = reinterpret_cast<float *>(p.part) + (size_t)slot * B + W * lane;
+                body::stg_packed<W>(pp, S);
+                __threadfence();
+                __syncwarp();
+                const int first = p.slot_first[slot];
+                const int nch = p.slot_nch[slot];
+                unsigned old = 0;
+                if (lane == 0) old = atomicAdd(p.cnt + first, 1u);
+                old = __shfl_sync(kFull, old, 0);
+                if (old != (unsigned)(nch - 1)) continue;
+                __threadfence();
 #pragma unroll
-            for (int j = 0; j < W; ++j) pp[32 * j] = S[j];
-            __threadfence();
-            __syncwarp();
-            const int first = p.slot_first[slot];
-            const int nch = p.slot_nch[slot];
-            unsigned old = 0;
-            if (lane == 0) old = atomicAdd(p.cnt + first, 1u);
-            old = __shfl_sync(kFull, old, 0);
-            if (old != (unsigned)(nch - 1)) continue;
-            __threadfence();
-#pragma unroll
-            for (int j = 0; j < W; ++j) S[j] = 0.0f;
+                for (int t = 0; t < W; ++t) S[t] = 0.0f;
 #pragma unroll 4
-            for (int c = 0; c < nch; ++c) {  // chunk order; the unrolled loads are independent
-                const float *q = reinterpret_cast<const float *>(p.part) + (size_t)(first + c) * B + lane;
+                for (int c = 0; c < nch; ++c) {  // chunk order; the unrolled loads are independent
+                    const float *q = reinterpret_cast<const float *>(p.part) + (size_t)(first + c) * B + W * lane;
+                    if constexpr (W >= 4) {
 #pragma unroll
-                for (int j = 0; j < W; ++j) S[j] += __ldcg(q + 32 * j);
+                        for (int t = 0; t < W; t += 4) {
+                            const float4 x = __ldcg(reinterpret_cast<const float4 *>(q + t));
+                            S[t] += x.x;
+                            S[t + 1] += x.y;
+                            S[t + 2] += x.z;
+                            S[t + 3] += x.w;
+                        }
+                    } else {
+#pragma unroll
+                        for (int t = 0; t < W; ++t) S[t] += __ldcg(q + t);
+                    }
+                }
+                if (lane == 0) p.cnt[first] = 0u;
             }
-            body::finalize_dep<W>(p.sigma, Sl, sig_ones, Cl, p.bc, v, f, S, lane);
-            if (lane == 0) p.cnt[first] = 0u;
+            if (!early) {
+#pragma unroll
+                for (int t = 0; t < (W + 1) / 2; ++t) cnt[t] = 0x00010001u;  // level 1: every count is 1
+                if (Sl && fw != 0u) body::ldg_packed<W, NC>(Sl + at, cnt);
+            }
+            float hi = 0.0f, lo = 0.0f;
+            body::finalize_packed<W, NC>(p.sigma, sig_ones || Sl != nullptr, cnt, Cl, fw, at, S, lane, hi, lo);
+            body::add_dependencies(p.bc, v, hi, lo, lane);
+            __syncwarp();  // the next item's copies overwrite sig
         }
     }
     // light vertices, as in the forward sweep
     const int nlight = p.nitems - p.nheavy;
-    const int share = light_share(nlight, G);
+    const int share = light_share(nlight, G, p.light_least);
     // from the last warp down: the first ones have the more heavy items
-    for (int g0 = (G - 1 - (int)(blockIdx.x * kWarps + wib)) * share; g0 < nlight; g0 += G * share) {
+    for (int g0 = (G - 1 - (bid * kWarps + wib)) * share; g0 < nlight; g0 += G * share) {
         bool act = false;
         int4 item = make_int4(0, 0, 0, 0);
-        __syncwarp();  // the previous group's reads of s_f are done
+        __syncwarp();  // the previous group's reads of f are done
         if (lane < share && g0 + lane < nlight) {
             item = __ldg(p.items + p.nheavy + g0 + lane);
             uint32_t f[W];
-            load_row<W>(Fl + (size_t)item.x * W, f);
+            load_row<W, NC>(Fl + (size_t)item.x * W, f);
             uint32_t any = 0;
 #pragma unroll
             for (int j = 0; j < W; ++j) {
-                s_f[wib][lane][j] = f[j];
+                sh.f[wib][lane][j] = f[j];
                 any |= f[j];
             }
             act = any != 0u;
@@ -559,10 +635,25 @@ __global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const 
         const unsigned lt = __ballot_sync(kFull, act);
         __syncwarp();
         if (lt)
-            body::bwd_light<W, true, true>(lt, item.x, item.y, item.z - item.y, s_f[wib],
+            body::bwd_light<W, NC, true>(lt, item.x, item.y, item.z - item.y, sh.f[wib],
                                            *reinterpret_cast<body::LightScratch<W> *>(ws.buf), p.col, ufs_f, Fs, Cs,
                                            p.sigma, Sl, sig_ones, Cl, p.bc, lane);
     }
+}
+
+template <int W, bool HOOK>
+__global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const int l) {
+    pdl::enter();
+    __shared__ BwdShared<W> sh;
+    __shared__ uint64_t s_bar[kWarps];
+    extern __shared__ __align__(128) uint8_t s_stage[];
+    const int lane = threadIdx.x & 31;
+    const int wib = threadIdx.x >> 5;
+    body::WarpStage ws{s_stage + wib * stage::kBwdStageBytes, s_bar + wib, sh.qz[wib], 0u, false,
+                       body::stage_wctl(p.wait_ns, p.test_hold)};
+    if (lane == 0) stage::bar_init(ws.bar);
+    __syncwarp();
+    backward_items<W, HOOK, true>(p, l, blockIdx.x, gridDim.x, sh, ws);
     if (lane == 0 && ws.fail) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
 }
 
@@ -578,18 +669,19 @@ __global__ void __launch_bounds__(kBlock, 4) k_backward(const MsParams p, const 
 // tile are issued before any is used. Every sum is an integer mod 2^64, so
 // the block totals go straight into the outputs with atomic adds (the run
 // zeroes them first) and the result does not depend on the order of adds.
-template <int W>
-__global__ void __launch_bounds__(kBlock, 2) k_hash(const MsParams p, const int L) {
+template <int W, bool NC, int kHL, int kX>
+__device__ __forceinline__ void hash_tiles(const MsParams &p, const int L, const int bid, const int nblk,
+                                           unsigned long long (&sh)[4][32 * W]) {
     constexpr int B = 32 * W;
-    constexpr int kHL = 12;  // frontier levels loaded up front; deeper ones in a loop
-    pdl::enter();
-    __shared__ unsigned long long sh[4][B];
+    // kHL frontier levels loaded up front (deeper ones in a loop), kX counts at a time
+    static_assert(32 % kX == 0, "whole runs of a tile's 32 vertices");
+    using body::ldx;
     for (int i = threadIdx.x; i < 4 * B; i += kBlock) (&sh[0][0])[i] = 0ull;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * kWarps + (threadIdx.x >> 5);
+    const int gw = bid * kWarps + (threadIdx.x >> 5);
     const int j = gw % W;                        // this warp's frontier word
-    const int tstride = gridDim.x * kWarps / W;  // warps per word
+    const int tstride = nblk * kWarps / W;  // warps per word
     const int ntiles = (p.n + 31) / 32;
     const size_t nW = (size_t)p.n * W;
     const uint32_t *Vl = p.V + (size_t)(L & 1) * nW;
@@ -613,27 +705,29 @@ __global__ void __launch_bounds__(kBlock, 2) k_hash(const MsParams p, const int 
         const size_t wk = (size_t)(in ? vk : 0) * W + j;
         uint32_t fw[kHL];
 #pragma unroll
-        for (int l = 0; l < kHL; ++l) fw[l] = (in && l <= L) ? __ldg(p.F + (size_t)l * nW + wk) : 0u;
-        const uint32_t rv = in ? (__ldg(Vl + wk) | __ldg(FL + wk)) : 0u;
+        for (int l = 0; l < kHL; ++l) fw[l] = (in && l <= L) ? ldx<NC>(p.F + (size_t)l * nW + wk) : 0u;
+        const uint32_t rv = in ? (ldx<NC>(Vl + wk) | ldx<NC>(FL + wk)) : 0u;
         const int nk = p.n - v0 < 32 ? p.n - v0 : 32;  // vertices in this tile
         const uint64_t *sg = p.sigma + (size_t)v0 * B + 32 * j + lane;
-        uint64_t x[16];
+        uint64_t x[kX];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) x[k] = k < nk ? __ldg(sg + (size_t)k * B) : 0ull;
+        for (int k = 0; k < kX; ++k) x[k] = k < nk ? ldx<NC>(sg + (size_t)k * B) : 0ull;
         const uint32_t R = transpose32(rv, lane);
         rc += (uint64_t)__popc(R);
 #pragma unroll
         for (int l = 0; l < kHL; ++l)
             if (l <= L) level_terms(fw[l], l, v0);
-        for (int l = kHL; l <= L; ++l) level_terms(in ? __ldg(p.F + (size_t)l * nW + wk) : 0u, l, v0);
+        for (int l = kHL; l <= L; ++l) level_terms(in ? ldx<NC>(p.F + (size_t)l * nW + wk) : 0u, l, v0);
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if ((R >> k) & 1u) hs += x[k] * (uint64_t)(v0 + k + 1);
+        for (int k0 = 0; k0 < 32; k0 += kX) {
 #pragma unroll
-        for (int k = 0; k < 16; ++k) x[k] = 16 + k < nk ? __ldg(sg + (size_t)(16 + k) * B) : 0ull;
+            for (int k = 0; k < kX; ++k)
+                if ((R >> (k0 + k)) & 1u) hs += x[k] * (uint64_t)(v0 + k0 + k + 1);
+            if (k0 + kX < 32)
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if ((R >> (16 + k)) & 1u) hs += x[k] * (uint64_t)(v0 + 16 + k + 1);
+                for (int k = 0; k < kX; ++k)
+                    x[k] = k0 + kX + k < nk ? ldx<NC>(sg + (size_t)(k0 + kX + k) * B) : 0ull;
+        }
     }
     atomicAdd(&sh[0][32 * j + lane], (unsigned long long)hs);
     atomicAdd(&sh[1][32 * j + lane], (unsigned long long)hd);
@@ -647,6 +741,13 @@ __global__ void __launch_bounds__(kBlock, 2) k_hash(const MsParams p, const int 
         atomicAdd(reinterpret_cast<unsigned long long *>(p.dist_sum + o), sh[2][b]);
         atomicAdd(reinterpret_cast<unsigned long long *>(p.reach + o), sh[3][b]);
     }
+}
+
+template <int W>
+__global__ void __launch_bounds__(kBlock, 2) k_hash(const MsParams p, const int L) {
+    pdl::enter();
+    __shared__ unsigned long long sh[4][32 * W];
+    hash_tiles<W, true, 12, 16>(p, L, blockIdx.x, gridDim.x, sh);
 }
 
 // Rows of the forward pass for bc_forward_rows: out[b][v] for this batch. The
@@ -717,6 +818,226 @@ __global__ void __launch_bounds__(kRowBlock) k_rows(const MsParams p, const int 
     }
 }
 
+// ---- the whole sweep of a run in one launch
+//
+// A level of a small graph is a few microseconds of work, less than a launch
+// costs the host, and the host learns a batch's depth before it can start the
+// backward levels. Here the GPU's resident blocks are split into groups, each
+// group takes batches grp, grp + groups, ... (the lanes of the launch-per-level
+// form) and runs all their levels itself, its blocks meeting at a barrier in
+// global memory after every level. The launch is cooperative, so every block
+// of a group is resident and the barrier cannot starve; its waits are bounded
+// all the same (kSweepWaitNs, then BC_STATUS_COPY_TIMEOUT, which the host
+// reports as a timeout).
+//
+// Data of one level is written by other SMs of the group and read after the
+// barrier: the barrier's fences order the generic accesses and drop stale L1
+// lines, a proxy fence orders them before the bulk copies, and nothing is read
+// through the non-coherent path (NC = false).
+constexpr uint64_t kSweepWaitNs = 10000000000ull;
+
+struct SweepSync {
+    unsigned arrive;       // barrier arrivals, counted up
+    unsigned produced[4];  // by level modulo 4: the level made a frontier
+    unsigned pad[27];
+};
+static_assert(kSweepGroups * sizeof(SweepSync) == kSweepSyncBytes, "barrier words of every group");
+
+template <int W>
+struct SweepShared {
+    union {
+        FwdShared<W> fwd;
+        BwdShared<W> bwd;
+        FirstShared first;
+        unsigned long long hash[4][32 * W];
+    };
+    MsParams p;  // the group's batch in work
+    uint64_t bar[kWarps];
+    unsigned level_made;
+    bool ok;
+};
+
+// All nblk blocks of the group pass; false once a wait ran out.
+template <int W>
+__device__ __forceinline__ bool group_barrier(SweepSync *sync, int nblk, unsigned &round, SweepShared<W> &sh) {
+    asm volatile("fence.proxy.async;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        ++round;
+        const unsigned want = round * (unsigned)nblk;
+        __threadfence();
+        atomicAdd(&sync->arrive, 1u);
+        bool ok = true;
+        uint64_t t0 = 0;
+        for (unsigned spin = 0;; ++spin) {
+            unsigned seen;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&sync->arrive) : "memory");
+            if ((int)(seen - want) >= 0) break;
+            if ((spin & 255u) == 255u) {
+                const uint64_t now = stage::now_ns();
+                if (t0 == 0) t0 = now;
+                if (now - t0 > kSweepWaitNs) {
+                    ok = false;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+        sh.ok = ok;
+    }
+    __syncthreads();
+    asm volatile("fence.proxy.async;" ::: "memory");
+    return sh.ok;
+}
+
+template <int W>
+__global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ SweepParams q) {
+    __shared__ SweepShared<W> sh;
+    extern __shared__ __align__(128) uint8_t s_stage[];
+    const int grp = blockIdx.x / q.group_blocks, bid = blockIdx.x % q.group_blocks, nblk = q.group_blocks;
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    const bool lead = bid == 0 && tid == 0;
+    SweepSync *sync = reinterpret_cast<SweepSync *>(q.sync) + grp;
+    unsigned round = 0;
+    body::WarpStage ws{s_stage + wib * stage::kFwdStageBytes, sh.bar + wib, nullptr, 0u, false, 0u};
+    if (lane == 0) stage::bar_init(ws.bar);
+    if (tid == 0) sh.p = q.g[grp];
+    __syncthreads();
+    MsParams &p = sh.p;
+    const size_t nB = (size_t)p.n * 32 * W;
+    for (int i = bid * kBlock + tid; i < p.n; i += nblk * kBlock) p.bc[i] = 0.0;
+
+    bool alive = true;
+    for (int bi = grp; alive && bi < q.nbat; bi += q.groups) {
+        const int b0 = bi * 32 * W;
+        if (tid == 0) {
+            p.nb = min(32 * W, q.nsrc - b0);
+            p.sources = q.sources + b0;
+            p.out_index = q.out_index ? q.out_index + b0 : nullptr;
+            const int o = q.out_index ? 0 : b0;
+            p.h_sigma = q.h_sigma + o;
+            p.h_dist = q.h_dist + o;
+            p.dist_sum = q.dist_sum + o;
+            p.reach = q.reach + o;
+            p.nitems = q.g[grp].nitems;
+            p.nheavy = q.g[grp].nheavy;
+            p.nslots = q.g[grp].nslots;
+            p.items = q.g[grp].items;
+            p.item_v = q.g[grp].item_v;
+            p.slot_first = q.g[grp].slot_first;
+            p.slot_nch = q.g[grp].slot_nch;
+        }
+        __syncthreads();
+        init_zero<W>(p, bid, nblk);
+        for (int i = bid * kBlock + tid; i < p.Lcap; i += nblk * kBlock) p.lsize[i] = 0u;
+        if (q.hash && bid == nblk - 1)
+            for (int b = tid; b < p.nb; b += kBlock) {
+                const int o = p.out_index ? p.out_index[b] : b;
+                p.h_sigma[o] = 0ull;
+                p.h_dist[o] = 0ull;
+                p.dist_sum[o] = 0;
+                p.reach[o] = 0;
+            }
+        if (lead)
+            for (int k = 0; k < 4; ++k) sync->produced[k] = 0u;
+        if (!group_barrier<W>(sync, nblk, round, sh)) break;
+        for (int b = bid * kBlock + tid; b < p.nb; b += nblk * kBlock) init_source<W>(p, b);
+        const int total = first_scan(p, sh.first);
+        // level 0 -> 1 top-down by the rule on the sources' arcs
+        const bool top = q.first_rule < 2 ? q.first_rule == 1 : (double)total * (double)q.alpha < (double)q.narcs;
+        if (top) first_arcs<W>(p, bid, nblk, sh.first, total);
+        if (lead) {
+            p.lsize[0] = (uint32_t)p.nb;
+            if (top) {
+                p.lsize[1] = (uint32_t)total;
+                atomicAdd(&p.ctl->dag_arcs, (unsigned long long)total);
+            }
+        }
+        if (tid == 0) p.first = top ? 1 : 0;
+        if (!group_barrier<W>(sync, nblk, round, sh)) break;
+
+        int L = 0;
+        for (int l = top ? 1 : 0; !(top && total == 0); ++l) {
+            if (l + 1 >= p.Lcap) {  // deeper than the state's levels: the host grows it and starts over
+                if (lead) atomicOr(&p.ctl->status, BC_STATUS_LEVEL_CAP);
+                alive = false;
+                break;
+            }
+            if (tid == 0) {
+                sh.fwd.flags = 0u;
+                sh.fwd.arcs = 0ull;
+                sh.fwd.front = 0u;
+            }
+            if (lead) sync->produced[(l + 2) & 3] = 0u;  // last read two levels ago
+            __syncthreads();
+            ws.qz = sh.fwd.qz[wib];
+            FwdFound found;
+            forward_items<W, false, false>(p, l, bid, nblk, sh.fwd, ws, p.S + (size_t)(l % p.s_levels) * nB,
+                                           p.S + (size_t)((l + 1) % p.s_levels) * nB, l == 1 && top, found);
+            forward_collect(sh.fwd, found, ws.fail);
+            __syncthreads();
+            if (tid == 0) {
+                const uint32_t f = sh.fwd.flags;
+                if (sh.fwd.arcs) atomicAdd(&p.ctl->dag_arcs, sh.fwd.arcs);
+                if (sh.fwd.front) atomicAdd(p.lsize + l + 1, sh.fwd.front);
+                if (f & 1u) atomicOr(&sync->produced[l & 3], 1u);
+                if (f & 2u) atomicOr(&p.ctl->status, BC_STATUS_SIGMA_OVERFLOW);
+                if (f & 4u) atomicOr(p.wide + l + 1, 1u);
+                if (f & 8u) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
+            }
+            if (!(alive = group_barrier<W>(sync, nblk, round, sh))) break;
+            if (tid == 0) sh.level_made = *(volatile unsigned *)&sync->produced[l & 3];
+            __syncthreads();
+            if (sh.level_made == 0u) {
+                L = l;
+                break;
+            }
+        }
+        if (!alive) break;
+        if (lead) atomicAdd(&p.ctl->depth_sum, (unsigned long long)L);
+        __syncthreads();
+        if (tid == 0) {
+            p.nitems = q.b_nitems;
+            p.nheavy = q.b_nheavy;
+            p.nslots = q.b_nslots;
+            p.items = q.b_items;
+            p.item_v = q.b_item_v;
+            p.slot_first = q.b_slot_first;
+            p.slot_nch = q.b_slot_nch;
+        }
+        __syncthreads();
+        ws.qz = sh.bwd.qz[wib];
+        for (int l = L; alive && l >= 1; --l) {
+            backward_items<W, false, false>(p, l, bid, nblk, sh.bwd, ws);
+            alive = group_barrier<W>(sync, nblk, round, sh);
+        }
+        if (!alive) break;
+        if (q.hash) {
+            hash_tiles<W, false, 6, 8>(p, L, bid, nblk, sh.hash);
+            if (!(alive = group_barrier<W>(sync, nblk, round, sh))) break;
+        }
+    }
+    if (lane == 0 && ws.fail) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
+    if (tid == 0 && !sh.ok && round > 0) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
+    // the last block of all reports the end and the status to the host
+    __syncthreads();
+    if (tid != 0) return;
+    __threadfence();
+    if (atomicAdd(q.finished, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    host_word(&p.hctl->done, q.seq, *(volatile uint32_t *)&p.ctl->status);
+}
+
+// bc[i] = (add: bc[i] +) the groups' sums, in group order.
+__global__ void __launch_bounds__(kBlock) k_sweep_merge(const __grid_constant__ SweepParams q, double *__restrict__ bc,
+                                                        int32_t n, bool add) {
+    for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock) {
+        double x = add ? bc[i] : 0.0;
+        for (int k = 0; k < q.groups; ++k) x += q.g[k].bc[i];
+        bc[i] = x;
+    }
+}
+
 __global__ void k_merge(const double *__restrict__ src, double *__restrict__ dst, int32_t n, const DevCtl *from,
                         DevCtl *to) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] += src[i];
@@ -748,34 +1069,33 @@ static_assert(sizeof(body::LightScratch<8>) <= stage::kFwdStageBytes && sizeof(b
 constexpr size_t kFwdSmem = (size_t)kWarps * stage::kFwdStageBytes;
 constexpr size_t kBwdSmem = (size_t)kWarps * stage::kBwdStageBytes;
 
-// Raise the kernel's dynamic shared memory limit once per device.
+// Blocks of the kernel that the current device holds at once. Asked, and the
+// kernel's dynamic shared memory limit raised, once per device.
+constexpr int kMaxDevices = 64;
+struct Resident {
+    std::atomic<int> blocks[kMaxDevices];
+};
 template <class K>
-void stage_attr(K kernel, size_t bytes, std::atomic<uint32_t> &done) {
+int resident_blocks(K kernel, size_t dyn_smem, Resident &known) {
     int dev = 0;
     cudaGetDevice(&dev);
-    const uint32_t bit = 1u << (dev & 31);
-    if (done.load(std::memory_order_acquire) & bit) return;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    done.fetch_or(bit, std::memory_order_acq_rel);
-}
-template <int W, bool HOOK>
-void fwd_attr() {
-    static std::atomic<uint32_t> done{0};
-    stage_attr(k_forward<W, HOOK>, kFwdSmem, done);
-}
-template <int W, bool HOOK>
-void bwd_attr() {
-    static std::atomic<uint32_t> done{0};
-    stage_attr(k_backward<W, HOOK>, kBwdSmem, done);
+    const bool kept = dev >= 0 && dev < kMaxDevices;
+    if (kept)
+        if (const int b = known.blocks[dev].load(std::memory_order_acquire); b > 0) return b;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_smem);
+    int per_sm = 0;
+    const bool ok =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, dyn_smem) == cudaSuccess && per_sm > 0;
+    if (!ok) return 0;
+    if (kept) known.blocks[dev].store(per_sm * sm_count(), std::memory_order_release);
+    return per_sm * sm_count();
 }
 
-template <class K>
-int item_blocks(const MsParams &p, K kernel, size_t dyn_smem = 0) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, dyn_smem) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
+// Persistent grid of a level kernel: as many blocks as are resident at once,
+// never more than the items need.
+int item_blocks(const MsParams &p, int resident) {
     const int need = (p.nitems + kWarps - 1) / kWarps;
-    const int cap = per_sm * sm_count();
+    const int cap = resident > 0 ? resident : sm_count();
     return need < cap ? need : cap;
 }
 
@@ -785,18 +1105,17 @@ bool uses_hook(const MsParams &p) { return p.wait_ns != 0 || p.test_hold != 0; }
 
 template <int W, bool HOOK>
 void launch_forward_t(const MsParams &p, int level, cudaStream_t st) {
-    fwd_attr<W, HOOK>();
-    pdl::launch(k_forward<W, HOOK>, item_blocks(p, k_forward<W, HOOK>, kFwdSmem), kBlock, kFwdSmem, st, p, level);
+    static Resident known;
+    const int g = item_blocks(p, resident_blocks(k_forward<W, HOOK>, kFwdSmem, known));
+    pdl::launch(k_forward<W, HOOK>, g, kBlock, kFwdSmem, st, p, level);
 }
 template <int W, bool HOOK>
 void launch_backward_t(const MsParams &p, int level, cudaStream_t st) {
-    bwd_attr<W, HOOK>();
-    pdl::launch(k_backward<W, HOOK>, item_blocks(p, k_backward<W, HOOK>, kBwdSmem), kBlock, kBwdSmem, st, p,
-                level);
+    static Resident known;
+    const int g = item_blocks(p, resident_blocks(k_backward<W, HOOK>, kBwdSmem, known));
+    pdl::launch(k_backward<W, HOOK>, g, kBlock, kBwdSmem, st, p, level);
 }
 
-// Persistent grid: as many blocks as fit on the GPU at once (occupancy of
-// the kernel instance), never more than the items need.
 template <int W>
 void launch_init_t(const MsParams &p, cudaStream_t st) {
     const size_t work = (size_t)p.n * W;
@@ -870,6 +1189,38 @@ void ms_launch_rows(int W, const MsParams &p, int nlevels, uint64_t *sig_out, in
     const int cap = 6 * sm_count();  // the tiles' shared memory: six blocks per SM
     const int g = need < 1 ? 1 : (need < cap ? need : cap);
     BCGB_DISPATCH_W(W, pdl::launch(k_rows<kW>, g, kRowBlock, 0, st, p, nlevels, sig_out, dist_out));
+}
+
+namespace {
+template <int W>
+int sweep_blocks_t() {
+    static Resident known;
+    return resident_blocks(k_sweep<W>, kFwdSmem, known);
+}
+template <int W>
+cudaError_t sweep_launch_t(const SweepParams &q, cudaStream_t st) {
+    void *args[] = {const_cast<SweepParams *>(&q)};
+    return cudaLaunchCooperativeKernel((const void *)k_sweep<W>, dim3(q.groups * q.group_blocks), dim3(kBlock), args,
+                                       kFwdSmem, st);
+}
+}  // namespace
+
+int ms_sweep_blocks(int W) {
+    int b = 0;
+    BCGB_DISPATCH_W(W, b = sweep_blocks_t<kW>());
+    return b;
+}
+
+cudaError_t ms_launch_sweep(int W, const SweepParams &q, cudaStream_t st) {
+    cudaError_t e = cudaErrorInvalidValue;
+    BCGB_DISPATCH_W(W, e = sweep_launch_t<kW>(q, st));
+    return e;
+}
+
+void ms_launch_sweep_merge(const SweepParams &q, double *bc, int32_t n, bool add, cudaStream_t st) {
+    int g = (n + kBlock - 1) / kBlock;
+    g = g < 1 ? 1 : (g > 4 * sm_count() ? 4 * sm_count() : g);
+    k_sweep_merge<<<g, kBlock, 0, st>>>(q, bc, n, add);
 }
 
 void ms_launch_merge(const double *src, double *dst, int32_t n, const DevCtl *from, DevCtl *to, cudaStream_t st) {

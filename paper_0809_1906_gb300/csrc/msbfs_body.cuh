@@ -210,6 +210,68 @@ __device__ __forceinline__ void unpack_lanes(T *p, const T (&x)[W], T (&out)[W],
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// W consecutive entries of a row in global memory, one vector load.
+template <int W, bool NC>
+__device__ __forceinline__ void ldg_packed(const uint16_t *p, uint32_t (&x)[(W + 1) / 2]) {
+    if constexpr (W == 8) {
+        const uint4 t = ldx<NC>(reinterpret_cast<const uint4 *>(p));
+        x[0] = t.x;
+        x[1] = t.y;
+        x[2] = t.z;
+        x[3] = t.w;
+    } else if constexpr (W == 4) {
+        const uint2 t = ldx<NC>(reinterpret_cast<const uint2 *>(p));
+        x[0] = t.x;
+        x[1] = t.y;
+    } else if constexpr (W == 2) {
+        x[0] = ldx<NC>(reinterpret_cast<const uint32_t *>(p));
+    } else {
+        x[0] = ldx<NC>(p);
+    }
+}
+template <int W, bool NC>
+__device__ __forceinline__ void ldg_packed(const float *p, float (&x)[W]) {
+    if constexpr (W >= 4) {
+#pragma unroll
+        for (int i = 0; i < W / 4; ++i) {
+            const float4 t = ldx<NC>(reinterpret_cast<const float4 *>(p) + i);
+            x[4 * i] = t.x;
+            x[4 * i + 1] = t.y;
+            x[4 * i + 2] = t.z;
+            x[4 * i + 3] = t.w;
+        }
+    } else if constexpr (W == 2) {
+        const float2 t = ldx<NC>(reinterpret_cast<const float2 *>(p));
+        x[0] = t.x;
+        x[1] = t.y;
+    } else {
+        x[0] = ldx<NC>(p);
+    }
+}
+template <int W>
+__device__ __forceinline__ void stg_packed(uint16_t *p, const uint32_t (&x)[(W + 1) / 2]) {
+    if constexpr (W == 8)
+        *reinterpret_cast<uint4 *>(p) = make_uint4(x[0], x[1], x[2], x[3]);
+    else if constexpr (W == 4)
+        *reinterpret_cast<uint2 *>(p) = make_uint2(x[0], x[1]);
+    else if constexpr (W == 2)
+        *reinterpret_cast<uint32_t *>(p) = x[0];
+    else
+        *p = (uint16_t)x[0];
+}
+template <int W>
+__device__ __forceinline__ void stg_packed(float *p, const float (&x)[W]) {
+    if constexpr (W >= 4) {
+#pragma unroll
+        for (int i = 0; i < W / 4; ++i)
+            reinterpret_cast<float4 *>(p)[i] = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+    } else if constexpr (W == 2) {
+        *reinterpret_cast<float2 *>(p) = make_float2(x[0], x[1]);
+    } else {
+        *p = x[0];
+    }
+}
+
 // One 32-arc chunk: lane k gets arc e (if e < end), its neighbour u_k (stored
 // in s_u[k]) and masks m_k[j] = frontier words of u_k AND want[j] (zero for
 // arcs that cannot contribute); s_nz[k] gets the W-bit set of non-zero words
@@ -459,92 +521,98 @@ __device__ __forceinline__ void bwd_sum_sparse(const int32_t *__restrict__ col, 
             const uint32_t p = pos[i];
 #pragma unroll
             for (int j = 0; j < W; ++j)
-                if (p == 32u * j + (uint32_t)lane) S[j] += t;
+                if (p == (uint32_t)(W * lane + j)) S[j] += t;  // packed view
         }
     }
 }
 
-template <int W, bool NC = true, bool STAGED = false, bool HOOK = false>
-__device__ __forceinline__ void bwd_sum(const int32_t *__restrict__ col, int beg, int end,
-                                        const uint32_t *__restrict__ ufs, const uint32_t *__restrict__ Fs,
-                                        const float *__restrict__ Cs, const uint32_t (&f)[W], int32_t *s_u,
-                                        uint32_t *s_nz, int lane, float (&S)[W], WarpStage *ws = nullptr) {
+// The staged form: S in the packed view (S[t]: source W lane + t).
+template <int W, bool NC, bool HOOK>
+__device__ __forceinline__ void bwd_sum_staged(const int32_t *__restrict__ col, int beg, int end,
+                                               const uint32_t *__restrict__ ufs, const uint32_t *__restrict__ Fs,
+                                               const float *__restrict__ Cs, const uint32_t (&f)[W], int32_t *s_u,
+                                               uint32_t *s_nz, int lane, float (&S)[W], WarpStage *ws) {
     constexpr int B = 32 * W;
-    if constexpr (STAGED) {
-        int nsrc = 0;
+    int nsrc = 0;
 #pragma unroll
-        for (int j = 0; j < W; ++j) nsrc += __popc(f[j]);
-        if (nsrc <= kSparseSrc) {
-            // list the sources in the stage's slot-mask array (free in this form)
-            if (lane == 0) {
-                int k = 0;
+    for (int j = 0; j < W; ++j) nsrc += __popc(f[j]);
+    if (nsrc <= kSparseSrc) {
+        // list the sources in the stage's slot-mask array (free in this form)
+        if (lane == 0) {
+            int k = 0;
 #pragma unroll
-                for (int j = 0; j < W; ++j) {
-                    uint32_t x = f[j];
-                    while (x) {
-                        ws->qz[k++] = 32u * j + (uint32_t)(__ffs(x) - 1);
-                        x &= x - 1;
-                    }
+            for (int j = 0; j < W; ++j) {
+                uint32_t x = f[j];
+                while (x) {
+                    ws->qz[k++] = 32u * j + (uint32_t)(__ffs(x) - 1);
+                    x &= x - 1;
                 }
             }
-            __syncwarp();
-            bwd_sum_sparse<W, NC>(col, beg, end, ufs, Fs, Cs, f, s_u, s_nz, lane, S, ws->qz, nsrc);
-            __syncwarp();
-            return;
         }
+        __syncwarp();
+        bwd_sum_sparse<W, NC>(col, beg, end, ufs, Fs, Cs, f, s_u, s_nz, lane, S, ws->qz, nsrc);
+        __syncwarp();
+        return;
     }
-    float Sp[W];  // staged sums, packed view (lane owns sources W*lane + t)
-#pragma unroll
-    for (int t = 0; t < W; ++t) Sp[t] = 0.0f;
-    bool staged = false;
     for (int e0 = beg; e0 < end; e0 += 32) {
         uint32_t m[W];
         int u;
         uint32_t nz;
         unsigned bal = probe_chunk<W, NC>(col, e0 + lane, end, ufs, Fs, f, m, s_u, s_nz, lane, u, nz);
-        if constexpr (STAGED) {
-            // rounds of up to R rows; a lane copies the span of its
-            // neighbour's c row from the first to the last word that can
-            // contribute, and the adder takes only the contributing words
-            constexpr int RB = 4 * B;
-            constexpr int R = (int)stage::kBwdStageBytes / RB < 32 ? (int)stage::kBwdStageBytes / RB : 32;
-            const float *st = reinterpret_cast<const float *>(ws->buf);
-            const int jl = (W * lane) >> 5;  // the row word holding this lane's sources
-            while (bal && !ws->fail) {
-                const int rank = __popc(bal & ((1u << lane) - 1u));
-                const bool go = ((bal >> lane) & 1u) && rank < R;
-                const unsigned take = __ballot_sync(kFull, go);
-                const int nq = __popc(take);
-                const int lo = __ffs(nz) - 1, hi = 31 - __clz(nz);
-                const uint32_t bytes = go ? 128u * (uint32_t)(hi - lo + 1) : 0u;
-                const uint32_t tot = __reduce_add_sync(kFull, bytes);
-                if (go) ws->qz[rank] = nz;
-                if (lane == 0) stage::expect_tx(ws->bar, tot + (HOOK ? stage_hold(ws) : 0u));
-                __syncwarp();
-                if (go) stage::copy(ws->buf + rank * RB + 128 * lo, Cs + (size_t)u * B + 32 * lo, bytes, ws->bar);
-                const uint32_t ph = ws->phase;
-                const bool ok = stage::wait(ws->bar, ph, HOOK ? stage_limit_us(ws) : 0u);
-                ws->phase ^= 1u;
-                if (!__all_sync(kFull, ok)) {
-                    give_up(ws, ph, lane, HOOK ? stage_hold(ws) : 0u);
-                    break;
-                }
+        // rounds of up to R rows; a lane copies the span of its neighbour's c
+        // row from the first to the last word that can contribute, and the
+        // adder takes only the contributing words
+        constexpr int RB = 4 * B;
+        constexpr int R = (int)stage::kBwdStageBytes / RB < 32 ? (int)stage::kBwdStageBytes / RB : 32;
+        const float *st = reinterpret_cast<const float *>(ws->buf);
+        const int jl = (W * lane) >> 5;  // the row word holding this lane's sources
+        while (bal && !ws->fail) {
+            const int rank = __popc(bal & ((1u << lane) - 1u));
+            const bool go = ((bal >> lane) & 1u) && rank < R;
+            const unsigned take = __ballot_sync(kFull, go);
+            const int nq = __popc(take);
+            const int lo = __ffs(nz) - 1, hi = 31 - __clz(nz);
+            const uint32_t bytes = go ? 128u * (uint32_t)(hi - lo + 1) : 0u;
+            const uint32_t tot = __reduce_add_sync(kFull, bytes);
+            if (go) ws->qz[rank] = nz;
+            if (lane == 0) stage::expect_tx(ws->bar, tot + (HOOK ? stage_hold(ws) : 0u));
+            __syncwarp();
+            if (go) stage::copy(ws->buf + rank * RB + 128 * lo, Cs + (size_t)u * B + 32 * lo, bytes, ws->bar);
+            const uint32_t ph = ws->phase;
+            const bool ok = stage::wait(ws->bar, ph, HOOK ? stage_limit_us(ws) : 0u);
+            ws->phase ^= 1u;
+            if (!__all_sync(kFull, ok)) {
+                give_up(ws, ph, lane, HOOK ? stage_hold(ws) : 0u);
+                break;
+            }
 #pragma unroll 2
-                for (int q = 0; q < nq; ++q) {
-                    if ((ws->qz[q] >> jl) & 1u) {
-                        float x[W];
-                        lds_packed<W>(st + q * B + W * lane, x);
+            for (int q = 0; q < nq; ++q) {
+                if ((ws->qz[q] >> jl) & 1u) {
+                    float x[W];
+                    lds_packed<W>(st + q * B + W * lane, x);
 #pragma unroll
-                        for (int t = 0; t < W; ++t) Sp[t] += x[t];
-                    }
+                    for (int t = 0; t < W; ++t) S[t] += x[t];
                 }
-                __syncwarp();
-                bal &= ~take;
-                staged = true;
             }
             __syncwarp();
-            continue;
+            bal &= ~take;
         }
+        __syncwarp();
+    }
+}
+
+// The word view (S[j]: source 32 j + lane), rows read straight from global memory.
+template <int W, bool NC>
+__device__ __forceinline__ void bwd_sum(const int32_t *__restrict__ col, int beg, int end,
+                                        const uint32_t *__restrict__ ufs, const uint32_t *__restrict__ Fs,
+                                        const float *__restrict__ Cs, const uint32_t (&f)[W], int32_t *s_u,
+                                        uint32_t *s_nz, int lane, float (&S)[W]) {
+    constexpr int B = 32 * W;
+    for (int e0 = beg; e0 < end; e0 += 32) {
+        uint32_t m[W];
+        int u;
+        uint32_t nz;
+        unsigned bal = probe_chunk<W, NC>(col, e0 + lane, end, ufs, Fs, f, m, s_u, s_nz, lane, u, nz);
         const float *base = Cs + lane;
         // two neighbours per step: 2W independent coalesced loads in flight
         while (bal) {
@@ -565,14 +633,6 @@ __device__ __forceinline__ void bwd_sum(const int32_t *__restrict__ col, int beg
             for (int j = 0; j < W; ++j) S[j] += x0[j] + x1[j];
         }
         __syncwarp();
-    }
-    if constexpr (STAGED) {
-        if (staged) {
-            float Sj[W];
-            unpack_lanes<W>(reinterpret_cast<float *>(ws->buf), Sp, Sj, lane);
-#pragma unroll
-            for (int j = 0; j < W; ++j) S[j] += Sj[j];
-        }
     }
 }
 
@@ -613,43 +673,16 @@ __device__ __forceinline__ float sigma_f32(uint64_t x) {
 }
 
 // Cl: the masked level-l c buffer (zeros for the sources v is not at level l
-// for; null at level 1, whose c values no level reads), written in full, or
-// with ALL_WORDS = false only in the words that
-// hold a level-l source of v (every backward adder reads word j of v's row
-// only when v is at level l for a source of word j). For s with d(s,v) = l: delta_s(v) = sigma_s(v) * S
-// and c_s(v) = (1 + delta_s(v)) / sigma_s(v) = 1/sigma_s(v) + S (1/sigma_s(v)
-// by the fast reciprocal, within 2 ulp; the correctly rounded one measured
-// 1.2 ms slower per R-MAT step). The batch's FP32 delta values of v are summed as an
-// unevaluated pair of FP32 words (two_sum_add: W per lane in order, then a
-// 5-step tree across the warp, a fixed order) and the total goes into bc[v]
-// in FP64.
-// sigma_s(v) comes from the level's masked uint16 row Sl when given (a
-// narrow level: every count below 2^16), is 1 when `ones` (level 1, reached
-// from the sources directly), else from the uint64 array. Ssh: when not null,
-// v's words of Sl already copied to shared memory ([W][32], the words with a
-// level-l source), read there instead.
-template <int W, bool ALL_WORDS = true>
-__device__ __forceinline__ void finalize_dep(const uint64_t *sigma, const uint16_t *Sl, bool ones, float *Cl,
-                                             double *bc, int v, const uint32_t (&f)[W], const float (&S)[W],
-                                             int lane, const uint16_t *Ssh = nullptr,
-                                             const uint64_t *Ssig = nullptr) {
-    constexpr int B = 32 * W;
-    float hi = 0.0f, lo = 0.0f;  // the running sum hi + lo, carried without rounding loss
-#pragma unroll
-    for (int j = 0; j < W; ++j) {
-        const size_t idx = (size_t)v * B + 32 * j + lane;
-        float c = 0.0f;
-        if ((f[j] >> lane) & 1u) {
-            const float sg = ones ? 1.0f
-                                  : (Ssh ? __uint2float_rn((uint32_t)Ssh[32 * j + lane])
-                                         : (Ssig ? sigma_f32(Ssig[32 * j + lane])
-                                                 : (Sl ? __uint2float_rn((uint32_t)Sl[idx]) : sigma_f32(sigma[idx]))));
-            const float d = sg * S[j];        // delta_s(v) = sigma_s(v) * sum_w c_s(w)
-            c = __fdividef(1.0f, sg) + S[j];  // c_s(v) for the level above (1/sigma within 2 ulp)
-            two_sum_add(hi, lo, d);
-        }
-        if (Cl && (ALL_WORDS || f[j] != 0u)) Cl[idx] = c;
-    }
+// for; null at level 1, whose c values no level reads), written in the words
+// that hold a level-l source of v: every backward adder reads word j of v's row
+// only when v is at level l for a source of word j. For s with d(s,v) = l:
+// delta_s(v) = sigma_s(v) * S and c_s(v) = (1 + delta_s(v)) / sigma_s(v) =
+// 1/sigma_s(v) + S (1/sigma_s(v) by the fast reciprocal, within 2 ulp; the
+// correctly rounded one measured 1.2 ms slower per R-MAT step). The batch's
+// FP32 delta values of v are summed as an unevaluated pair of FP32 words
+// (two_sum_add): the lane's sources in order, then a 5-step tree across the
+// warp, a fixed order; the total goes into bc[v] in FP64.
+__device__ __forceinline__ void add_dependencies(double *bc, int v, float hi, float lo, int lane) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         const float h2 = __shfl_xor_sync(kFull, hi, off);
@@ -660,11 +693,53 @@ __device__ __forceinline__ void finalize_dep(const uint64_t *sigma, const uint16
     if (lane == 0) bc[v] += (double)hi + (double)lo;
 }
 
-template <int W, bool ALL_WORDS = true>
-__device__ __forceinline__ void finalize_dep(const uint64_t *sigma, float *Cl, double *bc, int v,
-                                             const uint32_t (&f)[W], const float (&S)[W], int lane,
-                                             const uint64_t *Ssig = nullptr) {
-    finalize_dep<W, ALL_WORDS>(sigma, nullptr, false, Cl, bc, v, f, S, lane, nullptr, Ssig);
+// The word view (the many-graph kernel). Ssig: v's counts in shared memory
+// ([W][32], the words with a level-l source).
+template <int W>
+__device__ __forceinline__ void finalize_dep(float *Cl, double *bc, int v, const uint32_t (&f)[W], const float (&S)[W],
+                                             int lane, const uint64_t *Ssig) {
+    constexpr int B = 32 * W;
+    float hi = 0.0f, lo = 0.0f;  // the running sum hi + lo, carried without rounding loss
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+        const size_t idx = (size_t)v * B + 32 * j + lane;
+        float c = 0.0f;
+        if ((f[j] >> lane) & 1u) {
+            const float sg = sigma_f32(Ssig[32 * j + lane]);
+            const float d = sg * S[j];        // delta_s(v) = sigma_s(v) * sum_w c_s(w)
+            c = __fdividef(1.0f, sg) + S[j];  // c_s(v) for the level above (1/sigma within 2 ulp)
+            two_sum_add(hi, lo, d);
+        }
+        if (Cl && f[j] != 0u) Cl[idx] = c;
+    }
+    add_dependencies(bc, v, hi, lo, lane);
+}
+
+// The packed view (the one-graph sweeps): S[t] and the result belong to source
+// W lane + t; fw: the frontier word that holds the lane's sources. The counts
+// come from cnt, the lane's entries of the level's masked uint16 row (a narrow
+// level; all 1 at level 1 from the sources directly), or with `narrow` false
+// from the uint64 array. Against the word view this needs no exchange of the
+// sums between lanes, and one vector load and one or two vector stores per row
+// instead of W of each.
+template <int W, bool NC>
+__device__ __forceinline__ void finalize_packed(const uint64_t *sigma, bool narrow, const uint32_t (&cnt)[(W + 1) / 2],
+                                                float *Cl, uint32_t fw, size_t at, const float (&S)[W], int lane,
+                                                float &hi, float &lo) {
+    const uint32_t mine = fw >> ((W * lane) & 31);  // bits 0 .. W - 1: the lane's sources
+    float c[W];
+#pragma unroll
+    for (int t = 0; t < W; ++t) {
+        c[t] = 0.0f;
+        if ((mine >> t) & 1u) {
+            const float sg = narrow ? __uint2float_rn((cnt[t / 2] >> (16 * (t % 2))) & 0xFFFFu)
+                                    : sigma_f32(ldx<NC>(sigma + at + t));
+            const float d = sg * S[t];           // delta_s(v) = sigma_s(v) * sum_w c_s(w)
+            c[t] = __fdividef(1.0f, sg) + S[t];  // c_s(v) for the level above (1/sigma within 2 ulp)
+            two_sum_add(hi, lo, d);
+        }
+    }
+    if (Cl && fw != 0u) stg_packed<W>(Cl + at, c);
 }
 
 }  // namespace body

@@ -28,84 +28,22 @@ namespace bcgb {
 namespace body {
 
 using bcgb::kLightDeg;
-constexpr int kLightItems = 8;  // vertices of a pack
+using bcgb::kLightItems;
 
 // A warp's scratch in shared memory.
 template <int W>
 struct LightScratch {
-    uint32_t m[32][W];  // per arc of the pack: its neighbour's frontier words AND what its vertex wants
+    __align__(16) uint32_t m[32][W];  // per arc of the pack: its neighbour's frontier words AND what its vertex wants
     int32_t u[32];      // and its neighbour
     // per vertex: itself, its first arc in the graph and in the pack, arcs, index in the group
     int32_t v[kLightItems], beg[kLightItems], off[kLightItems], deg[kLightItems], idx[kLightItems];
     int32_t pos[kSparseSrc];   // backward: the sources of a vertex in the sparse-source form
-    uint32_t nf[kLightItems][W];  // forward: the vertices' new frontier words
+    __align__(16) uint32_t nf[kLightItems][W];  // forward: the vertices' new frontier words
     union {
         float2 acc[kLightItems][32];        // backward: each lane's sum of dependencies (hi, lo)
         __align__(16) uint32_t row[32 * W]; // forward: a vertex's counts, from the packed to the word view
     };
 };
-
-// W consecutive entries of a row in global memory, one vector load.
-template <int W, bool NC>
-__device__ __forceinline__ void ldg_packed(const uint16_t *p, uint32_t (&x)[(W + 1) / 2]) {
-    if constexpr (W == 8) {
-        const uint4 t = ldx<NC>(reinterpret_cast<const uint4 *>(p));
-        x[0] = t.x;
-        x[1] = t.y;
-        x[2] = t.z;
-        x[3] = t.w;
-    } else if constexpr (W == 4) {
-        const uint2 t = ldx<NC>(reinterpret_cast<const uint2 *>(p));
-        x[0] = t.x;
-        x[1] = t.y;
-    } else if constexpr (W == 2) {
-        x[0] = ldx<NC>(reinterpret_cast<const uint32_t *>(p));
-    } else {
-        x[0] = ldx<NC>(p);
-    }
-}
-template <int W, bool NC>
-__device__ __forceinline__ void ldg_packed(const float *p, float (&x)[W]) {
-    if constexpr (W >= 4) {
-#pragma unroll
-        for (int i = 0; i < W / 4; ++i) {
-            const float4 t = ldx<NC>(reinterpret_cast<const float4 *>(p) + i);
-            x[4 * i] = t.x;
-            x[4 * i + 1] = t.y;
-            x[4 * i + 2] = t.z;
-            x[4 * i + 3] = t.w;
-        }
-    } else if constexpr (W == 2) {
-        const float2 t = ldx<NC>(reinterpret_cast<const float2 *>(p));
-        x[0] = t.x;
-        x[1] = t.y;
-    } else {
-        x[0] = ldx<NC>(p);
-    }
-}
-template <int W>
-__device__ __forceinline__ void stg_packed(uint16_t *p, const uint32_t (&x)[(W + 1) / 2]) {
-    if constexpr (W == 8)
-        *reinterpret_cast<uint4 *>(p) = make_uint4(x[0], x[1], x[2], x[3]);
-    else if constexpr (W == 4)
-        *reinterpret_cast<uint2 *>(p) = make_uint2(x[0], x[1]);
-    else if constexpr (W == 2)
-        *reinterpret_cast<uint32_t *>(p) = x[0];
-    else
-        *p = (uint16_t)x[0];
-}
-template <int W>
-__device__ __forceinline__ void stg_packed(float *p, const float (&x)[W]) {
-    if constexpr (W >= 4) {
-#pragma unroll
-        for (int i = 0; i < W / 4; ++i)
-            reinterpret_cast<float4 *>(p)[i] = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
-    } else if constexpr (W == 2) {
-        *reinterpret_cast<float2 *>(p) = make_float2(x[0], x[1]);
-    } else {
-        *p = x[0];
-    }
-}
 
 // Take the next pack from the light items lt (a ballot over the warp's group;
 // v, beg, deg: the lane's own item): its vertices' arcs lie in the warp's lanes
@@ -405,22 +343,7 @@ __device__ __forceinline__ void bwd_light(unsigned lt, int v, int beg, int deg, 
 #pragma unroll
                 for (int t = 0; t < W; ++t) S[t] = TREE ? (S[t] + x[t]) + y[t] : S[t] + (x[t] + y[t]);
             }
-            float c[W];
-#pragma unroll
-            for (int t = 0; t < W; ++t) {
-                c[t] = 0.0f;
-                if ((mine >> t) & 1u) {
-                    float sg;
-                    if (sig_ones || Sl)
-                        sg = __uint2float_rn((cnt[t / 2] >> (16 * (t % 2))) & 0xFFFFu);
-                    else
-                        sg = sigma_f32(ldx<NC>(sigma + at + t));
-                    const float d = sg * S[t];              // delta_s(v) = sigma_s(v) * sum_w c_s(w)
-                    c[t] = __fdividef(1.0f, sg) + S[t];     // c_s(v) for the level above (1/sigma within 2 ulp)
-                    two_sum_add(hi, lo, d);
-                }
-            }
-            if (Cl && fw != 0u) stg_packed<W>(Cl + at, c);
+            finalize_packed<W, NC>(sigma, sig_ones || Sl != nullptr, cnt, Cl, fw, at, S, lane, hi, lo);
             L.acc[r][lane] = make_float2(hi, lo);
         }
         __syncwarp();

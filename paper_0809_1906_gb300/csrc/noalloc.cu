@@ -87,7 +87,7 @@ __global__ void k_noalloc_prepare(int32_t n, const int32_t *__restrict__ row_ptr
     for (int v = tid; v < n; v += stride) {
         const int a = row_ptr[v], b = row_ptr[v + 1];
         if (b < a) atomicOr(bad, 1u);
-        items[v] = make_int4(v, a, b, -1);  // no split vertices here
+        items[v] = make_int4(v, a, b, 0);
         item_v[v] = v;
         if (!sources) iota[v] = v;
     }
@@ -115,6 +115,8 @@ extern "C" int bc_run_noalloc(int32_t n, const int32_t *row_ptr, const int32_t *
     bcgb::MsParams p{};
     p.n = n;
     p.nitems = n;
+    p.light_least = 1;
+    p.nslots = 0;  // no split vertices
     p.nheavy = n;  // in vertex order: the light ones are not set apart
     p.nw32 = (n + 31) / 32;
     p.Lcap = kLcap;
