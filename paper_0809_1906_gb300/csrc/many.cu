@@ -5,7 +5,8 @@
 // decreasing cost (longest-processing-time first) and CTAs take them from an
 // atomic queue. A CTA runs its item's batches alone: the same per-vertex
 // forward and backward steps as the one-graph path (msbfs_body.cuh), with the
-// CTA's warps striding over vertices and __syncthreads between levels, so
+// CTA's warps striding over vertices (those of few arcs in packs,
+// msbfs_light.cuh) and __syncthreads between levels, so
 // no level ever waits on another CTA. Sources are the vertices in order,
 // B = 32*W per batch.
 //
@@ -26,10 +27,17 @@
 #include "bc_internal.cuh"
 #include "many.cuh"
 #include "msbfs_body.cuh"
+#include "msbfs_light.cuh"
 
 namespace bcgb {
 namespace {
 
+// Vertices of at most this many arcs run in packs (msbfs_light.cuh), the others
+// one warp each. These graphs have 6 to 8 arcs per vertex, and a CTA runs its
+// graph alone: one vertex at a time, a warp waited out every chain of loads.
+// 1000 graphs, n in [50, 5000], batch 256, whole pass with the reading of every
+// result: no packs 204 ms, up to 8 arcs 175, 16 145, 31 144.
+constexpr int kManyLightDeg = 16;
 constexpr int kMBlock = 256;
 constexpr int kMWarps = kMBlock / 32;
 constexpr unsigned kFull = 0xffffffffu;
@@ -42,8 +50,17 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
     __shared__ int32_t s_u[kMWarps][32];
     __shared__ uint32_t s_nz[kMWarps][32];
     __shared__ uint32_t s_w[kMWarps][32][W];  // per-lane words of a warp's 32 vertices
-    __shared__ unsigned long long s_sum[4][B];  // per-source summaries of the running batch
-    __shared__ __align__(16) uint64_t s_sig[kMWarps][W][32];  // counts of the vertex being finalized
+    // each warp's own scratch; between the sweeps (and block barriers) the
+    // batch's summaries
+    union WarpScratch {
+        uint64_t sig[W][32];  // counts of the vertex being finalized
+        body::LightScratch<W> light;
+    };
+    __shared__ __align__(16) union {
+        unsigned long long sum[4][B];  // per-source summaries of the running batch
+        WarpScratch warp[kMWarps];
+    } s_mem;
+    auto &s_sum = s_mem.sum;
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     uint64_t *sigma = p.sigma + (size_t)blockIdx.x * p.nmax * B;
     uint16_t *Sbuf = p.S + (size_t)blockIdx.x * 2 * p.nmax * B;
@@ -110,9 +127,12 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
                 // v0 + k * kMWarps), then works through the active ones
                 for (int v0 = wib; v0 < n; v0 += 32 * kMWarps) {
                     const int vk = v0 + lane * kMWarps;
-                    bool act = false;
+                    bool act = false, light = false;
+                    int bk = 0, ek = 0;
                     __syncwarp();  // the previous group's reads of s_w are done
                     if (vk < n) {
+                        bk = gd.row_ptr[vk];
+                        ek = gd.row_ptr[vk + 1];
                         uint32_t a[W], f[W];
                         body::load_row<W, false>(Vin + (size_t)vk * W, a);
                         body::load_row<W, false>(Fl + (size_t)vk * W, f);
@@ -125,12 +145,14 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
                             s_w[wib][lane][j] = u;
                             any |= u;
                         }
-                        act = any != 0u;
+                        act = any != 0u && bk < ek;
+                        light = act && ek - bk <= kManyLightDeg;
                         if (!act)
 #pragma unroll
                             for (int j = 0; j < W; ++j) Fn[(size_t)vk * W + j] = 0u;
                     }
-                    unsigned todo = __ballot_sync(kFull, act);
+                    unsigned todo = __ballot_sync(kFull, act && !light);
+                    const unsigned lt = __ballot_sync(kFull, light);
                     __syncwarp();
                     while (todo) {
                         const int v = v0 + (__ffs(todo) - 1) * kMWarps;
@@ -149,6 +171,10 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
                                                 s_u[wib], s_nz[wib], lane, acc, nf, ovf, arcs);
                         produced |= body::store_next<W, false>(sigma, Sn, Fn, ufn, v, acc, nf, lane, wide_next);
                     }
+                    if (lt)
+                        body::fwd_light<W, false>(lt, vk, bk, ek - bk, s_w[wib], s_mem.warp[wib].light, gd.col, ufl, Fl, Sl,
+                                                  sigma, wide, false, Sn, Fn, ufn, lane, ovf, arcs, produced, wide_next,
+                                                  nullptr);
                 }
                 wide = __syncthreads_or(wide_next);
                 if (!__syncthreads_or(produced)) {
@@ -200,6 +226,7 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
                     gd.dist_sum[s0 + b] = (int64_t)s_sum[2][b];
                     gd.reach[s0 + b] = (int64_t)s_sum[3][b];
                 }
+                __syncthreads();  // the warps' scratch takes the place of the sums
             }
             // backward levels (Theorem 1.1), BC into this item's target
             for (int l = L; l >= 1; --l) {
@@ -210,9 +237,12 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
                 const float *Cs = cval + (size_t)((l + 1) & 1) * nB;
                 for (int v0 = wib; v0 < n; v0 += 32 * kMWarps) {
                     const int vk = v0 + lane * kMWarps;
-                    bool act = false;
+                    bool act = false, light = false;
+                    int bk = 0, ek = 0;
                     __syncwarp();  // the previous group's reads of s_w are done
                     if (vk < n) {
+                        bk = gd.row_ptr[vk];
+                        ek = gd.row_ptr[vk + 1];
                         uint32_t f[W];
                         body::load_row<W, false>(Fl + (size_t)vk * W, f);
                         uint32_t any = 0;
@@ -222,9 +252,14 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
                             any |= f[j];
                         }
                         act = any != 0u;
+                        light = act && ek - bk <= kManyLightDeg;
                     }
-                    unsigned todo = __ballot_sync(kFull, act);
+                    unsigned todo = __ballot_sync(kFull, act && !light);
+                    const unsigned lt = __ballot_sync(kFull, light);
                     __syncwarp();
+                    if (lt)
+                        body::bwd_light<W, false, false>(lt, vk, bk, ek - bk, s_w[wib], s_mem.warp[wib].light, gd.col, ufs,
+                                                         Fs, Cs, sigma, nullptr, false, Cl, target, lane);
                     while (todo) {
                         const int v = v0 + (__ffs(todo) - 1) * kMWarps;
                         uint32_t f[W];
@@ -236,7 +271,7 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
 #pragma unroll
                         for (int j = 0; j < W; ++j)
                             if (f[j] != 0u) {
-                                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&s_sig[wib][j][lane]);
+                                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&s_mem.warp[wib].sig[j][lane]);
                                 asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst),
                                              "l"(sigma + (size_t)v * B + 32 * j + lane)
                                              : "memory");
@@ -248,8 +283,8 @@ __global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyPara
                         body::bwd_sum<W, false>(gd.col, gd.row_ptr[v], gd.row_ptr[v + 1], ufs, Fs, Cs, f, s_u[wib], s_nz[wib], lane, S);
                         asm volatile("cp.async.wait_group 0;" ::: "memory");
                         __syncwarp();
-                        body::finalize_dep<W>(Cl, target, v, f, S, lane, &s_sig[wib][0][0]);
-                        __syncwarp();  // the next vertex's copies overwrite s_sig
+                        body::finalize_dep<W>(Cl, target, v, f, S, lane, &s_mem.warp[wib].sig[0][0]);
+                        __syncwarp();  // the next vertex's copies overwrite sig
                     }
                 }
                 __syncthreads();

@@ -719,13 +719,13 @@ __device__ __forceinline__ void finalize_dep(float *Cl, double *bc, int v, const
 // W lane + t; fw: the frontier word that holds the lane's sources. The counts
 // come from cnt, the lane's entries of the level's masked uint16 row (a narrow
 // level; all 1 at level 1 from the sources directly), or with `narrow` false
-// from the uint64 array. Against the word view this needs no exchange of the
+// from the uint64 array or, when given, the lane's entries of it in raw. Against the word view this needs no exchange of the
 // sums between lanes, and one vector load and one or two vector stores per row
 // instead of W of each.
 template <int W, bool NC>
 __device__ __forceinline__ void finalize_packed(const uint64_t *sigma, bool narrow, const uint32_t (&cnt)[(W + 1) / 2],
                                                 float *Cl, uint32_t fw, size_t at, const float (&S)[W], int lane,
-                                                float &hi, float &lo) {
+                                                float &hi, float &lo, const uint64_t *raw = nullptr) {
     const uint32_t mine = fw >> ((W * lane) & 31);  // bits 0 .. W - 1: the lane's sources
     float c[W];
 #pragma unroll
@@ -733,7 +733,7 @@ __device__ __forceinline__ void finalize_packed(const uint64_t *sigma, bool narr
         c[t] = 0.0f;
         if ((mine >> t) & 1u) {
             const float sg = narrow ? __uint2float_rn((cnt[t / 2] >> (16 * (t % 2))) & 0xFFFFu)
-                                    : sigma_f32(ldx<NC>(sigma + at + t));
+                                    : sigma_f32(raw ? raw[t] : ldx<NC>(sigma + at + t));
             const float d = sg * S[t];           // delta_s(v) = sigma_s(v) * sum_w c_s(w)
             c[t] = __fdividef(1.0f, sg) + S[t];  // c_s(v) for the level above (1/sigma within 2 ulp)
             two_sum_add(hi, lo, d);

@@ -326,6 +326,25 @@ __device__ __forceinline__ void bwd_light(unsigned lt, int v, int beg, int deg, 
 #pragma unroll
             for (int t = 0; t < P; ++t) cnt[t] = 0x00010001u;  // level 1: every count is 1
             if (!sig_ones && Sl && fw != 0u) ldg_packed<W, NC>(Sl + at, cnt);
+            // the many-graph kernel keeps no narrow rows for the backward: its
+            // counts are on their way while the rows are added
+            uint64_t raw[W];
+            if constexpr (!TREE) {
+#pragma unroll
+                for (int t = 0; t < W; ++t) raw[t] = 1ull;
+                if (fw != 0u) {
+                    if constexpr (W >= 2) {
+#pragma unroll
+                        for (int t = 0; t < W; t += 2) {
+                            const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(sigma + at + t);
+                            raw[t] = x.x;
+                            raw[t + 1] = x.y;
+                        }
+                    } else {
+                        raw[0] = sigma[at];
+                    }
+                }
+            }
             float S[W];
 #pragma unroll
             for (int t = 0; t < W; ++t) S[t] = 0.0f;
@@ -343,7 +362,8 @@ __device__ __forceinline__ void bwd_light(unsigned lt, int v, int beg, int deg, 
 #pragma unroll
                 for (int t = 0; t < W; ++t) S[t] = TREE ? (S[t] + x[t]) + y[t] : S[t] + (x[t] + y[t]);
             }
-            finalize_packed<W, NC>(sigma, sig_ones || Sl != nullptr, cnt, Cl, fw, at, S, lane, hi, lo);
+            finalize_packed<W, NC>(sigma, TREE && (sig_ones || Sl != nullptr), cnt, Cl, fw, at, S, lane, hi, lo,
+                                   TREE ? nullptr : raw);
             L.acc[r][lane] = make_float2(hi, lo);
         }
         __syncwarp();

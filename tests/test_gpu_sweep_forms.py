@@ -122,3 +122,27 @@ def test_per_level_form_on_a_large_mesh(nat):
     g = G.grid_longrange(96, 0.05)
     g = G.Graph(g.n, g.row_ptr, g.col, None, "mesh96")
     check(nat, g, G.sample_sources(g.n, 700, 63))
+
+
+@pytest.mark.parametrize("batch", [32, 64, 128, 256])
+def test_many_graphs_around_the_pack_limit(nat, batch):
+    """The many-graph kernel's packs: degrees at their limit of 16 arcs, mixed
+    degrees, counts past 16 bits, an edgeless graph; BC and summaries per graph."""
+    gs = [circulant(90 + deg, deg) for deg in (1, 2, 8, 15, 16, 17, 34)]
+    gs += [G.barabasi_albert(300, 3, 64), G.grid_graph(16), G.csr_from_edges(40, [], []), G.star_graph(80),
+           G.random_small(257, 0.03, 6300, connect=False)]
+    hs = [nat.Graph.from_csr(g) for g in gs]
+    with nat.ManyPlan(hs, batch=batch) as plan:
+        for _ in range(2):
+            plan.run()
+            assert plan.result()[0] == nat.BC_OK
+        for g, h in zip(gs, hs):
+            ref = oracle.bc(g)
+            got, _, _ = h.result()
+            tol = np.maximum(1e-5 * np.abs(ref["bc"]), 1e-6 * g.n)
+            assert np.all(np.abs(got - ref["bc"]) <= tol), g.name
+            sums = h.source_hashes(g.n)
+            for name in HASHES:
+                assert np.array_equal(sums[name], ref[name]), (g.name, name)
+    for h in hs:
+        h.close()
