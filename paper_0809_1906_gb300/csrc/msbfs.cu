@@ -995,6 +995,9 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
         }
         if (!alive) break;
         if (lead) atomicAdd(&p.ctl->depth_sum, (unsigned long long)L);
+        // the summaries read what the forward pass left; the narrow deepest
+        // backward level follows without a barrier of their own
+        if (q.hash) hash_tiles<W, false, 6, 8>(p, L, bid, nblk, sh.hash);
         __syncthreads();
         if (tid == 0) {
             p.nitems = q.b_nitems;
@@ -1009,13 +1012,11 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
         ws.qz = sh.bwd.qz[wib];
         for (int l = L; alive && l >= 1; --l) {
             backward_items<W, false, false>(p, l, bid, nblk, sh.bwd, ws);
-            alive = group_barrier<W>(sync, nblk, round, sh);
+            if (l > 1) alive = group_barrier<W>(sync, nblk, round, sh);
         }
         if (!alive) break;
-        if (q.hash) {
-            hash_tiles<W, false, 6, 8>(p, L, bid, nblk, sh.hash);
-            if (!(alive = group_barrier<W>(sync, nblk, round, sh))) break;
-        }
+        // the group's next batch clears what this one still reads
+        if (bi + q.groups < q.nbat) alive = group_barrier<W>(sync, nblk, round, sh);
     }
     if (lane == 0 && ws.fail) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
     if (tid == 0 && !sh.ok && round > 0) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
