@@ -100,7 +100,7 @@ class ClockSampler:
 
 
 # Sources of the sweep kernels whose DRAM bytes profiles/traffic_rmat.json holds.
-SWEEP_SOURCES = ("msbfs.cu", "msbfs_body.cuh", "rowstage.cuh", "pdl.cuh", "bc_internal.cuh")
+SWEEP_SOURCES = ("msbfs.cu", "msbfs_body.cuh", "msbfs_light.cuh", "rowstage.cuh", "pdl.cuh", "bc_internal.cuh")
 
 
 def code_text(text: str) -> str:
