@@ -36,14 +36,21 @@ namespace {
 // one warp each. These graphs have 6 to 8 arcs per vertex, and a CTA runs its
 // graph alone: one vertex at a time, a warp waited out every chain of loads.
 // 1000 graphs, n in [50, 5000], batch 256, whole pass with the reading of every
-// result: no packs 204 ms, up to 8 arcs 175, 16 145, 31 144.
+// result (256 threads, three CTAs per SM): no packs 204 ms, up to 8 arcs 175, 16 145,
+// 31 144.
 constexpr int kManyLightDeg = 16;
-constexpr int kMBlock = 256;
+// A CTA runs one batch of a graph at a time, so its latency is the unit in which
+// the set's work is spread over the chip: two CTAs of twelve warps per SM finish
+// a batch sooner than three of eight, with fewer batch states competing for L2.
+// Kernel time of 256 x 3 / 384 x 2 / 768 x 1 per SM: 1000 graphs up to 5000
+// vertices 120.9 / 120.3 / 120.2 ms, 250 up to 1500 7.60 / 5.31 / 4.55, 300 up
+// to 400 (batch 64) 0.79 / 0.63 / 0.67: 384, the one that small sets like too.
+constexpr int kMBlock = 384;
 constexpr int kMWarps = kMBlock / 32;
 constexpr unsigned kFull = 0xffffffffu;
 
 template <int W>
-__global__ void __launch_bounds__(kMBlock, W >= 4 ? 3 : 4) k_many(const ManyParams p) {
+__global__ void __launch_bounds__(kMBlock, 2) k_many(const ManyParams p) {
     constexpr int B = 32 * W;
     __shared__ int s_item;
     __shared__ int s_last;
