@@ -40,12 +40,13 @@ namespace {
 // 31 144.
 constexpr int kManyLightDeg = 16;
 // A CTA runs one batch of a graph at a time, so its latency is the unit in which
-// the set's work is spread over the chip: two CTAs of twelve warps per SM finish
+// the set's work is spread over the chip: two CTAs of 12 to 14 warps per SM finish
 // a batch sooner than three of eight, with fewer batch states competing for L2.
 // Kernel time of 256 x 3 / 384 x 2 / 768 x 1 per SM: 1000 graphs up to 5000
 // vertices 120.9 / 120.3 / 120.2 ms, 250 up to 1500 7.60 / 5.31 / 4.55, 300 up
-// to 400 (batch 64) 0.79 / 0.63 / 0.67: 384, the one that small sets like too.
-constexpr int kMBlock = 384;
+// to 400 (batch 64) 0.79 / 0.63 / 0.67. At two per SM, 384 / 448 / 512 threads (80, 72,
+// 64 registers): 119.0 / 110.5 / 112.6, 5.25 / 4.88 / 4.98, 0.63 / 0.61 / 0.59 ms: 448.
+constexpr int kMBlock = 448;
 constexpr int kMWarps = kMBlock / 32;
 constexpr unsigned kFull = 0xffffffffu;
 
