@@ -237,8 +237,10 @@ int bc_source_hashes(bc_graph *g, uint64_t *h_sigma, uint64_t *h_dist, int64_t *
  *   sources  int32[k] (host or device), 0 <= k.
  *   sigma    uint64[k*n] (host or device): row i = sigma_{sources[i]}(.), 0 where unreachable.
  *   dist     int32[k*n] (host or device): d(sources[i], .), -1 where unreachable.
- * Either output may be NULL. Synchronises cuda_stream. Returns BC_OK or
- * BC_WARN_SIGMA_OVERFLOW, or an error.
+ * Either output may be NULL; one in this device's memory is written in place.
+ * Synchronises cuda_stream, and with it the internal streams, also when it
+ * fails: nothing writes to the outputs after the call. Returns BC_OK or
+ * BC_WARN_SIGMA_OVERFLOW, or an error (the outputs then hold parts of the rows).
  */
 int bc_forward_rows(bc_graph *g, const int32_t *sources, int32_t k, uint64_t *sigma, int32_t *dist,
                     const bc_options *opt, void *cuda_stream);

@@ -1289,7 +1289,38 @@ int first_level_top_down(const bc_graph *g, const int32_t *src_host, int32_t nb,
     return (double)arcs * (double)g->alpha < (double)g->narcs ? 1 : 0;
 }
 
-// The multi-source driver shared by bc_run and bc_forward_rows.
+// Joins the internal streams of a call into st, also when the call fails:
+// whatever they still run (rows into the caller's memory, a lane's state) then
+// ends before anything enqueued on st later, and before a wait for st returns.
+struct StreamJoin {
+    cudaStream_t st;
+    int count = 0;
+    cudaStream_t stream[kSweepLanes] = {};
+    cudaEvent_t event[kSweepLanes] = {};
+    explicit StreamJoin(cudaStream_t s) : st(s) {}
+    void add(cudaStream_t s, cudaEvent_t e) {
+        stream[count] = s;
+        event[count++] = e;
+    }
+    cudaError_t join() {
+        cudaError_t r = cudaSuccess;
+        for (int k = 0; k < count; ++k) {
+            cudaError_t e = cudaEventRecord(event[k], stream[k]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, event[k], 0);
+            if (r == cudaSuccess) r = e;
+        }
+        count = 0;
+        return r;
+    }
+    ~StreamJoin() { join(); }
+    StreamJoin(const StreamJoin &) = delete;
+    StreamJoin &operator=(const StreamJoin &) = delete;
+};
+
+// Lanes from which the light vertices run in full packs: the other batches
+// then fill the warps that this one leaves.
+constexpr int kFullPackLanes = 4;
+
 // Concurrent sweep over K lanes (K >= 2). Batch i runs on lane i % K, each
 // lane on its own stream with its own batch state and BC accumulator, so the
 // narrow, latency-bound levels of one batch overlap the wide levels of
@@ -1299,10 +1330,6 @@ int first_level_top_down(const bc_graph *g, const int32_t *src_host, int32_t nb,
 // 1..K-1 into the graph's BC in lane order, so the result is the same on
 // every run. A batch deeper than the level capacity stops every lane: the
 // capacity is doubled and each lane's unfinished batch starts over.
-// Lanes from which the light vertices run in full packs: the other batches
-// then fill the warps that this one leaves.
-constexpr int kFullPackLanes = 4;
-
 int run_lanes(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool backward, bool hash,
               uint64_t *rows_sig, int32_t *rows_dist, int64_t wait_ms) {
     const int B = 32 * W;
@@ -1314,8 +1341,10 @@ int run_lanes(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool bac
     }
     if (!g->ev0) CK(cudaEventCreateWithFlags(&g->ev0, cudaEventDisableTiming));
     CK(cudaEventRecord(g->ev0, st));
+    StreamJoin join(st);
     for (int k = 1; k < K; ++k) {
         SweepLane &ln = g->lanes[k - 1];
+        join.add(ln.st, ln.ev);
         CK(cudaStreamWaitEvent(ln.st, g->ev0, 0));
         CK(cudaMemsetAsync(ln.bc.p, 0, (size_t)g->n * sizeof(double), ln.st));
         CK(cudaMemsetAsync(ln.ctl, 0, sizeof(bcgb::DevCtl), ln.st));
@@ -1444,11 +1473,7 @@ int run_lanes(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool bac
         }
     }
     // join: st waits for every lane, then adds their BC and counters in lane order
-    for (int k = 1; k < K; ++k) {
-        SweepLane &ln = g->lanes[k - 1];
-        CK(cudaEventRecord(ln.ev, ln.st));
-        CK(cudaStreamWaitEvent(st, ln.ev, 0));
-    }
+    CK(join.join());
     for (int k = 1; k < K; ++k) {
         SweepLane &ln = g->lanes[k - 1];
         bcgb::ms_launch_merge(ln.bc.p, g->bc.p, g->n, ln.ctl, g->ctl, st);
@@ -1845,6 +1870,7 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
     const int32_t *srcs = relabel ? g->wpsrc.p : g->sources.p;
     if (lanes > 1 && !g->wev) CK(cudaEventCreateWithFlags(&g->wev, cudaEventDisableTiming));
     if (lanes > 1) CK(cudaEventRecord(g->wev, st));
+    StreamJoin join(st);
     for (int k = 1; k < lanes; ++k) {
         auto &l = g->wl[k - 1];
         if (!l.st) {
@@ -1857,6 +1883,7 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
         CK(l.rows.ensure((size_t)G * n));
         CK(l.ds.ensure((size_t)G * n));
         CK(l.bc.ensure((size_t)std::max(n, 1)));
+        join.add(l.st, l.ev);
         CK(cudaStreamWaitEvent(l.st, g->wev, 0));
         CK(cudaMemsetAsync(l.bc.p, 0, (size_t)std::max(n, 1) * sizeof(double), l.st));
     }
@@ -1919,11 +1946,7 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
         }
         CK(cudaGetLastError());
     }
-    for (int k = 1; k < lanes; ++k) {
-        auto &l = g->wl[k - 1];
-        CK(cudaEventRecord(l.ev, l.st));
-        CK(cudaStreamWaitEvent(st, l.ev, 0));
-    }
+    CK(join.join());
     for (int k = 1; k < lanes && backward; ++k) bcgb::ms_launch_merge(g->wl[k - 1].bc.p, g->bc.p, n, nullptr, nullptr, st);
     // sources whose path counts need 64 bits: again with the 64-bit kernel
     std::vector<uint8_t> redo((size_t)std::max(nsrc, 1));

@@ -1,0 +1,71 @@
+"""What a call leaves behind when it fails, and what the next one then gives:
+waits that run out, on the host and on the device, by limits that the caller
+sets. Nothing here faults or hangs the GPU; every wait is bounded."""
+import ctypes
+import time
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_0809_1906_gb300 import graphs as G
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nat():
+    from paper_0809_1906_gb300 import native
+    native.load()
+    return native
+
+
+def close(got, ref, n):
+    return np.all(np.abs(got - ref) <= np.maximum(1e-5 * np.abs(ref), 1e-6 * n))
+
+
+def ring_with_chords(n, chords, seed):
+    """A ring and random chords: connected, shallow, quick to build."""
+    rng = np.random.default_rng(seed)
+    u, v = rng.integers(0, n, chords), rng.integers(0, n, chords)
+    at = np.arange(n)
+    u, v = np.concatenate([at, u]), np.concatenate([(at + 1) % n, v])
+    keep = u != v
+    key = np.unique(np.minimum(u, v)[keep] * n + np.maximum(u, v)[keep])
+    return key // n, key % n
+
+
+def test_rows_left_unwritten_after_a_failed_call(nat):
+    """Rows go straight into the caller's device memory, from several internal
+    streams. A call whose host wait runs out (1 ms, on levels that take
+    several) must have ended on all of them when it returns: the caller may
+    free or refill the buffers. 256 sources in a small component keep the
+    caller's own stream short, so that a wait for it alone would not do."""
+    import torch
+    n, small = 1_000_000, 300
+    u, v = ring_with_chords(n - small, 4_000_000, 5)
+    ring = np.arange(small)
+    g = G.csr_from_edges(n, np.concatenate([u, n - small + ring]), np.concatenate([v, n - small + (ring + 1) % small]),
+                         name="two")
+    src = np.concatenate([n - small + np.arange(256), np.arange(256)]).astype(np.int32)
+    sig = torch.zeros((512, n), dtype=torch.int64, device="cuda")
+    dist = torch.zeros((512, n), dtype=torch.int32, device="cuda")
+    with nat.Graph.from_csr(g, trust_input=True) as h:
+        opt = nat.make_options(256, 0, 0, 1)
+        torch.cuda.synchronize()
+        code = h.lib.bc_forward_rows(h.handle, nat._addr(src), len(src), nat._addr(sig), nat._addr(dist),
+                                     ctypes.byref(opt), nat._stream_ptr(None))
+        t0 = time.perf_counter()
+        torch.cuda.synchronize()
+        left = time.perf_counter() - t0
+        assert code == nat.BC_ERR_TIMEOUT
+        # an idle device answers in tens of microseconds; the levels in flight take milliseconds
+        assert left < 5e-4, left
+        opt = nat.make_options(256)
+        code = h.lib.bc_forward_rows(h.handle, nat._addr(src), len(src), nat._addr(sig), nat._addr(dist),
+                                     ctypes.byref(opt), nat._stream_ptr(None))
+        assert code == nat.BC_OK
+    for i in (0, 255, 256, 511):
+        o = oracle.source(g, int(src[i]), with_delta=False)
+        assert np.array_equal(sig[i].cpu().numpy().view(np.uint64), o["sigma"])
+        assert np.array_equal(dist[i].cpu().numpy(), o["dist"].astype(np.int32))
