@@ -2650,6 +2650,8 @@ struct bc_many {
     int W = 1, grid = 0, Lcap = 64;
     bool hash = true;  // per-source summaries into each graph's handle
     int32_t nitems = 0;
+    std::vector<bcgb::ManyGraph> h_graphs;  // what d_graphs holds, once no longer stale
+    bool table_stale = false;
     DevBuf<bcgb::ManyGraph> d_graphs;
     DevBuf<bcgb::ManyItem> d_items;
     DevBuf<unsigned> queue, arrive, capped;
@@ -2687,6 +2689,27 @@ void free_many(bc_many *m) {
     delete m;
 }
 
+// Points the plan at its handles' summaries. A handle's own run with more
+// sources than vertices moves them, so every run of the plan looks again.
+int place_summaries(bc_many *m) {
+    if (!m->hash) return BC_OK;
+    for (size_t i = 0; i < m->graphs.size(); ++i) {
+        bc_graph *g = m->graphs[i];
+        bcgb::ManyGraph &d = m->h_graphs[i];
+        if (g->n == 0) continue;
+        const int r = ensure_summaries(g, (size_t)g->n);
+        if (r) return r;
+        // one block, rows a row's length apart: the first and last pointers tell
+        if (d.h_sigma == g->h_sigma.p && d.reach == g->reach.p) continue;
+        d.h_sigma = g->h_sigma.p;
+        d.h_dist = g->h_dist.p;
+        d.dist_sum = g->dist_sum.p;
+        d.reach = g->reach.p;
+        m->table_stale = true;
+    }
+    return BC_OK;
+}
+
 // Work items of the many-graph launch: each graph's source batches, split
 // into several items when one graph alone is more than an eighth of a CTA's
 // fair share of the total, then sorted by decreasing cost (LPT). The cost is a
@@ -2717,7 +2740,8 @@ int build_many(bc_many *m) {
         double cost;
     };
     std::vector<Item> items;
-    std::vector<bcgb::ManyGraph> gd(m->graphs.size());
+    std::vector<bcgb::ManyGraph> &gd = m->h_graphs;
+    gd.resize(m->graphs.size());
     int64_t part_off = 0;
     for (size_t i = 0; i < m->graphs.size(); ++i) {
         const bc_graph *g = m->graphs[i];
@@ -2732,15 +2756,6 @@ int build_many(bc_many *m) {
         gd[i].bc = g->bc.p;
         gd[i].h_sigma = gd[i].h_dist = nullptr;
         gd[i].dist_sum = gd[i].reach = nullptr;
-        if (m->hash && g->n > 0) {
-            bc_graph *gw = m->graphs[i];
-            const int rs = ensure_summaries(gw, (size_t)g->n);
-            if (rs) return rs;
-            gd[i].h_sigma = gw->h_sigma.p;
-            gd[i].h_dist = gw->h_dist.p;
-            gd[i].dist_sum = gw->dist_sum.p;
-            gd[i].reach = gw->reach.p;
-        }
         if (q > 1) part_off += (int64_t)q * g->n;
         for (int k = 0; k < q; ++k) {
             Item x;
@@ -2752,6 +2767,8 @@ int build_many(bc_many *m) {
             items.push_back(x);
         }
     }
+    const int rs = place_summaries(m);
+    if (rs) return rs;
     std::stable_sort(items.begin(), items.end(), [](const Item &a, const Item &b) { return a.cost > b.cost; });
     std::vector<bcgb::ManyItem> hit(items.size());
     for (size_t i = 0; i < items.size(); ++i) hit[i] = items[i].it;
@@ -2761,6 +2778,7 @@ int build_many(bc_many *m) {
     const size_t G = (size_t)m->grid;
     CK(m->d_graphs.ensure(gd.size()));
     CK(cudaMemcpy(m->d_graphs.p, gd.data(), gd.size() * sizeof(gd[0]), cudaMemcpyHostToDevice));
+    m->table_stale = false;
     CK(m->d_items.ensure(hit.size()));
     if (!hit.empty()) CK(cudaMemcpy(m->d_items.p, hit.data(), hit.size() * sizeof(hit[0]), cudaMemcpyHostToDevice));
     CK(m->queue.ensure(1));
@@ -2850,6 +2868,14 @@ int bc_many_run(bc_many *m, void *cuda_stream) {
     g_err.clear();
     if (!m) return fail(BC_ERR_ARG, "plan is NULL");
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    const int rs = place_summaries(m);
+    if (rs) return rs;
+    if (m->table_stale) {
+        if (m->ran) CK(cudaStreamSynchronize(m->last_stream));  // a replay in flight reads the table
+        CK(cudaMemcpy(m->d_graphs.p, m->h_graphs.data(), m->h_graphs.size() * sizeof(m->h_graphs[0]),
+                      cudaMemcpyHostToDevice));
+        m->table_stale = false;
+    }
     if (m->exec) CK(cudaGraphLaunch(m->exec, st));
     for (bc_graph *g : m->graphs) {
         g->has_run = true;

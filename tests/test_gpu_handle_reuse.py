@@ -1,0 +1,50 @@
+"""Handles used by several kinds of calls in turn: what one call leaves in a
+handle must not be taken for another's, nor a plan write where a handle's
+results no longer are."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_0809_1906_gb300 import graphs as G
+
+pytestmark = pytest.mark.gpu
+
+HASHES = ("hash_sigma", "hash_dist", "dist_sum", "reach")
+
+
+@pytest.fixture(scope="module")
+def nat():
+    from paper_0809_1906_gb300 import native
+    native.load()
+    return native
+
+
+def close(got, ref, n):
+    return np.all(np.abs(got - ref) <= np.maximum(1e-5 * np.abs(ref), 1e-6 * n))
+
+
+def test_plan_follows_its_handles_summaries(nat):
+    """A run of one handle with three sources per vertex (repeats are allowed)
+    needs longer summaries and moves them; the plan's next run writes to where
+    they are now."""
+    gs = [G.er_hamiltonian(120, 300, 71), G.barabasi_albert(90, 3, 72), G.csr_from_edges(30, [], [])]
+    refs = [oracle.bc(g) for g in gs]
+    hs = [nat.Graph.from_csr(g) for g in gs]
+    with nat.ManyPlan(hs, batch=64) as plan:
+        for rep in range(3):
+            plan.run()
+            assert plan.result()[0] == nat.BC_OK
+            for g, h, ref in zip(gs, hs, refs):
+                got, _, _ = h.result()
+                assert close(got, ref["bc"], g.n), (rep, g.name)
+                sums = h.source_hashes(g.n)
+                for name in HASHES:
+                    assert np.array_equal(sums[name], ref[name]), (rep, g.name, name)
+            g, h = gs[rep], hs[rep]
+            src = np.tile(np.arange(g.n, dtype=np.int32), 3)
+            h.run(src)
+            sums = h.source_hashes(len(src))
+            for name in HASHES:
+                assert np.array_equal(sums[name], np.tile(refs[rep][name], 3)), (rep, name)
+    for h in hs:
+        h.close()
