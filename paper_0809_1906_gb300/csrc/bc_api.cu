@@ -379,7 +379,6 @@ struct bc_graph {
 
     // the one-launch sweep: group 0's BC sums (its barrier words follow the control block)
     DevBuf<double> sweep_bc;
-    bool clear_pending = false;  // clear_outputs has still to run
     // ctl->status as last read from the device, current while status_known
     uint32_t status = 0;
     bool status_known = false;
@@ -826,8 +825,6 @@ int ensure_summaries(bc_graph *g, size_t k) {
 // What a run adds to, set to zero: BC (unless the run accumulates) and the
 // summaries of its sources. The one-launch sweep clears its own.
 int clear_outputs(bc_graph *g, int32_t nsrc, bool hash, cudaStream_t st) {
-    if (!g->clear_pending) return BC_OK;
-    g->clear_pending = false;
     if (!(g->last_opt.flags & BC_ACCUMULATE)) CK(cudaMemsetAsync(g->bc.p, 0, g->bc.n * sizeof(double), st));
     if (hash && nsrc)
         CK(cudaMemset2DAsync(g->summ.p, g->summ_row * sizeof(uint64_t), 0, (size_t)nsrc * sizeof(uint64_t), 4, st));
@@ -1574,7 +1571,6 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
             Timer t(g, st, BC_KERNEL_INIT);
             bcgb::ms_launch_sweep_merge(q, g->bc.p, n, (g->last_opt.flags & BC_ACCUMULATE) != 0, st);
             CK(cudaGetLastError());
-            g->clear_pending = false;
             g->status = (uint32_t)status;
             g->status_known = true;
             return BC_OK;
@@ -1587,12 +1583,15 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
     }
 }
 
+// The multi-source driver shared by bc_run and bc_forward_rows. With backward
+// the handle's BC and summaries are cleared here, by whichever form runs;
+// without, they are the caller's business.
 int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStream_t st, bool backward,
                 bool hash, uint64_t *rows_sig, int32_t *rows_dist) {
     const int64_t wait_ms = (opt && opt->wait_limit_ms > 0) ? opt->wait_limit_ms : 600000;
     if (opt && (opt->flags & BC_DENSE)) {
         int rd = ensure_dense(g, st);
-        if (!rd) rd = clear_outputs(g, nsrc, hash, st);
+        if (!rd && backward) rd = clear_outputs(g, nsrc, hash, st);
         if (rd) return rd;
         return run_dense_group(g, nsrc, opt, st, backward, hash, rows_sig, rows_dist);
     }
@@ -1613,7 +1612,7 @@ int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStr
         const bool sweep = backward && !rows_sig && !rows_dist && !g->timing && g->dev_wait_ns == 0 && g->test_hold == 0 &&
                            nsrc > 0 && one_launch(g, W, K);
         if (sweep) return run_sweep(g, nsrc, W, K, st, hash, wait_ms);
-        r = clear_outputs(g, nsrc, hash, st);
+        if (backward) r = clear_outputs(g, nsrc, hash, st);
         if (r) return r;
         if (K > 1) return run_lanes(g, nsrc, W, K, st, backward, hash, rows_sig, rows_dist, wait_ms);
     }
@@ -2275,7 +2274,6 @@ int bc_run(bc_graph *g, const int32_t *sources, int32_t num_sources, const bc_op
         r = ensure_summaries(g, (size_t)nsrc);
         if (r) return r;
     }
-    g->clear_pending = true;
     if (g->weighted || (flags & (BC_PLAIN | BC_PAIRS))) {
         r = clear_outputs(g, nsrc, hash, st);
         if (r) return r;

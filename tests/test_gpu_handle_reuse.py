@@ -48,3 +48,28 @@ def test_plan_follows_its_handles_summaries(nat):
                 assert np.array_equal(sums[name], np.tile(refs[rep][name], 3)), (rep, name)
     for h in hs:
         h.close()
+
+
+def test_result_survives_rows_after_a_failed_run(nat):
+    """A run that fails before it cleared the handle's BC leaves nothing to be
+    cleared later: rows asked of the handle after a plan has given it its result
+    leave that result alone."""
+    import torch
+    g = G.er_hamiltonian(400, 1600, 73)
+    ref = oracle.bc(g)
+    with nat.Graph.from_csr(g) as h:
+        stream = torch.cuda.Stream()
+        h.run(flags=nat.BC_KEEP_ORDER, stream=stream)  # state and sources in place: the next run only waits
+        h.result()
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(100_000_000)  # some 50 ms: the run's own work starts after it
+        with pytest.raises(nat.BcError) as e:
+            h.run(flags=nat.BC_KEEP_ORDER, wait_limit_ms=1, stream=stream)
+        assert e.value.code == nat.BC_ERR_TIMEOUT
+        torch.cuda.synchronize()
+        with nat.ManyPlan([h], batch=64) as plan:
+            plan.run()
+            assert plan.result()[0] == nat.BC_OK
+            h.forward_rows(np.arange(3, dtype=np.int32), batch=64)
+            got, _, _ = h.result()
+            assert close(got, ref["bc"], g.n)
