@@ -123,6 +123,11 @@ extern "C" {
    land, stops staging, and bc_result returns BC_ERR_TIMEOUT. Nothing faults
    or hangs: the wait is bounded and the context stays usable. */
 #define BC_TEST_WAIT_EXPIRY 0x200u
+/* The same for the one-launch form of small unweighted runs: every barrier
+   between its levels also expects one arrival that nobody makes, so its bounded
+   wait (10 s; with this flag, bc_options.device_wait_us if set) runs out, the
+   launch ends by itself and bc_result returns BC_ERR_TIMEOUT. */
+#define BC_TEST_BARRIER_EXPIRY 0x800u
 #define BC_FORCE_BOTTOMUP 0x400u /* level 0 -> 1 also by the bottom-up pull over every vertex instead of
                                     the top-down push from the sources' arcs */
 

@@ -315,6 +315,7 @@ struct bc_graph {
     float alpha = 1.0f, beta = 1.0f / 64.0f;
     uint64_t dev_wait_ns = 0;  // bound on each device wait (0: the kernels' default)
     uint32_t test_hold = 0;    // BC_TEST_WAIT_EXPIRY
+    bool test_barrier = false;  // BC_TEST_BARRIER_EXPIRY
     bool bottom_up0 = false;   // BC_FORCE_BOTTOMUP: level 0 -> 1 pulled too
     // options bc_run uses when given NULL (bc_autotune / bc_set_default_options)
     bool has_defaults = false;
@@ -379,6 +380,7 @@ struct bc_graph {
 
     // the one-launch sweep: group 0's BC sums (its barrier words follow the control block)
     DevBuf<double> sweep_bc;
+    bool counters_unsure = false;  // a sweep whose status nobody has read: it may have given up
     // ctl->status as last read from the device, current while status_known
     uint32_t status = 0;
     bool status_known = false;
@@ -798,6 +800,7 @@ void set_run_options(bc_graph *g, const bc_options *opt) {
     g->beta = (opt && opt->beta > 0.0f) ? std::min(opt->beta, 1.0f) : 1.0f / 64.0f;
     g->dev_wait_ns = (opt && opt->device_wait_us > 0) ? (uint64_t)opt->device_wait_us * 1000ull : 0ull;
     g->test_hold = (opt && (opt->flags & BC_TEST_WAIT_EXPIRY)) ? 16u : 0u;
+    g->test_barrier = opt && (opt->flags & BC_TEST_BARRIER_EXPIRY);
     g->bottom_up0 = opt && (opt->flags & BC_FORCE_BOTTOMUP);
 }
 
@@ -1498,6 +1501,12 @@ bool one_launch(const bc_graph *g, int W, int K) {
     return std::max(units(g->fplan), units(g->bplan)) <= 8 * kSweepUnits * warps;
 }
 
+// Bound on each wait at a barrier of the one-launch sweep. Such a wait lasts as
+// long as the slowest block's level, not a copy's microseconds, so
+// bc_options.device_wait_us does not apply to it: a run that sets that bound
+// takes the launch-per-level form, whose only device waits are for copies.
+constexpr uint64_t kBarrierWaitNs = 10000000000ull;
+
 // Batches of a run as one cooperative launch (k_sweep): group k takes batches
 // k, k + K, ... with lane k's state and its own BC sums, added in group order at
 // the end. A batch deeper than the level capacity ends the launch; the capacity
@@ -1524,6 +1533,8 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
         q.first_rule = g->bottom_up0 ? 0 : g->directed ? 1 : 2;
         q.alpha = g->alpha;
         q.seq = ++g->seq;
+        q.barrier_ns = g->test_barrier && g->dev_wait_ns ? g->dev_wait_ns : kBarrierWaitNs;
+        q.barrier_absent = g->test_barrier ? 1u : 0u;
         q.narcs = g->narcs;
         q.sources = g->sources.p;
         q.out_index = g->reordered ? g->src_index.p : nullptr;
@@ -1548,6 +1559,7 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
             q.g[k].hctl = g->hctl_d;
             if (k == 0) q.g[k].bc = g->sweep_bc.p;
         }
+        g->counters_unsure = true;
         {
             Timer t(g, st, BC_KERNEL_FORWARD);
             CK(bcgb::ms_launch_sweep(W, q, st));
@@ -1567,12 +1579,14 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
                 return fail(BC_ERR_STATE, "the sweep ended without reporting its status");
             if (spins % 65536 == 65535) std::this_thread::yield();
         }
-        if (!((uint32_t)status & BC_STATUS_LEVEL_CAP)) {
+        // (a launch that gave up is not tried again: bc_result reports it)
+        if (!((uint32_t)status & BC_STATUS_LEVEL_CAP) || ((uint32_t)status & BC_STATUS_COPY_TIMEOUT)) {
             Timer t(g, st, BC_KERNEL_INIT);
             bcgb::ms_launch_sweep_merge(q, g->bc.p, n, (g->last_opt.flags & BC_ACCUMULATE) != 0, st);
             CK(cudaGetLastError());
             g->status = (uint32_t)status;
             g->status_known = true;
+            g->counters_unsure = ((uint32_t)status & BC_STATUS_COPY_TIMEOUT) != 0;
             return BC_OK;
         }
         CK(cudaStreamSynchronize(st));
@@ -1583,6 +1597,17 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
     }
 }
 
+// Before level kernels of their own: the arrival counters of split vertices,
+// which the level kernels leave at zero and a sweep that gave up may not have.
+int reset_counters(bc_graph *g, cudaStream_t st) {
+    if (!g->counters_unsure) return BC_OK;
+    if (g->cnt.p) CK(cudaMemsetAsync(g->cnt.p, 0, g->cnt.n * sizeof(uint32_t), st));
+    for (auto &ln : g->lanes)
+        if (ln.cnt.p) CK(cudaMemsetAsync(ln.cnt.p, 0, ln.cnt.n * sizeof(uint32_t), st));
+    g->counters_unsure = false;
+    return BC_OK;
+}
+
 // The multi-source driver shared by bc_run and bc_forward_rows. With backward
 // the handle's BC and summaries are cleared here, by whichever form runs;
 // without, they are the caller's business.
@@ -1591,6 +1616,7 @@ int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStr
     const int64_t wait_ms = (opt && opt->wait_limit_ms > 0) ? opt->wait_limit_ms : 600000;
     if (opt && (opt->flags & BC_DENSE)) {
         int rd = ensure_dense(g, st);
+        if (!rd) rd = reset_counters(g, st);
         if (!rd && backward) rd = clear_outputs(g, nsrc, hash, st);
         if (rd) return rd;
         return run_dense_group(g, nsrc, opt, st, backward, hash, rows_sig, rows_dist);
@@ -1609,10 +1635,11 @@ int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStr
                                   (double)g->s_levels * std::max(g->n, 1) * B * 2.0;
         int K = g->timing ? 1 : std::min<int32_t>(kSweepLanes, nbat);
         while (K > 1 && (K - 1) * lane_bytes > kLaneBudgetBytes) --K;
-        const bool sweep = backward && !rows_sig && !rows_dist && !g->timing && g->dev_wait_ns == 0 && g->test_hold == 0 &&
-                           nsrc > 0 && one_launch(g, W, K);
+        const bool sweep = backward && !rows_sig && !rows_dist && !g->timing &&
+                           (g->dev_wait_ns == 0 || g->test_barrier) && g->test_hold == 0 && nsrc > 0 && one_launch(g, W, K);
         if (sweep) return run_sweep(g, nsrc, W, K, st, hash, wait_ms);
-        if (backward) r = clear_outputs(g, nsrc, hash, st);
+        r = reset_counters(g, st);
+        if (!r && backward) r = clear_outputs(g, nsrc, hash, st);
         if (r) return r;
         if (K > 1) return run_lanes(g, nsrc, W, K, st, backward, hash, rows_sig, rows_dist, wait_ms);
     }
@@ -2302,7 +2329,7 @@ int bc_run(bc_graph *g, const int32_t *sources, int32_t num_sources, const bc_op
     }
     if (flags & BC_HALVE) {
         Timer t(g, st, BC_KERNEL_HASH);
-        bcgb::launch_scale(g->bc.p, g->n, 0.5, st);
+        bcgb::launch_scale(g->bc.p, g->n, 0.5, g->ctl, st);
     }
     CK(cudaGetLastError());
     g->last_nsrc = nsrc;

@@ -146,13 +146,15 @@ struct SweepParams {
     int32_t b_nitems, b_nheavy, b_nslots;
     const int4 *b_items;
     const int32_t *b_item_v, *b_slot_first, *b_slot_nch;
+    uint64_t barrier_ns;      // bound on each wait at a group's barrier
+    uint32_t barrier_absent;  // arrivals that every barrier expects and none makes (the test hook; else 0)
     void *sync;          // kSweepSyncBytes bytes, zero at launch
     unsigned *finished;  // zero at launch
     MsParams g[kSweepGroups];
 };
 int ms_sweep_blocks(int W);  // blocks resident on the device at once (0: error)
 cudaError_t ms_launch_sweep(int W, const SweepParams &q, cudaStream_t st);
-// bc = the groups' sums (add: += them)
+// bc = the groups' sums (add: += them); nothing once a wait of the sweep gave up
 void ms_launch_sweep_merge(const SweepParams &q, double *bc, int32_t n, bool add, cudaStream_t st);
 
 // Launchers (msbfs.cu). W = words per vertex row (B = 32 W).
@@ -164,7 +166,7 @@ void ms_launch_backward(int W, const MsParams &p, int level, cudaStream_t st);
 void ms_launch_hash(int W, const MsParams &p, int nlevels, cudaStream_t st);
 void ms_launch_rows(int W, const MsParams &p, int nlevels, uint64_t *sig_out, int32_t *dist_out,
                     cudaStream_t st);
-void launch_scale(double *x, int32_t n, double f, cudaStream_t st);
+void launch_scale(double *x, int32_t n, double f, const DevCtl *ctl, cudaStream_t st);
 // dst[i] += src[i] for i < n; unless from is null, to's status |= from's and
 // its arc and depth sums += from's
 void ms_launch_merge(const double *src, double *dst, int32_t n, const DevCtl *from, DevCtl *to, cudaStream_t st);

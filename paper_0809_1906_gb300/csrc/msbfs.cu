@@ -827,15 +827,13 @@ __global__ void __launch_bounds__(kRowBlock) k_rows(const MsParams p, const int 
 // form) and runs all their levels itself, its blocks meeting at a barrier in
 // global memory after every level. The launch is cooperative, so every block
 // of a group is resident and the barrier cannot starve; its waits are bounded
-// all the same (kSweepWaitNs, then BC_STATUS_COPY_TIMEOUT, which the host
-// reports as a timeout).
+// all the same (SweepParams::barrier_ns, then BC_STATUS_COPY_TIMEOUT, which the
+// host reports as a timeout).
 //
 // Data of one level is written by other SMs of the group and read after the
 // barrier: the barrier's fences order the generic accesses and drop stale L1
 // lines, a proxy fence orders them before the bulk copies, and nothing is read
 // through the non-coherent path (NC = false).
-constexpr uint64_t kSweepWaitNs = 10000000000ull;
-
 struct SweepSync {
     unsigned arrive;       // barrier arrivals, counted up
     unsigned produced[4];  // by level modulo 4: the level made a frontier
@@ -859,12 +857,13 @@ struct SweepShared {
 
 // All nblk blocks of the group pass; false once a wait ran out.
 template <int W>
-__device__ __forceinline__ bool group_barrier(SweepSync *sync, int nblk, unsigned &round, SweepShared<W> &sh) {
+__device__ __forceinline__ bool group_barrier(const SweepParams &q, SweepSync *sync, int nblk, unsigned &round,
+                                              SweepShared<W> &sh) {
     asm volatile("fence.proxy.async;" ::: "memory");
     __syncthreads();
     if (threadIdx.x == 0) {
         ++round;
-        const unsigned want = round * (unsigned)nblk;
+        const unsigned want = round * (unsigned)nblk + q.barrier_absent;
         __threadfence();
         atomicAdd(&sync->arrive, 1u);
         bool ok = true;
@@ -876,7 +875,7 @@ __device__ __forceinline__ bool group_barrier(SweepSync *sync, int nblk, unsigne
             if ((spin & 255u) == 255u) {
                 const uint64_t now = stage::now_ns();
                 if (t0 == 0) t0 = now;
-                if (now - t0 > kSweepWaitNs) {
+                if (now - t0 > q.barrier_ns) {
                     ok = false;
                     break;
                 }
@@ -906,6 +905,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
     MsParams &p = sh.p;
     const size_t nB = (size_t)p.n * 32 * W;
     for (int i = bid * kBlock + tid; i < p.n; i += nblk * kBlock) p.bc[i] = 0.0;
+    // the arrival counters of split vertices, which a launch that gave up leaves as they were
+    for (int i = bid * kBlock + tid; i < max(p.nslots, q.b_nslots); i += nblk * kBlock) p.cnt[i] = 0u;
 
     bool alive = true;
     for (int bi = grp; alive && bi < q.nbat; bi += q.groups) {
@@ -940,7 +941,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
             }
         if (lead)
             for (int k = 0; k < 4; ++k) sync->produced[k] = 0u;
-        if (!group_barrier<W>(sync, nblk, round, sh)) break;
+        if (!group_barrier<W>(q, sync, nblk, round, sh)) break;
         for (int b = bid * kBlock + tid; b < p.nb; b += nblk * kBlock) init_source<W>(p, b);
         const int total = first_scan(p, sh.first);
         // level 0 -> 1 top-down by the rule on the sources' arcs
@@ -954,7 +955,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
             }
         }
         if (tid == 0) p.first = top ? 1 : 0;
-        if (!group_barrier<W>(sync, nblk, round, sh)) break;
+        if (!group_barrier<W>(q, sync, nblk, round, sh)) break;
 
         int L = 0;
         for (int l = top ? 1 : 0; !(top && total == 0); ++l) {
@@ -985,7 +986,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
                 if (f & 4u) atomicOr(p.wide + l + 1, 1u);
                 if (f & 8u) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
             }
-            if (!(alive = group_barrier<W>(sync, nblk, round, sh))) break;
+            if (!(alive = group_barrier<W>(q, sync, nblk, round, sh))) break;
             if (tid == 0) sh.level_made = *(volatile unsigned *)&sync->produced[l & 3];
             __syncthreads();
             if (sh.level_made == 0u) {
@@ -1012,11 +1013,11 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
         ws.qz = sh.bwd.qz[wib];
         for (int l = L; alive && l >= 1; --l) {
             backward_items<W, false, false>(p, l, bid, nblk, sh.bwd, ws);
-            if (l > 1) alive = group_barrier<W>(sync, nblk, round, sh);
+            if (l > 1) alive = group_barrier<W>(q, sync, nblk, round, sh);
         }
         if (!alive) break;
         // the group's next batch clears what this one still reads
-        if (bi + q.groups < q.nbat) alive = group_barrier<W>(sync, nblk, round, sh);
+        if (bi + q.groups < q.nbat) alive = group_barrier<W>(q, sync, nblk, round, sh);
     }
     if (lane == 0 && ws.fail) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
     if (tid == 0 && !sh.ok && round > 0) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
@@ -1029,9 +1030,11 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
     host_word(&p.hctl->done, q.seq, *(volatile uint32_t *)&p.ctl->status);
 }
 
-// bc[i] = (add: bc[i] +) the groups' sums, in group order.
+// bc[i] = (add: bc[i] +) the groups' sums, in group order. The sums of a launch
+// that gave up are left out: bc keeps what earlier runs put there.
 __global__ void __launch_bounds__(kBlock) k_sweep_merge(const __grid_constant__ SweepParams q, double *__restrict__ bc,
                                                         int32_t n, bool add) {
+    if (q.g[0].ctl->status & BC_STATUS_COPY_TIMEOUT) return;
     for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock) {
         double x = add ? bc[i] : 0.0;
         for (int k = 0; k < q.groups; ++k) x += q.g[k].bc[i];
@@ -1049,7 +1052,8 @@ __global__ void k_merge(const double *__restrict__ src, double *__restrict__ dst
     }
 }
 
-__global__ void k_scale(double *x, int32_t n, double f) {
+__global__ void k_scale(double *x, int32_t n, double f, const DevCtl *ctl) {
+    if (ctl->status & BC_STATUS_COPY_TIMEOUT) return;  // a run that gave up: x may be an earlier run's
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] *= f;
 }
 
@@ -1230,11 +1234,11 @@ void ms_launch_merge(const double *src, double *dst, int32_t n, const DevCtl *fr
     k_merge<<<g, kBlock, 0, st>>>(src, dst, n, from, to);
 }
 
-void launch_scale(double *x, int32_t n, double f, cudaStream_t st) {
+void launch_scale(double *x, int32_t n, double f, const DevCtl *ctl, cudaStream_t st) {
     if (n <= 0) return;
     int g = (n + kBlock - 1) / kBlock;
     g = g > 4 * sm_count() ? 4 * sm_count() : g;
-    k_scale<<<g, kBlock, 0, st>>>(x, n, f);
+    k_scale<<<g, kBlock, 0, st>>>(x, n, f, ctl);
 }
 
 }  // namespace bcgb

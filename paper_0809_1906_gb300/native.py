@@ -44,6 +44,7 @@ BC_KEEP_ORDER = 0x80
 BC_PAIRS = 0x100
 BC_TEST_WAIT_EXPIRY = 0x200
 BC_FORCE_BOTTOMUP = 0x400
+BC_TEST_BARRIER_EXPIRY = 0x800
 
 BC_KERNEL_INIT = 0
 BC_KERNEL_FORWARD = 1

@@ -69,3 +69,27 @@ def test_rows_left_unwritten_after_a_failed_call(nat):
         o = oracle.source(g, int(src[i]), with_delta=False)
         assert np.array_equal(sig[i].cpu().numpy().view(np.uint64), o["sigma"])
         assert np.array_equal(dist[i].cpu().numpy(), o["dist"].astype(np.int32))
+
+
+@pytest.mark.parametrize("g", [G.er_hamiltonian(400, 1600, 81), G.star_graph(700)], ids=lambda g: g.name)
+def test_barrier_expiry_spoils_no_sum(nat, g):
+    """A barrier of the one-launch form whose last arrival never comes gives up
+    after 2 ms: bc_result reports the timeout, the sums of the runs before stay
+    as they were (halving included), and the next runs on the handle, in either
+    form, are right. The star's hub is split into items that meet at counters."""
+    ref = oracle.bc(g)["bc"]
+    with nat.Graph.from_csr(g) as h:
+        h.run()
+        first, code, _ = h.result()
+        assert code == nat.BC_OK and close(first, ref, g.n)
+        h.run(flags=nat.BC_ACCUMULATE | nat.BC_HALVE | nat.BC_TEST_BARRIER_EXPIRY, device_wait_us=2000)
+        with pytest.raises(nat.BcError) as e:
+            h.result()
+        assert e.value.code == nat.BC_ERR_TIMEOUT
+        for flags in (0, nat.BC_TIMING):
+            h.run(flags=nat.BC_ACCUMULATE | nat.BC_TEST_BARRIER_EXPIRY, device_wait_us=2000)
+            h.run(flags=nat.BC_ACCUMULATE | flags)
+            got, code, st = h.result()
+            assert code == nat.BC_OK and st == 0
+            first = first + ref
+            assert close(got, first, 3 * g.n)
