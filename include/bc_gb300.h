@@ -144,8 +144,9 @@ extern "C" {
  *   delta          bucket width of the weighted path: 0 or 1 (exact distances
  *                  settle one value at a time, which the tie-aware path counts
  *                  need); any other value returns BC_ERR_UNSUPPORTED.
- *   wait_limit_ms  bound on every host-side wait for device progress
- *                  (0 = 600000). Expiry returns BC_ERR_TIMEOUT.
+ *   wait_limit_ms  bound on every host-side wait for device progress, that is
+ *                  for the next batch's forward pass to end, however many
+ *                  batches there are (0 = 600000). Expiry returns BC_ERR_TIMEOUT.
  *   alpha          direction of the unweighted forward sweep at level 0 -> 1,
  *                  the level whose frontier (the batch's sources) is known before
  *                  it runs: top-down (a push over the sources' arcs) while those
@@ -159,7 +160,10 @@ extern "C" {
  *                  the one before it (a launch past the last level still costs
  *                  a grid's start-up). 0 = 1/64.
  *   device_wait_us bound on each device-side wait for staged row copies
- *                  (0 = 2 s). Expiry sets BC_STATUS_COPY_TIMEOUT.
+ *                  (0 = 2 s). Expiry sets BC_STATUS_COPY_TIMEOUT. A run that
+ *                  sets it launches every level apart: small unweighted runs
+ *                  otherwise go in one launch, whose barriers have a bound of
+ *                  their own (10 s, then the same status bit).
  */
 typedef struct bc_options {
     int32_t batch;
@@ -204,7 +208,8 @@ int bc_create_graph(int32_t n, const int32_t *row_ptr, const int32_t *col, const
  *                bc_set_default_options), else the built-in defaults.
  * Without BC_ACCUMULATE the result starts from zero. Returns when all work is
  * enqueued on cuda_stream, except for the bounded host waits the level loop
- * needs to learn each batch's depth. Unweighted batches run on up to eight
+ * needs to learn each batch's depth (a small run in one launch: until every
+ * batch's forward pass has ended). Unweighted batches run on up to eight
  * concurrent lanes (batch i on lane i mod lanes, each lane with its own state
  * and BC accumulator, added in lane order at the end); weighted waves on two.
  * The assignment is fixed, so repeated runs give identical results. Errors:

@@ -384,6 +384,7 @@ struct bc_graph {
     // ctl->status as last read from the device, current while status_known
     uint32_t status = 0;
     bool status_known = false;
+    uint32_t status_seq = 0;  // the sweep that leaves it in hctl->done at its end (0: read ctl->status)
     std::vector<uint64_t> summ_host;  // bc_source_hashes
     int staged_all = 0;  // `sources` holds every vertex: 1 in id order, 2 in landmark order (0: anything else)
 
@@ -1564,14 +1565,30 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
             Timer t(g, st, BC_KERNEL_FORWARD);
             CK(bcgb::ms_launch_sweep(W, q, st));
         }
-        int status = 0;
-        const auto t0 = std::chrono::steady_clock::now();
-        for (long spins = 0; !bcgb::word_for(&g->hctl->done, q.seq, &status); ++spins) {
+        // wait until every batch's forward pass has ended (or the launch, early);
+        // each wait, up to the next batch that any group reports, has the limit
+        int status = 0, seen[kSweepLanes] = {};
+        bool ended = false;
+        auto t0 = std::chrono::steady_clock::now();
+        for (long spins = 0;; ++spins) {
+            ended = bcgb::word_for(&g->hctl->done, q.seq, &status);
+            if (ended) break;
+            bool all = true, moved = false;
+            for (int k = 0; k < K; ++k) {
+                int x = 0;
+                if (bcgb::word_for(&g->hctl->fwd[k], q.seq, &x) && x != seen[k]) {
+                    seen[k] = x;
+                    moved = true;
+                }
+                all &= seen[k] == (nbat - k + K - 1) / K;
+            }
+            if (all) break;
+            if (moved) t0 = std::chrono::steady_clock::now();
             if (spins % 1024 != 1023) continue;
             const auto ms =
                 std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count();
             if (ms > wait_ms)
-                return fail(BC_ERR_TIMEOUT, "the device did not report the end of the sweep within the wait limit");
+                return fail(BC_ERR_TIMEOUT, "the device did not report the end of a forward pass within the wait limit");
             const cudaError_t e = cudaStreamQuery(st);
             if (e != cudaSuccess && e != cudaErrorNotReady)
                 return fail(BC_ERR_CUDA, std::string("device error during a sweep: ") + cudaGetErrorString(e));
@@ -1580,13 +1597,11 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
             if (spins % 65536 == 65535) std::this_thread::yield();
         }
         // (a launch that gave up is not tried again: bc_result reports it)
-        if (!((uint32_t)status & BC_STATUS_LEVEL_CAP) || ((uint32_t)status & BC_STATUS_COPY_TIMEOUT)) {
+        if (!ended || !((uint32_t)status & BC_STATUS_LEVEL_CAP) || ((uint32_t)status & BC_STATUS_COPY_TIMEOUT)) {
             Timer t(g, st, BC_KERNEL_INIT);
             bcgb::ms_launch_sweep_merge(q, g->bc.p, n, (g->last_opt.flags & BC_ACCUMULATE) != 0, st);
             CK(cudaGetLastError());
-            g->status = (uint32_t)status;
-            g->status_known = true;
-            g->counters_unsure = ((uint32_t)status & BC_STATUS_COPY_TIMEOUT) != 0;
+            g->status_seq = q.seq;
             return BC_OK;
         }
         CK(cudaStreamSynchronize(st));
@@ -2294,6 +2309,7 @@ int bc_run(bc_graph *g, const int32_t *sources, int32_t num_sources, const bc_op
     g->dense_flops_f8 = 0.0;
     g->has_run = false;
     g->status_known = false;
+    g->status_seq = 0;
     const bool hash = !(flags & BC_NO_HASH);
     // the control block's run counters and the sweep's barrier words
     CK(cudaMemsetAsync(g->ctl, 0, kCtlBytes, st));
@@ -2345,10 +2361,17 @@ int bc_result(bc_graph *g, double *bc, uint32_t *status_flags) {
     if (!g) return fail(BC_ERR_ARG, "graph is NULL");
     if (!g->has_run) return fail(BC_ERR_STATE, "no completed bc_run");
     if (bc && g->n) CK(cudaMemcpyAsync(bc, g->bc.p, (size_t)g->n * sizeof(double), cudaMemcpyDefault, g->last_stream));
-    // the status word, unless the host has its final value already
-    if (!g->status_known)
+    // the status word, unless the host has its final value already or a sweep leaves it in host memory
+    if (!g->status_known && !g->status_seq)
         CK(cudaMemcpyAsync(&g->status, &g->ctl->status, sizeof(uint32_t), cudaMemcpyDefault, g->last_stream));
     CK(cudaStreamSynchronize(g->last_stream));
+    if (!g->status_known && g->status_seq) {
+        int x = 0;
+        if (!bcgb::word_for(&g->hctl->done, g->status_seq, &x))
+            return fail(BC_ERR_STATE, "the sweep ended without reporting its status");
+        g->status = (uint32_t)x;
+        g->counters_unsure = (g->status & BC_STATUS_COPY_TIMEOUT) != 0;
+    }
     g->status_known = true;
     const uint32_t status = g->status;
     if (status_flags) *status_flags = status;
@@ -2436,6 +2459,7 @@ int bc_forward_rows(bc_graph *g, const int32_t *sources, int32_t k, uint64_t *si
     }
     CK(cudaMemsetAsync(&g->ctl->status, 0, sizeof(uint32_t), st));
     g->status_known = false;
+    g->status_seq = 0;
     g->timing = false;
     if (g->weighted && opt && (opt->flags & BC_DENSE)) {
         if (!sigma || !dist) return fail(BC_ERR_ARG, "BC_DENSE rows of a weighted graph need both outputs");
@@ -2909,6 +2933,7 @@ int bc_many_run(bc_many *m, void *cuda_stream) {
         g->last_stream = st;
         g->last_nsrc = g->n;
         g->launches = 0;
+        g->status_seq = 0;  // an earlier sweep's word is not this run's
     }
     m->last_stream = st;
     m->ran = true;

@@ -48,12 +48,15 @@ struct DevCtl {
 // sequence number in its high half and the value in its low half, so the host
 // learns both from one read: nothing has to be ordered, and the last block of
 // a level does not wait for its writes to reach host memory.
+constexpr int kSweepGroups = 8;  // groups of the one-launch sweep (SweepParams)
 struct HostCtl {
-    unsigned long long done;      // (seq << 32) | depth L once the forward pass ended (-1: level capacity hit)
+    unsigned long long done;      // (seq << 32) | depth L once the forward pass ended (-1: level capacity hit);
+                                  // the one-launch sweep: (seq << 32) | status, at its end
     unsigned long long progress;  // (seq << 32) | number of forward levels completed
     unsigned long long counts;    // (vertices in the newest frontier << 32) | (in the one before), each
                                   // -1 when not counted; a hint for the host's look-ahead only
     unsigned long long pad;
+    unsigned long long fwd[kSweepGroups];  // (seq << 32) | batches of the group whose forward pass has ended
 };
 
 #ifdef __CUDACC__
@@ -128,7 +131,6 @@ struct MsParams {
 
 // One launch for the whole sweep of a run (k_sweep, msbfs.cu): groups of
 // blocks take batches in turn, group k with the state in g[k].
-constexpr int kSweepGroups = 8;
 constexpr size_t kSweepSyncBytes = kSweepGroups * 128;
 struct SweepParams {
     int32_t groups, group_blocks;

@@ -995,7 +995,10 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
             }
         }
         if (!alive) break;
-        if (lead) atomicAdd(&p.ctl->depth_sum, (unsigned long long)L);
+        if (lead) {
+            atomicAdd(&p.ctl->depth_sum, (unsigned long long)L);
+            host_word(&p.hctl->fwd[grp], q.seq, (uint32_t)(bi / q.groups + 1));
+        }
         // the summaries read what the forward pass left; the narrow deepest
         // backward level follows without a barrier of their own
         if (q.hash) hash_tiles<W, false, 6, 8>(p, L, bid, nblk, sh.hash);

@@ -93,3 +93,40 @@ def test_barrier_expiry_spoils_no_sum(nat, g):
             assert code == nat.BC_OK and st == 0
             first = first + ref
             assert close(got, first, 3 * g.n)
+
+
+def test_wait_limit_is_per_batch(nat):
+    """1250 batches in one launch take several times the host's wait limit, each
+    of them a fraction of it: the run is not cut short."""
+    import torch
+    g = G.er_hamiltonian(2000, 8000, 82)
+    src = np.tile(np.arange(g.n, dtype=np.int32), 20)
+    ref = 20.0 * oracle.bc(g)["bc"]
+    with nat.Graph.from_csr(g) as h:
+        h.run(src, batch=32)
+        h.result()
+        t0 = time.perf_counter()
+        h.run(src, batch=32)
+        h.result()
+        whole = 1e3 * (time.perf_counter() - t0)
+        assert whole > 15.0, whole  # else the limit below says nothing
+        h.run(src, batch=32, wait_limit_ms=4)
+        got, code, _ = h.result()
+    assert code == nat.BC_OK and close(got, ref, 20 * g.n)
+
+
+def test_run_returns_before_the_backward_pass_ends(nat):
+    """bc_run waits for the forward passes alone: on a path of 1500 levels the
+    backward pass, as long again, is still under way when it returns."""
+    import torch
+    g = G.path_graph(1500)
+    src = np.arange(32, dtype=np.int32)
+    with nat.Graph.from_csr(g) as h:
+        h.run(src, batch=32)
+        h.result()
+        h.run(src, batch=32)
+        time.sleep(3e-4)
+        running = not torch.cuda.current_stream().query()
+        got, code, _ = h.result()
+    assert code == nat.BC_OK and close(got, oracle.bc(g, src)["bc"], g.n)
+    assert running
