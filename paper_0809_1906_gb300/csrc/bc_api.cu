@@ -204,10 +204,12 @@ struct ItemPlan {
     }
 };
 
-// A handle's control block: DevCtl, then the sweep's finish counter and barrier
-// words, cleared together before a run.
-constexpr size_t kCtlSweepAt = 256;
-static_assert(sizeof(bcgb::DevCtl) <= kCtlSweepAt - 128, "the finish counter lies between the two");
+// A handle's control block: DevCtl, the sweep's batches done by group, its finish
+// and capacity words, its barrier words. All are cleared before a run, those
+// from kCtlFinishAt on before the run resumes.
+constexpr size_t kCtlNextAt = 96, kCtlFinishAt = 128, kCtlSweepAt = 256;
+static_assert(sizeof(bcgb::DevCtl) <= kCtlNextAt && kCtlNextAt + 4 * bcgb::kSweepGroups <= kCtlFinishAt,
+              "the parts of the control block");
 constexpr size_t kCtlBytes = kCtlSweepAt + bcgb::kSweepSyncBytes;
 constexpr int kSweepLanes = 8;                    // concurrent batches of the unweighted sweep
 constexpr int kSideStreams = 4;                   // side streams of the dense path's per-batch summaries
@@ -1510,8 +1512,9 @@ constexpr uint64_t kBarrierWaitNs = 10000000000ull;
 
 // Batches of a run as one cooperative launch (k_sweep): group k takes batches
 // k, k + K, ... with lane k's state and its own BC sums, added in group order at
-// the end. A batch deeper than the level capacity ends the launch; the capacity
-// doubles and the run starts over (nothing has reached g->bc yet).
+// the end. A batch deeper than the level capacity ends its group's part of the
+// launch; the capacity doubles, and a second launch goes on from there in every
+// group that has batches left, with the sums so far.
 int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool hash, int64_t wait_ms) {
     const int B = 32 * W;
     const int32_t n = g->n, nbat = (nsrc + B - 1) / B;
@@ -1519,7 +1522,7 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
     if (resident < K) return fail(BC_ERR_CUDA, "the sweep kernel does not fit the device");
     CK(g->sweep_bc.ensure((size_t)std::max(n, 1)));
     int Lcap = g->Lcap;
-    for (;;) {
+    for (bool resume = false;; resume = true) {
         for (int k = 1; k < K; ++k) {
             const int r = ensure_lane(g, g->lanes[k - 1], W, Lcap);
             if (r) return r;
@@ -1553,7 +1556,10 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
         q.b_slot_first = g->bplan.slot_first;
         q.b_slot_nch = g->bplan.slot_nch;
         q.sync = reinterpret_cast<char *>(g->ctl) + kCtlSweepAt;
-        q.finished = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(g->ctl) + kCtlSweepAt - 128);
+        q.finished = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(g->ctl) + kCtlFinishAt);
+        q.capped = q.finished + 1;
+        q.next = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(g->ctl) + kCtlNextAt);
+        q.resume = resume ? 1 : 0;
         for (int k = 0; k < K; ++k) {
             q.g[k] = lane_params(g, k);
             q.g[k].ctl = g->ctl;
@@ -1608,7 +1614,7 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
         Lcap *= 2;
         const int r = ensure_state(g, W, Lcap);
         if (r) return r;
-        CK(cudaMemsetAsync(g->ctl, 0, kCtlBytes, st));
+        CK(cudaMemsetAsync(reinterpret_cast<char *>(g->ctl) + kCtlFinishAt, 0, kCtlBytes - kCtlFinishAt, st));
     }
 }
 

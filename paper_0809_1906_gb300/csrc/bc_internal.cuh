@@ -151,7 +151,11 @@ struct SweepParams {
     uint64_t barrier_ns;      // bound on each wait at a group's barrier
     uint32_t barrier_absent;  // arrivals that every barrier expects and none makes (the test hook; else 0)
     void *sync;          // kSweepSyncBytes bytes, zero at launch
-    unsigned *finished;  // zero at launch
+    // zero at a run's first launch: blocks that finished, whether a group met a batch
+    // deeper than its levels, and each group's batches done (where a launch that
+    // resumes goes on; its BC sums are kept)
+    unsigned *finished, *capped, *next;
+    int32_t resume;
     MsParams g[kSweepGroups];
 };
 int ms_sweep_blocks(int W);  // blocks resident on the device at once (0: error)

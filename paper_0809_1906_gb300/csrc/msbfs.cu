@@ -851,6 +851,7 @@ struct SweepShared {
     };
     MsParams p;  // the group's batch in work
     uint64_t bar[kWarps];
+    unsigned long long arcs;  // this block's arcs of the batch in work, counted once its forward pass ends
     unsigned level_made;
     bool ok;
 };
@@ -904,12 +905,16 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
     __syncthreads();
     MsParams &p = sh.p;
     const size_t nB = (size_t)p.n * 32 * W;
-    for (int i = bid * kBlock + tid; i < p.n; i += nblk * kBlock) p.bc[i] = 0.0;
+    const int first = grp + q.groups * (int)q.next[grp];  // written after the group's first barrier only
+    if (lead && q.resume) host_word(&p.hctl->fwd[grp], q.seq, (uint32_t)(first / q.groups));
+    if (!q.resume)
+        for (int i = bid * kBlock + tid; i < p.n; i += nblk * kBlock) p.bc[i] = 0.0;
     // the arrival counters of split vertices, which a launch that gave up leaves as they were
     for (int i = bid * kBlock + tid; i < max(p.nslots, q.b_nslots); i += nblk * kBlock) p.cnt[i] = 0u;
 
     bool alive = true;
-    for (int bi = grp; alive && bi < q.nbat; bi += q.groups) {
+    int bi = first;
+    for (; alive && bi < q.nbat; bi += q.groups) {
         const int b0 = bi * 32 * W;
         if (tid == 0) {
             p.nb = min(32 * W, q.nsrc - b0);
@@ -949,18 +954,21 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
         if (top) first_arcs<W>(p, bid, nblk, sh.first, total);
         if (lead) {
             p.lsize[0] = (uint32_t)p.nb;
-            if (top) {
-                p.lsize[1] = (uint32_t)total;
-                atomicAdd(&p.ctl->dag_arcs, (unsigned long long)total);
-            }
+            if (top) p.lsize[1] = (uint32_t)total;
         }
-        if (tid == 0) p.first = top ? 1 : 0;
+        if (tid == 0) {
+            p.first = top ? 1 : 0;
+            sh.arcs = lead && top ? (unsigned long long)total : 0ull;
+        }
         if (!group_barrier<W>(q, sync, nblk, round, sh)) break;
 
         int L = 0;
         for (int l = top ? 1 : 0; !(top && total == 0); ++l) {
-            if (l + 1 >= p.Lcap) {  // deeper than the state's levels: the host grows it and starts over
-                if (lead) atomicOr(&p.ctl->status, BC_STATUS_LEVEL_CAP);
+            if (l + 1 >= p.Lcap) {  // deeper than the state's levels: the host grows it, the group goes on from here
+                if (lead) {
+                    atomicExch(q.capped, 1u);
+                    q.next[grp] = (unsigned)(bi / q.groups);
+                }
                 alive = false;
                 break;
             }
@@ -979,7 +987,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
             __syncthreads();
             if (tid == 0) {
                 const uint32_t f = sh.fwd.flags;
-                if (sh.fwd.arcs) atomicAdd(&p.ctl->dag_arcs, sh.fwd.arcs);
+                sh.arcs += sh.fwd.arcs;
                 if (sh.fwd.front) atomicAdd(p.lsize + l + 1, sh.fwd.front);
                 if (f & 1u) atomicOr(&sync->produced[l & 3], 1u);
                 if (f & 2u) atomicOr(&p.ctl->status, BC_STATUS_SIGMA_OVERFLOW);
@@ -995,6 +1003,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
             }
         }
         if (!alive) break;
+        if (tid == 0 && sh.arcs) atomicAdd(&p.ctl->dag_arcs, sh.arcs);
         if (lead) {
             atomicAdd(&p.ctl->depth_sum, (unsigned long long)L);
             host_word(&p.hctl->fwd[grp], q.seq, (uint32_t)(bi / q.groups + 1));
@@ -1022,6 +1031,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
         // the group's next batch clears what this one still reads
         if (bi + q.groups < q.nbat) alive = group_barrier<W>(q, sync, nblk, round, sh);
     }
+    if (lead && bi >= q.nbat) q.next[grp] = (unsigned)(bi / q.groups);
     if (lane == 0 && ws.fail) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
     if (tid == 0 && !sh.ok && round > 0) atomicOr(&p.ctl->status, BC_STATUS_COPY_TIMEOUT);
     // the last block of all reports the end and the status to the host
@@ -1030,7 +1040,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_sweep(const __grid_constant__ Swe
     __threadfence();
     if (atomicAdd(q.finished, 1u) != gridDim.x - 1) return;
     __threadfence();
-    host_word(&p.hctl->done, q.seq, *(volatile uint32_t *)&p.ctl->status);
+    host_word(&p.hctl->done, q.seq,
+              *(volatile uint32_t *)&p.ctl->status | (*(volatile unsigned *)q.capped ? BC_STATUS_LEVEL_CAP : 0u));
 }
 
 // bc[i] = (add: bc[i] +) the groups' sums, in group order. The sums of a launch
