@@ -14,8 +14,11 @@
 // word can contribute, no staging. Masked rows are written in the same view,
 // one vector store per row.
 //
-// Sums: counts are integers; dependencies are added per source in the order
-// that msbfs_body.cuh adds them (see bwd_light), so results do not change.
+// Sums: counts are integers; each source's dependency is added in the order
+// that msbfs_body.cuh adds it (see bwd_light), so those are the same. A vertex's
+// sum over the batch's sources is formed in another fixed order (eight lanes one
+// after another, then a two-step tree) with the low words added rounded, so BC
+// may differ from the per-vertex form in the last bits of that FP32 pair.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -48,7 +51,11 @@ struct LightScratch {
 // Take the next pack from the light items lt (a ballot over the warp's group;
 // v, beg, deg: the lane's own item): its vertices' arcs lie in the warp's lanes
 // one after another. Returns the number of vertices; starts has the first lane
-// of each, total is the number of arcs.
+// of each that has arcs, total is the number of arcs. A lane finds its arc's
+// vertex by counting the starts up to it, so vertices without arcs (a directed
+// graph's sinks, in the backward sweep) must be the last of their group: the
+// plans sort by decreasing degree (build_items), and a vertex of an undirected
+// graph that any level reaches has arcs.
 template <int W>
 __device__ __forceinline__ int light_select(unsigned &lt, int v, int beg, int deg_, LightScratch<W> &L, int lane,
                                             unsigned &starts, int &total) {
@@ -71,7 +78,7 @@ __device__ __forceinline__ int light_select(unsigned &lt, int v, int beg, int de
         L.idx[r] = lane;
     }
     const unsigned c = __ballot_sync(kFull, chosen);
-    starts = __reduce_or_sync(kFull, chosen ? 1u << (incl - deg) : 0u);
+    starts = __reduce_or_sync(kFull, chosen && deg > 0 ? 1u << (incl - deg) : 0u);  // incl - deg < 32
     total = __reduce_max_sync(kFull, chosen ? incl : 0);
     lt &= ~c;
     __syncwarp();
@@ -274,7 +281,7 @@ __device__ __forceinline__ void bwd_light(unsigned lt, int v, int beg, int deg, 
             const int o = L.off[r], dg = L.deg[r], k = L.idx[r];
             const size_t at = (size_t)L.v[r] * B + W * lane;
             const uint32_t fw = f[k][jl], mine = fw >> sh;
-            unsigned seg = (contrib >> o) & ((1u << dg) - 1u);
+            unsigned seg = dg > 0 ? (contrib >> o) & ((1u << dg) - 1u) : 0u;  // o may be 32 without arcs
             float hi = 0.0f, lo = 0.0f;
             const int nsrc = TREE ? __reduce_add_sync(kFull, __popc(mine & ((1u << W) - 1u))) : kSparseSrc + 1;
             if (TREE && nsrc <= kSparseSrc) {
