@@ -107,6 +107,7 @@ cudaError_t alloc(void **p, size_t bytes, size_t *got) {
         cudaGetLastError();
         trim(dev);
         e = cudaMalloc(p, bytes);
+        if (e != cudaSuccess) cudaGetLastError();  // reported by this call, not again by a later one
     }
     if (e == cudaSuccess) *got = bytes;
     return e;
@@ -541,6 +542,8 @@ int check_graph(int32_t n, const std::vector<int32_t> &rp, const std::vector<int
 int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int32_t> &rp) {
     if (pl.chunk == chunk && pl.items) return BC_OK;
     const int32_t n = g->n;
+    pl.chunk = 0;  // no plan until the new one is in place: an allocation may fail
+    pl.items = nullptr;
     // items: the chunks of the split vertices (in vertex order), then the
     // other vertices by decreasing degree (a stable counting sort: degree <= chunk)
     int64_t nitems = 0, nslots = 0, nlight = 0;
@@ -641,6 +644,7 @@ int ensure_state(bc_graph *g, int W, int Lcap) {
     const size_t n = (size_t)std::max(g->n, 1);
     const size_t B = 32 * (size_t)W;
     const size_t nw32 = (n + 31) / 32;
+    g->W = 0;  // no state until all of it is in place: an allocation may fail
     CK(g->sigma.ensure(n * B));
     g->s_levels = s_levels_for(n, B, Lcap);
     CK(g->Smask.ensure((size_t)g->s_levels * n * B));
@@ -740,19 +744,28 @@ int ensure_lane(bc_graph *g, SweepLane &ln, int W, int Lcap) {
     if (!ln.st) {
         fresh = true;
         ln.dev = dev;
-        CK(cudaStreamCreateWithFlags(&ln.st, cudaStreamNonBlocking));
-        CK(cudaEventCreateWithFlags(&ln.ev, cudaEventDisableTiming));
-        CK(cudaMalloc((void **)&ln.ctl, sizeof(bcgb::DevCtl)));
-        CK(cudaMemset(ln.ctl, 0, sizeof(bcgb::DevCtl)));
-        CK(cudaHostAlloc((void **)&ln.hctl, sizeof(bcgb::HostCtl), cudaHostAllocMapped | cudaHostAllocPortable));
-        std::memset(ln.hctl, 0, sizeof(bcgb::HostCtl));
-        CK(cudaHostGetDevicePointer((void **)&ln.hctl_d, ln.hctl, 0));
+        auto make = [&]() -> int {
+            CK(cudaStreamCreateWithFlags(&ln.st, cudaStreamNonBlocking));
+            CK(cudaEventCreateWithFlags(&ln.ev, cudaEventDisableTiming));
+            CK(cudaMalloc((void **)&ln.ctl, sizeof(bcgb::DevCtl)));
+            CK(cudaMemset(ln.ctl, 0, sizeof(bcgb::DevCtl)));
+            CK(cudaHostAlloc((void **)&ln.hctl, sizeof(bcgb::HostCtl), cudaHostAllocMapped | cudaHostAllocPortable));
+            std::memset(ln.hctl, 0, sizeof(bcgb::HostCtl));
+            CK(cudaHostGetDevicePointer((void **)&ln.hctl_d, ln.hctl, 0));
+            return BC_OK;
+        };
+        const int r = make();
+        if (r) {
+            ln.release();  // no half-made lane stays on the handle
+            return r;
+        }
     }
     const size_t slots = (size_t)std::max({g->fplan.nslots, g->bplan.nslots, 1});
     if (!fresh && ln.W == W && ln.Lcap >= Lcap && ln.n >= g->n && ln.slots >= slots && ln.sigma.p) return BC_OK;
     const size_t n = (size_t)std::max(g->n, 1);
     const size_t B = 32 * (size_t)W;
     const size_t nw32 = (n + 31) / 32;
+    ln.W = 0;  // as in ensure_state
     CK(ln.sigma.ensure(n * B));
     ln.s_levels = s_levels_for(n, B, Lcap);
     CK(ln.Smask.ensure((size_t)ln.s_levels * n * B));
@@ -1006,7 +1019,7 @@ int stage_sources(bc_graph *g, const int32_t *sources, int32_t num, int32_t *cou
 }
 
 int ensure_dense(bc_graph *g, cudaStream_t st) {
-    if (g->dA.p) return BC_OK;
+    if (g->npad) return BC_OK;  // set once both adjacency matrices are built
     if (g->weighted) return fail(BC_ERR_UNSUPPORTED, "BC_DENSE needs an unweighted graph");
     if (g->directed) return fail(BC_ERR_UNSUPPORTED, "BC_DENSE needs an undirected graph");
     if (g->n > bcgb::kDenseMaxN) return fail(BC_ERR_UNSUPPORTED, "BC_DENSE supports n <= 65536");
@@ -1026,6 +1039,7 @@ int ensure_dense(bc_graph *g, cudaStream_t st) {
 int ensure_dense_group(bc_graph *g, int nb, int Lcap, cudaStream_t st) {
     if (g->gNB >= nb && g->gLcap == Lcap && g->gsigma.p) return BC_OK;
     const size_t n = (size_t)std::max(g->n, 1), nw32 = (n + 31) / 32;
+    g->gNB = 0;  // as in ensure_state
     CK(g->gsigma.ensure((size_t)nb * n * 128));
     CK(g->gF.ensure((size_t)nb * Lcap * n * 4));
     CK(g->gV.ensure((size_t)nb * 2 * n * 4));
@@ -1889,6 +1903,7 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
     int lanes = g->timing ? 1 : std::min<int32_t>(kWeightedLanes, nwaves);
     while (lanes > 1 && lanes * lane_bytes > kWeightedLaneBudget) --lanes;
     if (g->wG < G || g->wK != K || g->wC != C) {
+        g->wG = 0;  // as in ensure_state
         CK(g->worder.ensure((size_t)G * n));
         CK(g->wgrp.ensure((size_t)G * (n + 1)));
         CK(g->wslots.ensure((size_t)G * K * C));
@@ -2008,6 +2023,7 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
     // its launches hold at most three sources per SM (its CTAs are 256 threads)
     const int G64 = std::min(G, 3 * sm_count_host());
     if (!rpos.empty() && g->wG64 < G64) {
+        g->wG64 = 0;  // as in ensure_state
         CK(g->wdist.ensure((size_t)G64 * n));
         CK(g->wsigma.ensure((size_t)G64 * n));
         CK(g->wcval.ensure((size_t)G64 * n));

@@ -130,3 +130,26 @@ def test_run_returns_before_the_backward_pass_ends(nat):
         got, code, _ = h.result()
     assert code == nat.BC_OK and close(got, oracle.bc(g, src)["bc"], g.n)
     assert running
+
+
+def test_out_of_memory_leaves_the_handle_usable(nat):
+    """A path of three million vertices needs more level capacity than the GPU
+    holds: the run reports that it is out of memory, and so does the next one
+    (it must not take the half-grown state for a whole one); sources of a small
+    component beside it then run on the same handle."""
+    n, k = 3_000_000, 5
+    at = np.arange(n - 1)
+    g = G.csr_from_edges(n + k, np.concatenate([at, n + np.arange(k - 1)]), np.concatenate([at + 1, n + 1 + np.arange(k - 1)]),
+                         name="paths")
+    src = n + np.arange(k, dtype=np.int32)
+    ref = oracle.bc(G.path_graph(k))["bc"]
+    with nat.Graph.from_csr(g, trust_input=True) as h:
+        for _ in range(2):
+            with pytest.raises(nat.BcError) as e:
+                h.run(np.array([0], np.int32))
+            assert e.value.code == nat.BC_ERR_OOM
+        h.run(src)
+        got, code, st = h.result()
+        assert code == nat.BC_OK and st == 0
+    assert np.all(got[:n] == 0.0) and close(got[n:], ref, k)
+    nat.release_cached_memory()
