@@ -1500,22 +1500,44 @@ int run_lanes(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool bac
 }
 
 // Whether a run is one launch (run_sweep) instead of a launch per level
-// (run_lanes): while the items of a level that fall to one warp of a group, in
-// heavy items (a light one counts 3/8 of that, in its pack), are at most
-// kSweepUnits. Whole calls, ms per level / one launch, all sources unless
-// stated, with the units a warp has:
-//   random n = 300 (0.8)   0.161 / 0.128    R-MAT n = 3153 (4.6)  1.07 / 0.77
-//   random n = 1024 (0.8)  0.309 / 0.212    R-MAT n = 6184, 2048 sources (9.6) 1.01 / 0.95
-//   random n = 5000 (8.6)  1.81 / 1.69      R-MAT n = 23756, 300 sources (9.3) 0.90 / 0.87
-//   random n = 5900 (12)   2.16 / 2.24      R-MAT n = 12124, directed (17) 7.6 / 8.7
-//   40 x 40 mesh (1.3)     0.74 / 0.50      128 x 128 mesh (13.5) 24 / 35
-// Beyond, a level is enough work to fill the GPU by itself, and a kernel for
-// one direction alone, with every block of the GPU, runs it better.
-constexpr int64_t kSweepUnits = 10;
-bool one_launch(const bc_graph *g, int W, int K) {
-    auto units = [](const ItemPlan &pl) { return 8 * (int64_t)pl.nheavy + 3 * (int64_t)(pl.nitems - pl.nheavy); };
-    const int64_t warps = 8 * (int64_t)(bcgb::ms_sweep_blocks(W) / K);
-    return std::max(units(g->fplan), units(g->bplan)) <= 8 * kSweepUnits * warps;
+// (run_lanes): while a level is too little work to be worth launches of its
+// own. The work of a level is its items per warp of a group, a light item
+// counted as part of a heavy one; the launch per level gains on the other form
+// where batches are few (a batch has the whole GPU) or uneven (groups idle in
+// the last round, where a lane's level would have the GPU to itself), and, from
+// kFullPackLanes batches on, by its full packs on light items. Whole calls, ms
+// per level / one launch, with the units that the branch compares:
+//   one batch, or one and up to B / 32 sources more; units of a warp of all the GPU
+//     random n = 300, 256 sources (0.08) 0.146 / 0.127   random n = 2000 (0.51)  0.174 / 0.166
+//     random n = 4000 (1.0) 0.210 / 0.235                R-MAT n = 1736 (0.42)   0.312 / 0.323
+//     64 x 64 mesh (0.84)   0.410 / 0.451                R-MAT n = 23756, 257 sources (6.0) 0.699 / 0.843
+//   two and three batches
+//     random n = 1024 k 270 (0.4) 0.189 / 0.156          R-MAT n = 23756 k 300 (9.2) 0.867 / 0.772
+//     R-MAT n = 12510 k 600 (7.4) 0.828 / 0.728          random n = 20000, m = 160000 k 400 (11) 0.633 / 0.713
+//   more, units divided by the share of the groups' rounds that is used
+//     random n = 9000, 4 batches (9.3) 0.734 / 0.636     R-MAT n = 12510, 4 batches (13) 0.876 / 1.113
+//     random n = 7500, 8 (15.2) 1.021 / 0.904            120 x 120 mesh, 4 batches (12) 1.490 / 1.717
+//     R-MAT n = 6184, 25 (15.9) 2.45 / 2.25              100 x 100 mesh, 40 (16.8) 9.2 / 10.3
+//     R-MAT n = 6184, 9 (22) 1.117 / 1.371               110 x 110 mesh, 48 (20) 13.0 / 15.3
+//   in the caller's order the sources of a word are spread, a level holds more
+//     R-MAT n = 6184, 25 (15.9) 3.19 / 3.53              random n = 5000, 20 (12.4) 1.793 / 1.635
+//   narrower rows are less work per item
+//     R-MAT n = 6184, 12 batches of 128 (17) 0.926 / 0.832
+//     R-MAT n = 6184, 10 batches of 64 (21) 0.747 / 0.587   R-MAT n = 12510, the same (43) 0.989 / 1.032
+constexpr double kSweepUnitsOne = 0.6, kSweepUnitsFew = 10.0, kSweepUnitsMost = 16.8, kSweepUnitsPerGroup = 2.6;
+bool one_launch(const bc_graph *g, int32_t nsrc, int W, int K) {
+    const int B = 32 * W, resident = bcgb::ms_sweep_blocks(W);
+    if (resident < K) return false;
+    auto units = [&](double light, int blocks) {  // items of a level that fall to one of the blocks' warps (eight each)
+        auto of = [&](const ItemPlan &pl) { return (double)pl.nheavy + light * (double)(pl.nitems - pl.nheavy); };
+        return std::max(of(g->fplan), of(g->bplan)) / (8.0 * blocks);
+    };
+    const int32_t batches = std::max<int32_t>(1, (nsrc - B / 32 + B - 1) / B);  // a sliver at the end is none
+    if (batches == 1) return units(0.75, resident) <= kSweepUnitsOne;
+    if (K < kFullPackLanes) return units(0.375, resident / K) <= kSweepUnitsFew;
+    const double used = std::min(1.0, (double)nsrc / ((double)B * K * ((batches + K - 1) / K)));
+    const double most = std::min(kSweepUnitsMost, kSweepUnitsPerGroup * K) * (g->reordered ? 1.0 : 0.8) * (W <= 2 ? 1.5 : W == 4 ? 1.2 : 1.0);
+    return units(0.75, resident / K) <= most * used;
 }
 
 // Bound on each wait at a barrier of the one-launch sweep. Such a wait lasts as
@@ -1671,7 +1693,7 @@ int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStr
         int K = g->timing ? 1 : std::min<int32_t>(kSweepLanes, nbat);
         while (K > 1 && (K - 1) * lane_bytes > kLaneBudgetBytes) --K;
         const bool sweep = backward && !rows_sig && !rows_dist && !g->timing &&
-                           (g->dev_wait_ns == 0 || g->test_barrier) && g->test_hold == 0 && nsrc > 0 && one_launch(g, W, K);
+                           (g->dev_wait_ns == 0 || g->test_barrier) && g->test_hold == 0 && nsrc > 0 && one_launch(g, nsrc, W, K);
         if (sweep) return run_sweep(g, nsrc, W, K, st, hash, wait_ms);
         r = reset_counters(g, st);
         if (!r && backward) r = clear_outputs(g, nsrc, hash, st);

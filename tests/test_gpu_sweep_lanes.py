@@ -99,4 +99,15 @@ def test_sinks_behind_full_packs(nat, eights, sinks, keep_off):
     """Packs filled by four vertices of eight arcs with vertices of no arcs
     behind them in the same group (a warp's share is 13 or more here)."""
     g = eights_and_sinks(eights, sinks, 65)
-    check(nat, g, np.arange(0, g.n, 21, dtype=np.int32), 32, 2 if keep_off else 0, device_wait_us=keep_off)
+    check(nat, g, np.arange(0, g.n, 12, dtype=np.int32), 32, 2 if keep_off else 0, device_wait_us=keep_off)
+
+
+@pytest.mark.parametrize("scale,sources,keep,lanes", [(13, 257, False, True), (13, 300, False, False),
+                                                      (13, 2304, False, True), (12, 2304, False, False),
+                                                      (13, 2600, True, True), (12, 900, True, False)])
+def test_uneven_and_spread_batches_take_the_lanes(nat, scale, sources, keep, lanes):
+    """Which form runs when one batch holds all but a sliver of the sources, the
+    groups' last round is nearly empty, or the caller's order is kept, on both
+    sides of the line; either form gives the oracle's values."""
+    g = G.rmat_lcc(scale, 16)
+    check(nat, g, G.sample_sources(g.n, sources, 66), 256, 2 if lanes else 0, flags=nat.BC_KEEP_ORDER if keep else 0)
