@@ -2740,7 +2740,7 @@ const char *bc_last_error(void) { return g_err.c_str(); }
 
 struct bc_many {
     std::vector<bc_graph *> graphs;
-    int W = 1, grid = 0, Lcap = 64;
+    int W = 1, grid = 0, threads = 0, Lcap = 64;
     bool hash = true;  // per-source summaries into each graph's handle
     int32_t nitems = 0;
     std::vector<bcgb::ManyGraph> h_graphs;  // what d_graphs holds, once no longer stale
@@ -2819,14 +2819,16 @@ int build_many(bc_many *m) {
     std::vector<GInfo> info(m->graphs.size());
     double total = 0.0;
     int nmax = 1;
+    int64_t batches = 0;
     for (size_t i = 0; i < m->graphs.size(); ++i) {
         const bc_graph *g = m->graphs[i];
         info[i].nb = (g->n + B - 1) / B;
         info[i].cost = (double)info[i].nb * (double)(g->n + g->narcs + 1);
         total += info[i].cost;
+        batches += info[i].nb;
         nmax = std::max(nmax, g->n);
     }
-    m->grid = bcgb::many_blocks_per_sm(m->W) * sm_count_host();
+    m->threads = bcgb::many_plan(m->W, nmax, batches, sm_count_host(), &m->grid);
     const double share = std::max(1.0, total / (8.0 * m->grid));
     struct Item {
         bcgb::ManyItem it;
@@ -2914,7 +2916,7 @@ int build_many(bc_many *m) {
     if (e == cudaSuccess) e = cudaMemsetAsync(m->capped.p, 0, gd.size() * sizeof(unsigned), cap);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->ctl, 0, sizeof(bcgb::DevCtl), cap);
     if (e == cudaSuccess && m->nitems > 0) {
-        bcgb::many_launch(m->W, p, m->grid, cap);
+        bcgb::many_launch(m->W, m->threads, p, m->grid, cap);
         e = cudaGetLastError();
     }
     cudaGraph_t gr = nullptr;

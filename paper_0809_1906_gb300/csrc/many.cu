@@ -46,12 +46,26 @@ constexpr int kManyLightDeg = 16;
 // vertices 120.9 / 120.3 / 120.2 ms, 250 up to 1500 7.60 / 5.31 / 4.55, 300 up
 // to 400 (batch 64) 0.79 / 0.63 / 0.67. At two per SM, 384 / 448 / 512 threads (80, 72,
 // 64 registers): 119.0 / 110.5 / 112.6, 5.25 / 4.88 / 4.98, 0.63 / 0.61 / 0.59 ms: 448.
-constexpr int kMBlock = 448;
-constexpr int kMWarps = kMBlock / 32;
+// A batch of a graph of some fifty vertices has no work for 14 warps, and a set of
+// thousands of them keeps more, smaller CTAs busy (whole pass, ms, 128 x 8 / 256 x 4 /
+// 448 x 2):
+//   2000 graphs of 20 to 60 vertices, batch 32   0.368 / 0.409 / 0.514, batch 256 0.454 / 0.493 / 0.550
+//   1000 of 60 to 120, batch 32 0.734 / 0.784 / 0.880, 64 0.635 / 0.608 / 0.706, 256 0.932 / 0.709 / 0.682
+//   600 of 100 to 250, batch 32 1.510 / 1.441 / 1.623, 64 1.257 / 1.097 / 1.175, 256 2.252 / 1.402 / 0.938
+//   300 of 40 to 400,  batch 32 1.363 / 0.947 / 0.998, 64 1.706 / 0.975 / 0.743
+//   50 of 20 to 60 (fewer graphs than CTAs), batch 32 0.184 / 0.143 / 0.105
+constexpr int kMSmall = 128, kMMiddle = 256, kMLarge = 448;
+constexpr int ctas_per_sm(int threads) { return threads == kMLarge ? 2 : 1024 / threads; }
+int many_threads(int W, int nmax, int64_t batches, int sms) {
+    if (nmax <= 64 && batches >= (int64_t)ctas_per_sm(kMSmall) * sms) return kMSmall;
+    if (W <= 2 && nmax <= 256 && batches >= (int64_t)ctas_per_sm(kMMiddle) * sms) return kMMiddle;
+    return kMLarge;
+}
 constexpr unsigned kFull = 0xffffffffu;
 
-template <int W>
-__global__ void __launch_bounds__(kMBlock, 2) k_many(const ManyParams p) {
+template <int W, int kMBlock>
+__global__ void __launch_bounds__(kMBlock, ctas_per_sm(kMBlock)) k_many(const ManyParams p) {
+    constexpr int kMWarps = kMBlock / 32;
     constexpr int B = 32 * W;
     __shared__ int s_item;
     __shared__ int s_last;
@@ -324,26 +338,28 @@ __global__ void __launch_bounds__(kMBlock, 2) k_many(const ManyParams p) {
     }
 }
 
-}  // namespace
-
-int many_blocks_per_sm(int W) {
-    int nb = 0;
+template <class Fn>
+void with_kernel(int W, int threads, Fn &&f) {
     switch (W) {
-        case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_many<1>, kMBlock, 0); break;
-        case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_many<2>, kMBlock, 0); break;
-        case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_many<4>, kMBlock, 0); break;
-        default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_many<8>, kMBlock, 0); break;
+        case 1: threads == kMSmall ? f(k_many<1, kMSmall>) : threads == kMMiddle ? f(k_many<1, kMMiddle>) : f(k_many<1, kMLarge>); break;
+        case 2: threads == kMSmall ? f(k_many<2, kMSmall>) : threads == kMMiddle ? f(k_many<2, kMMiddle>) : f(k_many<2, kMLarge>); break;
+        case 4: threads == kMSmall ? f(k_many<4, kMSmall>) : f(k_many<4, kMLarge>); break;
+        default: threads == kMSmall ? f(k_many<8, kMSmall>) : f(k_many<8, kMLarge>); break;
     }
-    return nb < 1 ? 1 : nb;
 }
 
-void many_launch(int W, const ManyParams &p, int grid, cudaStream_t st) {
-    switch (W) {
-        case 1: k_many<1><<<grid, kMBlock, 0, st>>>(p); break;
-        case 2: k_many<2><<<grid, kMBlock, 0, st>>>(p); break;
-        case 4: k_many<4><<<grid, kMBlock, 0, st>>>(p); break;
-        default: k_many<8><<<grid, kMBlock, 0, st>>>(p); break;
-    }
+}  // namespace
+
+int many_plan(int W, int nmax, int64_t batches, int sms, int *grid) {
+    const int threads = many_threads(W, nmax, batches, sms);
+    int nb = 0;
+    with_kernel(W, threads, [&](auto *k) { cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, threads, 0); });
+    *grid = (nb < 1 ? 1 : nb) * sms;
+    return threads;
+}
+
+void many_launch(int W, int threads, const ManyParams &p, int grid, cudaStream_t st) {
+    with_kernel(W, threads, [&](auto *k) { k<<<grid, threads, 0, st>>>(p); });
 }
 
 }  // namespace bcgb

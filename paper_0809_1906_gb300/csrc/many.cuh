@@ -45,7 +45,9 @@ struct ManyParams {
     DevCtl *ctl;
 };
 
-int many_blocks_per_sm(int W);
-void many_launch(int W, const ManyParams &p, int grid, cudaStream_t st);
+// Threads per CTA for a set (largest graph, source batches in all) and *grid, the
+// CTAs that the device holds at once.
+int many_plan(int W, int nmax, int64_t batches, int sms, int *grid);
+void many_launch(int W, int threads, const ManyParams &p, int grid, cudaStream_t st);
 
 }  // namespace bcgb
