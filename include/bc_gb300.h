@@ -137,7 +137,7 @@ extern "C" {
  *   batch          sources per batch for the unweighted multi-source path:
  *                  32, 64, 128 or 256 (0 = 256; BC_DENSE uses 128). For
  *                  weighted graphs: sources per wave (0 = 32 to 4 per SM
- *                  below 131072 vertices, by size and weights, else 3 per SM).
+ *                  below 131072 vertices, by arcs and weights, else 3 per SM).
  *   flags          BC_* option bits above.
  *   chunk          arcs per work item for high-degree vertices (0 = 256 in both
  *                  sweeps; a given value applies to both).

@@ -1914,7 +1914,8 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
     const int C = (int)std::min<int64_t>({std::max<int64_t>(64, 4 * (((int64_t)n + K - 1) / K)),
                                           std::max<int64_t>(1024, (1ll << 20) / K), (int64_t)n + 64});
     const size_t per_src = (size_t)n * (8 + 4 + 4 + 4) + 4 + (size_t)K * C * 4;
-    const int per_sm = bcgb::w_packed_per_sm(n, g->maxw);
+    const int threads = bcgb::w_packed_threads(n, g->narcs, g->maxw);
+    const int per_sm = bcgb::w_packed_per_sm(threads);
     int G = (opt && opt->batch > 0) ? opt->batch : per_sm * sm_count_host();
     G = (int)std::min<size_t>((size_t)G, std::max<size_t>(1, (8ull << 30) / per_src));
     G = std::max(1, std::min(G, std::max(nsrc, 1)));
@@ -1973,6 +1974,7 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
     }
     bcgb::WParams base{};
     base.n = n;
+    base.threads = threads;
     base.K = K;
     base.C = C;
     base.dmax = (int32_t)std::min<int64_t>((int64_t)n * g->maxw, INT32_MAX - 1);

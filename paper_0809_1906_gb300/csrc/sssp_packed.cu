@@ -395,19 +395,19 @@ void launch_t(const WParams &p, int nsrc, cudaStream_t st) {
 
 }  // namespace
 
-int w_packed_threads(int32_t n, int32_t maxw) {
+int w_packed_threads(int32_t n, int64_t narcs, int32_t maxw) {
     if (n >= kWSmallN) return 512;
-    const int32_t width = n / (maxw < 1 ? 1 : maxw);
-    return width < 72 ? 32 : width < 150 ? 64 : width < 4000 ? 128 : 256;
+    const int64_t w = maxw < 1 ? 1 : maxw;
+    if (n / w >= 4000) return 256;
+    const int64_t width = narcs / (4 * w);
+    if (width < 72 && narcs <= 5 * (int64_t)n) return 32;
+    return width < 150 ? 64 : 128;
 }
 
-int w_packed_per_sm(int32_t n, int32_t maxw) {
-    const int t = w_packed_threads(n, maxw);
-    return t == 512 ? 3 : 1024 / t;
-}
+int w_packed_per_sm(int threads) { return threads == 512 ? 3 : 1024 / threads; }
 
 void w_launch_wave_packed(const WParams &p, int nsrc, cudaStream_t st) {
-    switch (w_packed_threads(p.n, p.K - 1)) {
+    switch (p.threads) {
         case 32: launch_t<32>(p, nsrc, st); break;
         case 64: launch_t<64>(p, nsrc, st); break;
         case 128: launch_t<128>(p, nsrc, st); break;

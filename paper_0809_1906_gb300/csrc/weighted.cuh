@@ -18,6 +18,7 @@ constexpr int32_t kWPackN = (1 << (32 - kArcWBits)) - 1;  // n at most this: eve
 
 struct WParams {
     int32_t n;
+    int32_t threads;  // packed kernel: threads per source (w_packed_threads)
     int32_t K;     // ring size (> max weight)
     int32_t C;     // entry capacity of one bucket
     int32_t dmax;  // bound on any distance (n * max weight), a loop guard
@@ -66,27 +67,40 @@ void w_pack_arcs(const int32_t *row_ptr, const int32_t *col, const int32_t *w, i
 void w_launch_wave(const WParams &p, int nsrc, cudaStream_t st);         // 64-bit counts
 void w_launch_wave_packed(const WParams &p, int nsrc, cudaStream_t st);  // packed state, 32-bit counts
 // Threads per source of the packed kernel. A distance step settles n / (distinct
-// distances) vertices, and the number of distinct distances grows with the
-// largest weight, so n / maxw stands for a step's width: narrow steps leave
-// wide CTAs idle at every barrier, wide ones are worked through in turns by
-// narrow CTAs. Square grids with 5% long-range edges, weights 1..maxw, all
-// sources up to n = 4096, else 2048; ms with 32 / 64 / 128 / 256 threads (and as
-// many sources resident as 64 registers a thread allow); the 128-thread
-// kernel before records, ballots and one-warp sources in brackets:
+// distances) vertices and relaxes their arcs; the number of distinct distances
+// grows with the largest weight, so narcs / maxw stands for a step's work
+// (narcs / (4 maxw), the vertices of a mesh): narrow steps leave wide CTAs idle at
+// every barrier, wide ones are worked through in turns by narrow CTAs. Square
+// grids with 5% long-range edges, weights 1..maxw, all sources up to n = 4096,
+// else 2048; ms with 32 / 64 / 128 / 256 threads (and as many sources resident as
+// 64 registers a thread allow); the 128-thread kernel before records, ballots and
+// one-warp sources in brackets:
 //   n = 2304,  maxw 100 (width 23):   1.53 / 1.86 / 2.82 / 5.10  (3.56)
 //   n = 4096,  maxw 100 (width 41):   3.12 / 3.91 / 6.06 / 10.1  (7.88)
 //   n = 10000, maxw 100 (width 100):  4.29 / 4.06 / 4.68 / 7.44  (5.82)
 //   n = 17956, maxw 100 (width 180):  8.36 / 7.96 / 7.47 / 9.83  (9.19)
+//   n = 99856, maxw 4000 (width 26):  153 / 163 / 146 / 264
 //   n = 1024,  maxw 3   (width 341):  0.30 / 0.27 / 0.24 / 0.30  (0.38)
 //   n = 10000, maxw 3   (width 3333): 3.00 / 2.69 / 2.09 / 2.13  (2.71)
 //   n = 17956, maxw 3   (width 5985): 6.54 / 6.10 / 4.55 / 3.60  (5.58)
+// Few hops reach everything in a random or a skewed graph, so its distances are
+// fewer than a mesh's and its steps wider, and one lane walks a hub's whole row
+// while a narrow CTA waits: above a mean degree of 5, two warps at least.
+//   R-MAT n = 1736,  maxw 100 (width 121):   11.5 / 7.3 / 8.4 / 10.0
+//   R-MAT n = 3352,  maxw 100 (width 260):   23.6 / 23.9 / 22.6 / 31.4
+//   R-MAT n = 12510, maxw 100, 3000 sources (width 1000): 130 / 110 / 85 / 82
+//   R-MAT n = 12510, maxw 4000 (width 26):   184 / 178 / 224 / 330
+//   R-MAT n = 46894, maxw 1000, 2000 sources (width 450): 941 / 551 / 575 / 629
+//   random n = 5000, m = 25000, maxw 200 (width 62): 15.2 / 11.4 / 11.4 / 18.9
+//   attachment n = 5000, three arcs a vertex, maxw 100 (width 75): 11.5 / 10.1 / 10.9 / 18.6
+//   G(3000, 0.05), maxw 50 (width 2250):     34.8 / 33.0 / 26.5 / 24.5
 // From kWSmallN vertices on a source's state (8 n bytes) no longer fits L2
 // beside the others', and fewer, wider sources win: n = 262144, maxw 100, 4096
 // sources, 256 threads at four per SM 246 ms, 512 at three per SM (two
 // resident) 221 ms (241 before).
 constexpr int32_t kWSmallN = 131072;
-int w_packed_threads(int32_t n, int32_t maxw);
-int w_packed_per_sm(int32_t n, int32_t maxw);  // sources per SM of a default wave
+int w_packed_threads(int32_t n, int64_t narcs, int32_t maxw);
+int w_packed_per_sm(int threads);  // sources per SM of a default wave
 // bc[vid[v]] += the FP64 sum over r < nrows of rows[r][v], rows in order (vid null: bc[v])
 void w_launch_reduce(const float *rows, int nrows, int n, const int32_t *vid, double *bc, int sms,
                      cudaStream_t st);
