@@ -1,6 +1,7 @@
 // bc_api.cu -- the C ABI (include/bc_gb300.h): graph upload and checks,
 // work-item plan, device memory plan, and the batch scheduler that drives the
 // level loop of the multi-source path.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1540,11 +1541,28 @@ bool one_launch(const bc_graph *g, int32_t nsrc, int W, int K) {
     return units(0.75, resident / K) <= most * used;
 }
 
+// Whether kernels on st may use all the device's SMs: a stream of a green
+// context has a part of them, where the blocks of a cooperative launch sized
+// for the device are not resident together.
+bool whole_device(cudaStream_t st) {
+    using Fn = CUresult (*)(CUstream, CUgreenCtx *);
+    static const Fn fn = [] {
+        void *ptr = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &ptr, 12050, cudaEnableDefault, &q);
+        cudaGetLastError();
+        return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<Fn>(ptr) : nullptr;
+    }();
+    CUgreenCtx green = nullptr;
+    return !fn || fn(st, &green) != CUDA_SUCCESS || green == nullptr;
+}
+
 // Bound on each wait at a barrier of the one-launch sweep. Such a wait lasts as
 // long as the slowest block's level, not a copy's microseconds, so
 // bc_options.device_wait_us does not apply to it: a run that sets that bound
 // takes the launch-per-level form, whose only device waits are for copies.
 constexpr uint64_t kBarrierWaitNs = 10000000000ull;
+constexpr int kSweepRefused = 100;  // run_sweep: no launch, nothing done (not a status of the library)
 
 // Batches of a run as one cooperative launch (k_sweep): group k takes batches
 // k, k + K, ... with lane k's state and its own BC sums, added in group order at
@@ -1605,7 +1623,12 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
         g->counters_unsure = true;
         {
             Timer t(g, st, BC_KERNEL_FORWARD);
-            CK(bcgb::ms_launch_sweep(W, q, st));
+            const cudaError_t e = bcgb::ms_launch_sweep(W, q, st);
+            if (e == cudaErrorCooperativeLaunchTooLarge && !resume) {
+                cudaGetLastError();
+                return kSweepRefused;
+            }
+            CK(e);
         }
         // wait until every batch's forward pass has ended (or the launch, early);
         // each wait, up to the next batch that any group reports, has the limit
@@ -1693,8 +1716,12 @@ int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStr
         int K = g->timing ? 1 : std::min<int32_t>(kSweepLanes, nbat);
         while (K > 1 && (K - 1) * lane_bytes > kLaneBudgetBytes) --K;
         const bool sweep = backward && !rows_sig && !rows_dist && !g->timing &&
-                           (g->dev_wait_ns == 0 || g->test_barrier) && g->test_hold == 0 && nsrc > 0 && one_launch(g, nsrc, W, K);
-        if (sweep) return run_sweep(g, nsrc, W, K, st, hash, wait_ms);
+                           (g->dev_wait_ns == 0 || g->test_barrier) && g->test_hold == 0 && nsrc > 0 && one_launch(g, nsrc, W, K) &&
+                           whole_device(st);
+        if (sweep) {
+            r = run_sweep(g, nsrc, W, K, st, hash, wait_ms);
+            if (r != kSweepRefused) return r;  // refused: the blocks do not fit the device together just now
+        }
         r = reset_counters(g, st);
         if (!r && backward) r = clear_outputs(g, nsrc, hash, st);
         if (r) return r;
