@@ -215,7 +215,7 @@ __device__ __forceinline__ void forward_items(const MsParams &p, const int l, co
                                               FwdShared<W> &sh, body::WarpStage &ws, const uint16_t *Sl, uint16_t *Sn,
                                               const bool ones, FwdFound &found) {
     constexpr int B = 32 * W;
-    // probe_chunk's per-arc notes: nobody reads them in the staged form
+    // probe_chunk's per-arc notes: read where the level's counts are wide, not by the staged form
     __shared__ int32_t s_u[kWarps][32];
     __shared__ uint32_t s_nz[kWarps][32];
     const int lane = threadIdx.x & 31;
@@ -459,7 +459,7 @@ template <int W, bool HOOK, bool NC>
 __device__ __forceinline__ void backward_items(const MsParams &p, const int l, const int bid, const int nblk,
                                                BwdShared<W> &sh, body::WarpStage &ws) {
     constexpr int B = 32 * W;
-    // probe_chunk's per-arc notes: nobody reads them in the staged form
+    // probe_chunk's per-arc notes: nobody reads them in the backward's two forms
     __shared__ int32_t s_u[kWarps][32];
     __shared__ uint32_t s_nz[kWarps][32];
     const int lane = threadIdx.x & 31;

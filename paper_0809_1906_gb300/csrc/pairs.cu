@@ -155,7 +155,8 @@ __global__ void __launch_bounds__(256) k_pair_reduce(const double *__restrict__ 
 
 // Source ranges: while the v x t tiles are fewer than kPairBlocks (about four
 // waves at two blocks per SM, so that the last wave weighs little), the rows
-// are split, into whole stages.
+// are split, into whole stages. A constant, not the device's count: the ranges
+// fix the order of the partial sums, and with it the last bits of BC.
 constexpr int kPairBlocks = 1216;
 int pair_ranges(int n, int *rows) {
     const int tiles = ((n + kTV - 1) / kTV) * ((n + kTT - 1) / kTT), stages = (n + kTS - 1) / kTS;
