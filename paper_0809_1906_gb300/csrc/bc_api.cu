@@ -1927,6 +1927,7 @@ int ensure_packed(bc_graph *g, bool relabel, cudaStream_t st) {
 // delta rows are added in the order of the flagged sources.
 constexpr int kWeightedLanes = 2;  // measured: 3 or 4 lanes no faster on the 512x512 grid
 
+constexpr size_t kWeightedWaveBudget = 8ull << 30;        // state of one wave
 constexpr double kWeightedLaneBudget = 24.0 * (1 << 30);  // packed wave state of all lanes
 
 int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t st, bool backward, bool hash,
@@ -1936,15 +1937,29 @@ int run_weighted(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream_t 
     if (K > bcgb::kMaxRing)
         return fail(BC_ERR_UNSUPPORTED, "weighted path: maximum weight must be below " +
                                             std::to_string(bcgb::kMaxRing));
-    // bucket entries: four times their mean number if the ring held every vertex
-    // once, up to 4 MB a source (a fuller bucket is read by a scan over the vertices)
-    const int C = (int)std::min<int64_t>({std::max<int64_t>(64, 4 * (((int64_t)n + K - 1) / K)),
-                                          std::max<int64_t>(1024, (1ll << 20) / K), (int64_t)n + 64});
-    const size_t per_src = (size_t)n * (8 + 4 + 4 + 4) + 4 + (size_t)K * C * 4;
     const int threads = bcgb::w_packed_threads(n, g->narcs, g->maxw);
     const int per_sm = bcgb::w_packed_per_sm(threads);
     int G = (opt && opt->batch > 0) ? opt->batch : per_sm * sm_count_host();
-    G = (int)std::min<size_t>((size_t)G, std::max<size_t>(1, (8ull << 30) / per_src));
+    // Bucket entries, up to 4 MB a source. A fuller bucket is read by a scan over
+    // all vertices, which costs a step n reads: in skewed and dense graphs most
+    // vertices lie within a few distances of one another. 32 times the mean number
+    // (if the ring held every vertex once) while G sources' states fit the budget,
+    // at the least 16 times and 256, but no more than half the vertices, or four
+    // times, beyond that (64 x 64 mesh, maxw 5: 1.74 ms with 2732 entries, 1.81 with
+    // 4160). Whole runs, ms, with 4 / 16 / 32 times (64, 256,
+    // 512 at the least): R-MAT n = 46894, maxw 1000 506 / 225 / 225, n = 12510,
+    // maxw 100 57 / 35 / 35; G(3000, 0.05), maxw 1000 117 / 31 / 31, maxw 50 26 / 21 / 17;
+    // random n = 20000, weights 3900..4000 91 / 42 / 42; meshes the same, but with
+    // maxw 4000, n = 90000, where room for 1024 entries left fewer sources in flight:
+    // 80 / 80 / 142.
+    const int64_t mean = ((int64_t)n + K - 1) / K, state = 20ll * n + 4;
+    const int64_t fit = ((int64_t)kWeightedWaveBudget / G - state) / (4ll * K);
+    const int C = (int)std::min<int64_t>({std::max(std::max<int64_t>(256, 16 * mean),
+                                                   std::min(std::max<int64_t>(512, 32 * mean), fit)),
+                                          std::max<int64_t>({256, 4 * mean, n / 2}),
+                                          std::max<int64_t>(1024, (1ll << 20) / K), (int64_t)n + 64});
+    const size_t per_src = (size_t)n * (8 + 4 + 4 + 4) + 4 + (size_t)K * C * 4;
+    G = (int)std::min<size_t>((size_t)G, std::max<size_t>(1, kWeightedWaveBudget / per_src));
     G = std::max(1, std::min(G, std::max(nsrc, 1)));
     const int32_t nwaves = (nsrc + G - 1) / G;
     // lanes: up to kWeightedLanes within the memory budget; BC_TIMING: one

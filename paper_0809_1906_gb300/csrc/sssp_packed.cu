@@ -400,7 +400,7 @@ int w_packed_threads(int32_t n, int64_t narcs, int32_t maxw) {
     const int64_t w = maxw < 1 ? 1 : maxw;
     if (n / w >= 4000) return 256;
     const int64_t width = narcs / (4 * w);
-    if (width < 72 && narcs <= 5 * (int64_t)n) return 32;
+    if (width < (narcs <= 5 * (int64_t)n ? 72 : 40)) return 32;
     return width < 150 ? 64 : 128;
 }
 

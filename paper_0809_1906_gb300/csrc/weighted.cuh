@@ -85,15 +85,18 @@ void w_launch_wave_packed(const WParams &p, int nsrc, cudaStream_t st);  // pack
 //   n = 17956, maxw 3   (width 5985): 6.54 / 6.10 / 4.55 / 3.60  (5.58)
 // Few hops reach everything in a random or a skewed graph, so its distances are
 // fewer than a mesh's and its steps wider, and one lane walks a hub's whole row
-// while a narrow CTA waits: above a mean degree of 5, two warps at least.
-//   R-MAT n = 1736,  maxw 100 (width 121):   11.5 / 7.3 / 8.4 / 10.0
-//   R-MAT n = 3352,  maxw 100 (width 260):   23.6 / 23.9 / 22.6 / 31.4
-//   R-MAT n = 12510, maxw 100, 3000 sources (width 1000): 130 / 110 / 85 / 82
-//   R-MAT n = 12510, maxw 4000 (width 26):   184 / 178 / 224 / 330
-//   R-MAT n = 46894, maxw 1000, 2000 sources (width 450): 941 / 551 / 575 / 629
-//   random n = 5000, m = 25000, maxw 200 (width 62): 15.2 / 11.4 / 11.4 / 18.9
-//   attachment n = 5000, three arcs a vertex, maxw 100 (width 75): 11.5 / 10.1 / 10.9 / 18.6
-//   G(3000, 0.05), maxw 50 (width 2250):     34.8 / 33.0 / 26.5 / 24.5
+// while a narrow CTA waits: above a mean degree of 5, one warp only up to a width
+// of 40 (all sources unless stated; 4864, 2432, 1216, 608 sources resident).
+//   R-MAT n = 1736,  maxw 100 (width 113):   5.5 / 3.9 / 5.6 / 8.1
+//   R-MAT n = 3352,  maxw 100 (width 240):   12.7 / 13.2 / 13.8 / 22.3
+//   R-MAT n = 3352,  maxw 1000 (width 24):   20.7 / 31.7 / 43.2 / 82.7
+//   R-MAT n = 12510, maxw 100, 2000 sources (width 1070): 65 / 38 / 35 / 41
+//   R-MAT n = 12510, maxw 4000, 2000 sources (width 27):  164 / 157 / 151 / 257
+//   R-MAT n = 46894, maxw 1000, 1500 sources (width 455): 347 / 212 / 225 / 244
+//   random n = 5000, m = 25000, maxw 200 (width 62): 15.0 / 11.3 / 11.2 / 18.8
+//   attachment n = 5000, three arcs a vertex, maxw 100 (width 75): 11.4 / 10.1 / 10.9 / 18.6
+//   G(3000, 0.05), maxw 1000 (width 112):    26.1 / 30.7 / 31.6 / 47.3
+//   G(3000, 0.05), maxw 50 (width 2250):     27.7 / 27.3 / 21.0 / 19.7
 // From kWSmallN vertices on a source's state (8 n bytes) no longer fits L2
 // beside the others', and fewer, wider sources win: n = 262144, maxw 100, 4096
 // sources, 256 threads at four per SM 246 ms, 512 at three per SM (two
