@@ -36,6 +36,9 @@
  *     buffers are kept for the next graphs created on the same device;
  *     bc_release_cached_memory frees the cached blocks, and an allocation that
  *     fails frees them and retries. Caller buffers stay owned by the caller.
+ *   - Calls on one handle may follow one another on a stream without waiting
+ *     for the one before. A caller that goes on with another stream makes that
+ *     stream wait for the first one (bc_result waits too).
  *   - A graph handle may be used by one thread at a time. It lives on the
  *     device that is current when it is created, and every call on it
  *     (bc_destroy_graph included) must be made with that device current.

@@ -540,7 +540,7 @@ int check_graph(int32_t n, const std::vector<int32_t> &rp, const std::vector<int
 // Work items: one per vertex, except vertices with more than `chunk` arcs,
 // which are split into chunks that combine through partial slots. Heavy
 // chunks come first, then vertices by descending degree.
-int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int32_t> &rp) {
+int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int32_t> &rp, cudaStream_t st) {
     if (pl.chunk == chunk && pl.items) return BC_OK;
     const int32_t n = g->n;
     pl.chunk = 0;  // no plan until the new one is in place: an allocation may fail
@@ -597,7 +597,8 @@ int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int3
     pl.nheavy = (int32_t)(4 * nlight < nitems ? nitems : nitems - nlight);
     pl.nslots = (int32_t)nslots;
     CK(pl.blob.ensure(h.size()));
-    if (!h.empty()) CK(cudaMemcpy(pl.blob.p, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    // in st's order: the run before may still read the plan that this one replaces
+    if (!h.empty()) CK(cudaMemcpyAsync(pl.blob.p, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     pl.items = reinterpret_cast<const int4 *>(pl.blob.p);
     pl.item_v = pl.blob.p + 4 * nitems;
     pl.slot_first = pl.item_v + nitems;
@@ -613,12 +614,12 @@ int build_items(bc_graph *g, ItemPlan &pl, int32_t chunk, const std::vector<int3
 // with lanes fewer, larger items win). An explicit chunk size applies to both.
 // Two plans are kept because the forward pulls over in-arcs and the backward
 // over out-arcs (different on directed graphs).
-int build_plans(bc_graph *g, const bc_options *opt) {
+int build_plans(bc_graph *g, const bc_options *opt, cudaStream_t st) {
     const int32_t fc = (opt && opt->chunk > 0) ? opt->chunk : 256;
     const int32_t bch = (opt && opt->chunk > 0) ? opt->chunk : 256;
     // the forward sweep pulls over in-arcs, the backward over out-arcs
-    int r = build_items(g, g->fplan, fc, g->directed ? g->h_row_ptr_in : g->h_row_ptr);
-    if (!r) r = build_items(g, g->bplan, bch, g->h_row_ptr);
+    int r = build_items(g, g->fplan, fc, g->directed ? g->h_row_ptr_in : g->h_row_ptr, st);
+    if (!r) r = build_items(g, g->bplan, bch, g->h_row_ptr, st);
     return r;
 }
 
@@ -640,7 +641,8 @@ int s_levels_for(size_t n, size_t B, int Lcap) {
     return (double)Lcap * (double)n * (double)B * 2.0 <= kSLevelsBudget ? Lcap : 2;
 }
 
-int ensure_state(bc_graph *g, int W, int Lcap) {
+// st: the stream of the run that asks (the run before may still use the state there)
+int ensure_state(bc_graph *g, int W, int Lcap, cudaStream_t st) {
     if (g->W == W && g->Lcap >= Lcap && g->sigma.p) return BC_OK;
     const size_t n = (size_t)std::max(g->n, 1);
     const size_t B = 32 * (size_t)W;
@@ -658,7 +660,7 @@ int ensure_state(bc_graph *g, int W, int Lcap) {
     CK(g->part.ensure(slots * B));
     CK(g->pmask.ensure(slots * W));
     CK(g->cnt.ensure(slots));
-    CK(cudaMemset(g->cnt.p, 0, g->cnt.n * sizeof(uint32_t)));
+    CK(cudaMemsetAsync(g->cnt.p, 0, g->cnt.n * sizeof(uint32_t), st));
     g->W = W;
     g->Lcap = Lcap;
     return BC_OK;
@@ -737,7 +739,7 @@ bcgb::MsParams make_params(bc_graph *g) {
 
 // Batch state of sweep lane k >= 1 (same shapes as ensure_state's), plus its
 // stream, control blocks and BC accumulator, created on first use.
-int ensure_lane(bc_graph *g, SweepLane &ln, int W, int Lcap) {
+int ensure_lane(bc_graph *g, SweepLane &ln, int W, int Lcap, cudaStream_t st) {
     int dev = 0;
     CK(cudaGetDevice(&dev));
     bool fresh = false;
@@ -749,7 +751,7 @@ int ensure_lane(bc_graph *g, SweepLane &ln, int W, int Lcap) {
             CK(cudaStreamCreateWithFlags(&ln.st, cudaStreamNonBlocking));
             CK(cudaEventCreateWithFlags(&ln.ev, cudaEventDisableTiming));
             CK(cudaMalloc((void **)&ln.ctl, sizeof(bcgb::DevCtl)));
-            CK(cudaMemset(ln.ctl, 0, sizeof(bcgb::DevCtl)));
+            CK(cudaMemsetAsync(ln.ctl, 0, sizeof(bcgb::DevCtl), ln.st));
             CK(cudaHostAlloc((void **)&ln.hctl, sizeof(bcgb::HostCtl), cudaHostAllocMapped | cudaHostAllocPortable));
             std::memset(ln.hctl, 0, sizeof(bcgb::HostCtl));
             CK(cudaHostGetDevicePointer((void **)&ln.hctl_d, ln.hctl, 0));
@@ -778,7 +780,7 @@ int ensure_lane(bc_graph *g, SweepLane &ln, int W, int Lcap) {
     CK(ln.part.ensure(slots * B));
     CK(ln.pmask.ensure(slots * W));
     CK(ln.cnt.ensure(slots));
-    CK(cudaMemset(ln.cnt.p, 0, ln.cnt.n * sizeof(uint32_t)));
+    CK(cudaMemsetAsync(ln.cnt.p, 0, ln.cnt.n * sizeof(uint32_t), st));
     CK(ln.bc.ensure(n));
     ln.W = W;
     ln.Lcap = Lcap;
@@ -1096,9 +1098,9 @@ int run_dense_group(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream
     const int32_t n = g->n;
     const size_t nn = (size_t)std::max(n, 1), nw32 = (nn + 31) / 32;
     const bool sparse_bwd = opt && (opt->flags & BC_SPARSE_BACKWARD);
-    int r = build_plans(g, opt);
+    int r = build_plans(g, opt, st);
     if (r) return r;
-    r = ensure_state(g, W, std::max(g->Lcap, 32));
+    r = ensure_state(g, W, std::max(g->Lcap, 32), st);
     if (r) return r;
     const int nbat = (nsrc + B - 1) / B;
     for (int gb0 = 0; gb0 < nbat;) {
@@ -1229,7 +1231,7 @@ int run_dense_group(bc_graph *g, int32_t nsrc, const bc_options *opt, cudaStream
         }
         if (capped) {  // deeper than the level capacity: grow it and redo this group
             CK(cudaStreamSynchronize(st));
-            r = ensure_state(g, W, g->Lcap * 2);
+            r = ensure_state(g, W, g->Lcap * 2, st);
             if (r) return r;
             continue;
         }
@@ -1354,7 +1356,7 @@ int run_lanes(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool bac
     const int32_t nbat = (nsrc + B - 1) / B;
     int Lcap = g->Lcap;
     for (int k = 1; k < K; ++k) {
-        const int r = ensure_lane(g, g->lanes[k - 1], W, Lcap);
+        const int r = ensure_lane(g, g->lanes[k - 1], W, Lcap, st);
         if (r) return r;
     }
     if (!g->ev0) CK(cudaEventCreateWithFlags(&g->ev0, cudaEventDisableTiming));
@@ -1435,8 +1437,8 @@ int run_lanes(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool bac
                 // start each lane's unfinished batch again
                 for (int q = 0; q < K; ++q) CK(cudaStreamSynchronize(lane_stream(q)));
                 Lcap *= 2;
-                int r = ensure_state(g, W, Lcap);
-                for (int q = 1; q < K && !r; ++q) r = ensure_lane(g, g->lanes[q - 1], W, Lcap);
+                int r = ensure_state(g, W, Lcap, st);
+                for (int q = 1; q < K && !r; ++q) r = ensure_lane(g, g->lanes[q - 1], W, Lcap, g->lanes[q - 1].st);
                 if (r) return r;
                 for (int q = 0; q < K; ++q)
                     if (jobs[q].phase == 1) {
@@ -1578,7 +1580,7 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
     int Lcap = g->Lcap;
     for (bool resume = false;; resume = true) {
         for (int k = 1; k < K; ++k) {
-            const int r = ensure_lane(g, g->lanes[k - 1], W, Lcap);
+            const int r = ensure_lane(g, g->lanes[k - 1], W, Lcap, st);
             if (r) return r;
         }
         bcgb::SweepParams q{};
@@ -1671,7 +1673,7 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
         }
         CK(cudaStreamSynchronize(st));
         Lcap *= 2;
-        const int r = ensure_state(g, W, Lcap);
+        const int r = ensure_state(g, W, Lcap, st);
         if (r) return r;
         CK(cudaMemsetAsync(reinterpret_cast<char *>(g->ctl) + kCtlFinishAt, 0, kCtlBytes - kCtlFinishAt, st));
     }
@@ -1701,9 +1703,9 @@ int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStr
         if (rd) return rd;
         return run_dense_group(g, nsrc, opt, st, backward, hash, rows_sig, rows_dist);
     }
-    int r = build_plans(g, opt);
+    int r = build_plans(g, opt, st);
     if (r) return r;
-    r = ensure_state(g, W, std::max(g->Lcap, 32));
+    r = ensure_state(g, W, std::max(g->Lcap, 32), st);
     if (r) return r;
     const int B = 32 * W;
     {
@@ -1761,7 +1763,7 @@ int run_batches(bc_graph *g, int32_t nsrc, int W, const bc_options *opt, cudaStr
         if (r) return r;
         if (L < 0) {  // deeper than the level capacity: grow it and redo this batch
             CK(cudaStreamSynchronize(st));
-            r = ensure_state(g, W, g->Lcap * 2);
+            r = ensure_state(g, W, g->Lcap * 2, st);
             if (r) return r;
             continue;
         }
@@ -2383,8 +2385,8 @@ int bc_run(bc_graph *g, const int32_t *sources, int32_t num_sources, const bc_op
     if (order) {
         // size the sweep state for this run's width first, so the landmark
         // pass (32 sources) runs in it instead of allocating its own
-        r = build_plans(g, opt);
-        if (!r) r = ensure_state(g, W, std::max(g->Lcap, 32));
+        r = build_plans(g, opt, st);
+        if (!r) r = ensure_state(g, W, std::max(g->Lcap, 32), st);
         if (!r) r = ensure_rank(g, st);
         if (r) return r;
     }

@@ -73,3 +73,30 @@ def test_result_survives_rows_after_a_failed_run(nat):
             h.forward_rows(np.arange(3, dtype=np.int32), batch=64)
             got, _, _ = h.result()
             assert close(got, ref["bc"], g.n)
+
+
+@pytest.mark.parametrize("first,second", [((32, 8), (32, 0)), ((256, 4), (64, 16)), ((64, 0), (32, 8))])
+def test_next_run_waits_for_the_last_ones_plan_and_state(nat, first, second):
+    """Runs one after another on a stream of its own, none of them waited for:
+    the next one, with other work items and another width, replaces plans and
+    counters only after the backward pass before it (a long path hung on a hub of
+    split items) has read them."""
+    import torch
+    at = np.arange(1200)
+    spokes = 1200 + np.arange(900)
+    g = G.csr_from_edges(2100, np.concatenate([at[:-1], np.zeros(900, np.int64)]), np.concatenate([at[1:], spokes]),
+                         name="path+hub")
+    src = np.concatenate([np.arange(0, 1200, 50), spokes[:8]]).astype(np.int32)
+    ref = oracle.bc(g, src)["bc"]
+    stream = torch.cuda.Stream()
+    with nat.Graph.from_csr(g) as h:
+        for batch, chunk in (first, second):  # the level capacity and both plans' room are there afterwards
+            h.run(src, batch=batch, chunk=chunk, stream=stream)
+            h.result()
+        for rep in range(3):
+            h.run(src, batch=first[0], chunk=first[1], stream=stream)
+            h.run(src, batch=second[0], chunk=second[1], stream=stream, flags=nat.BC_ACCUMULATE)
+            h.run(src, batch=first[0], chunk=first[1], stream=stream, flags=nat.BC_ACCUMULATE)
+            got, code, st = h.result()
+            assert code == nat.BC_OK and st == 0
+            assert close(got, 3.0 * ref, 3 * g.n), rep
