@@ -1638,6 +1638,10 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
         bool ended = false;
         auto t0 = std::chrono::steady_clock::now();
         for (long spins = 0;; ++spins) {
+            // the clock first, then the words: a host thread that was held up
+            // between the two finds what the device reported meanwhile
+            const bool look = spins % 1024 == 1023;
+            const auto now = look ? std::chrono::steady_clock::now() : t0;
             ended = bcgb::word_for(&g->hctl->done, q.seq, &status);
             if (ended) break;
             bool all = true, moved = false;
@@ -1651,10 +1655,8 @@ int run_sweep(bc_graph *g, int32_t nsrc, int W, int K, cudaStream_t st, bool has
             }
             if (all) break;
             if (moved) t0 = std::chrono::steady_clock::now();
-            if (spins % 1024 != 1023) continue;
-            const auto ms =
-                std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count();
-            if (ms > wait_ms)
+            if (moved || !look) continue;
+            if (std::chrono::duration_cast<std::chrono::milliseconds>(now - t0).count() > wait_ms)
                 return fail(BC_ERR_TIMEOUT, "the device did not report the end of a forward pass within the wait limit");
             const cudaError_t e = cudaStreamQuery(st);
             if (e != cudaSuccess && e != cudaErrorNotReady)

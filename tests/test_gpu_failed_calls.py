@@ -24,47 +24,44 @@ def close(got, ref, n):
     return np.all(np.abs(got - ref) <= np.maximum(1e-5 * np.abs(ref), 1e-6 * n))
 
 
-def ring_with_chords(n, chords, seed):
-    """A ring and random chords: connected, shallow, quick to build."""
-    rng = np.random.default_rng(seed)
-    u, v = rng.integers(0, n, chords), rng.integers(0, n, chords)
-    at = np.arange(n)
-    u, v = np.concatenate([at, u]), np.concatenate([(at + 1) % n, v])
-    keep = u != v
-    key = np.unique(np.minimum(u, v)[keep] * n + np.maximum(u, v)[keep])
-    return key // n, key % n
-
-
 def test_rows_left_unwritten_after_a_failed_call(nat):
     """Rows go straight into the caller's device memory, from several internal
-    streams. A call whose host wait runs out (1 ms, on levels that take
-    several) must have ended on all of them when it returns: the caller may
-    free or refill the buffers. 256 sources in a small component keep the
-    caller's own stream short, so that a wait for it alone would not do."""
+    streams. A call whose host wait runs out (1 ms, with the stream held for some
+    20) must have ended on all of them when it returns: the caller may free or
+    refill the buffers. The first batch's sources are isolated, so the caller's own
+    stream is done early; the second one's second level takes longer (24
+    hubs, each joined to every one of 400,000 vertices)."""
     import torch
-    n, small = 1_000_000, 300
-    u, v = ring_with_chords(n - small, 4_000_000, 5)
-    ring = np.arange(small)
-    g = G.csr_from_edges(n, np.concatenate([u, n - small + ring]), np.concatenate([v, n - small + (ring + 1) % small]),
-                         name="two")
-    src = np.concatenate([n - small + np.arange(256), np.arange(256)]).astype(np.int32)
+    leaves, hubs, alone = 400_000, 24, 256
+    n = leaves + hubs + alone
+    g = G.csr_from_edges(n, np.tile(np.arange(leaves), hubs), np.repeat(leaves + np.arange(hubs), leaves), name="hubs")
+    src = np.concatenate([leaves + hubs + np.arange(alone), np.arange(256)]).astype(np.int32)
     sig = torch.zeros((512, n), dtype=torch.int64, device="cuda")
     dist = torch.zeros((512, n), dtype=torch.int32, device="cuda")
+
+    def rows(h, wait_ms):
+        opt = nat.make_options(256, 0, 0, wait_ms)
+        return h.lib.bc_forward_rows(h.handle, nat._addr(src), len(src), nat._addr(sig), nat._addr(dist),
+                                     ctypes.byref(opt), nat._stream_ptr(stream))
+
+    stream = torch.cuda.Stream()
+    left = []
     with nat.Graph.from_csr(g, trust_input=True) as h:
-        opt = nat.make_options(256, 0, 0, 1)
+        assert rows(h, 0) == nat.BC_OK  # plans and state are in place: the next calls only launch
+        for _ in range(3):  # the least of three: a held-up host thread is no failure
+            torch.cuda.synchronize()
+            with torch.cuda.stream(stream):
+                torch.cuda._sleep(40_000_000)
+            code = rows(h, 1)
+            t0 = time.perf_counter()
+            torch.cuda.synchronize()
+            left.append(time.perf_counter() - t0)
+            assert code == nat.BC_ERR_TIMEOUT
+        sig.zero_(), dist.zero_()
         torch.cuda.synchronize()
-        code = h.lib.bc_forward_rows(h.handle, nat._addr(src), len(src), nat._addr(sig), nat._addr(dist),
-                                     ctypes.byref(opt), nat._stream_ptr(None))
-        t0 = time.perf_counter()
-        torch.cuda.synchronize()
-        left = time.perf_counter() - t0
-        assert code == nat.BC_ERR_TIMEOUT
-        # an idle device answers in tens of microseconds; the levels in flight take milliseconds
-        assert left < 5e-4, left
-        opt = nat.make_options(256)
-        code = h.lib.bc_forward_rows(h.handle, nat._addr(src), len(src), nat._addr(sig), nat._addr(dist),
-                                     ctypes.byref(opt), nat._stream_ptr(None))
-        assert code == nat.BC_OK
+        assert rows(h, 0) == nat.BC_OK
+    # an idle device answers in some 30 us; the level in flight left 680 us
+    assert min(left) < 2.5e-4, left
     for i in (0, 255, 256, 511):
         o = oracle.source(g, int(src[i]), with_delta=False)
         assert np.array_equal(sig[i].cpu().numpy().view(np.uint64), o["sigma"])
@@ -124,12 +121,14 @@ def test_run_returns_before_the_backward_pass_ends(nat):
     with nat.Graph.from_csr(g) as h:
         h.run(src, batch=32)
         h.result()
-        h.run(src, batch=32)
-        time.sleep(3e-4)
-        running = not torch.cuda.current_stream().query()
-        got, code, _ = h.result()
-    assert code == nat.BC_OK and close(got, oracle.bc(g, src)["bc"], g.n)
-    assert running
+        running = []
+        for _ in range(3):  # one of three: the host thread may be held up between the two
+            h.run(src, batch=32)
+            time.sleep(3e-4)
+            running.append(not torch.cuda.current_stream().query())
+            got, code, _ = h.result()
+            assert code == nat.BC_OK and close(got, oracle.bc(g, src)["bc"], g.n)
+    assert any(running)
 
 
 def test_out_of_memory_leaves_the_handle_usable(nat):
